@@ -344,6 +344,7 @@ kss_status kss_setup(kss_ctx ctx, const kss_cell* cell, const kss_atoms* atoms, 
     s->d_Vx32.alloc(nr * sizeof(float));
     launch_vloc(s.get(), ctx->stream);
     launch_vloc_views(s.get(), ctx->stream);
+    launch_fx_tables(s.get(), ctx->stream);
     s->vmax = device_max(s->d_V64.as<double>(), nr, ctx->stream);
 
     if (s->nproj) {
@@ -694,7 +695,8 @@ namespace kss {
 size_t sys_device_bytes(kss_sys s) {
   size_t b = s->d_V64.bytes + s->d_Vx64.bytes + s->d_Vx32.bytes + s->d_D64.bytes + s->d_D32.bytes +
              s->d_Q64.bytes + s->d_Q32.bytes;
-  for (int i = 0; i < 3; ++i) b += s->d_tw64[i].bytes + s->d_tw32[i].bytes;
+  for (int i = 0; i < 3; ++i) b += s->d_tw64[i].bytes + s->d_tw32[i].bytes + s->d_rot[i].bytes;
+  for (const auto& kv : s->vfx) b += kv.second.bytes;
   for (const auto& kv : s->vpi64) b += kv.second.bytes;
   for (const auto& kv : s->vpi32) b += kv.second.bytes;
   for (const auto& kv : s->vfused32) b += kv.second.bytes;

@@ -13,6 +13,8 @@
 
 #include <type_traits>
 
+#include "fx64.cuh"
+
 namespace kss {
 namespace fftr {
 
@@ -105,6 +107,46 @@ template <typename C, typename T> __device__ __forceinline__ C muli_m(C a, T s, 
   return r;
 }
 
+// ---- fixed point (fx64.cuh): the same codelets on 64-bit integers ----------------------------
+// (a c) for a compile-time factor c = kcos62(M, N) (SIN = false) or ksin62(M, N), in units of
+// 2^-62: c is taken as 0, +-1/2 or +-1 plus a rest of size at most one half, which is all that is
+// multiplied (a rest of zero or one half costs no multiplication).
+template <bool SIN, int M, int N>
+__device__ __forceinline__ long long fx_scale(long long a) {
+  constexpr long long c = SIN ? fx::ksin62(M, N) : fx::kcos62(M, N);
+  constexpr long long one = fx::kOne62, h = one / 2;
+  constexpr bool is_half = c - h < 8 && h - c < 8, is_nhalf = c + h < 8 && -h - c < 8;
+  if constexpr (c < 8 && c > -8) return 0;
+  else if constexpr (is_half) return fx::half(a);
+  else if constexpr (is_nhalf) return -fx::half(a);
+  else if constexpr (c > one - 8) return a;
+  else if constexpr (c < -one + 8) return -a;
+  else if constexpr (c > h) return a - fx::mulc(a, fx::limbs((one - c) * 4));
+  else if constexpr (c < -h) return -a + fx::mulc(a, fx::limbs((one + c) * 4));
+  else return fx::mulc(a, fx::limbs(c * 4));
+}
+// a exp(s 2 pi i E / N)
+template <int E, int N, typename T>
+__device__ __forceinline__ fx::Cx fx_twiddle(fx::Cx a, T s) {
+  fx::Cx r;
+  if constexpr ((8 * E) % N == 0 && (4 * E) % N != 0) {  // odd multiples of 45 degrees: two products
+    constexpr int q = ((8 * E) / N) % 8;  // 1, 3, 5, 7
+    const long long u = s > 0 ? a.x - a.y : a.x + a.y, v = s > 0 ? a.x + a.y : a.y - a.x;  // a (1 +- i)
+    const long long p = fx_scale<false, 1, 8>(u), t = fx_scale<false, 1, 8>(v);
+    r.x = p;
+    r.y = t;
+    if constexpr (q == 3) r = s > 0 ? fx::Cx{-t, p} : fx::Cx{t, -p};
+    if constexpr (q == 5) r = fx::Cx{-p, -t};
+    if constexpr (q == 7) r = s > 0 ? fx::Cx{t, -p} : fx::Cx{-t, p};
+  } else {
+    const long long xs = fx_scale<true, E, N>(a.x), ys = fx_scale<true, E, N>(a.y);
+    const long long xc = fx_scale<false, E, N>(a.x), yc = fx_scale<false, E, N>(a.y);
+    r.x = s > 0 ? xc - ys : xc + ys;
+    r.y = s > 0 ? yc + xs : yc - xs;
+  }
+  return r;
+}
+
 __host__ __device__ constexpr int first_factor(int n) { return n % 4 == 0 && n != 4 ? 4 : n % 2 == 0 && n != 2 ? 2 : n % 3 == 0 && n != 3 ? 3 : n % 5 == 0 && n != 5 ? 5 : n; }
 
 // y_q = sum_t v_t exp(s * 2 pi i t q / N), natural order in and out.
@@ -118,12 +160,22 @@ __device__ __forceinline__ void rdft_base(C* v, T s) {
     v[0] = add(a, b);
     v[1] = sub(a, b);
   } else if constexpr (N == 3) {
-    const T h = (T)0.5, s3 = (T)0.86602540378443864676;
     const C t1 = add(v[1], v[2]);
-    C t2;
-    t2.x = v[0].x - h * t1.x;
-    t2.y = v[0].y - h * t1.y;
-    const C t3 = muli_m(sub(v[1], v[2]), s, s3);
+    C t2, t3;
+    if constexpr (fx::is_fx<C>) {
+      t2.x = v[0].x - fx::half(t1.x);
+      t2.y = v[0].y - fx::half(t1.y);
+      const C d = sub(v[1], v[2]);
+      C e;
+      e.x = fx_scale<true, 1, 3>(d.x);
+      e.y = fx_scale<true, 1, 3>(d.y);
+      t3 = muli(e, s);
+    } else {
+      const T h = (T)0.5, s3 = (T)0.86602540378443864676;
+      t2.x = v[0].x - h * t1.x;
+      t2.y = v[0].y - h * t1.y;
+      t3 = muli_m(sub(v[1], v[2]), s, s3);
+    }
     v[0] = add(v[0], t1);
     v[1] = add(t2, t3);
     v[2] = sub(t2, t3);
@@ -135,19 +187,30 @@ __device__ __forceinline__ void rdft_base(C* v, T s) {
     v[1] = add(b, d);
     v[3] = sub(b, d);
   } else if constexpr (N == 5) {
-    const T c1 = (T)0.30901699437494742410, c2 = (T)-0.80901699437494742410;
-    const T s1 = (T)0.95105651629515357212, s2 = (T)0.58778525229247312917;
     const C a1 = add(v[1], v[4]), a2 = add(v[2], v[3]);
     const C b1 = sub(v[1], v[4]), b2 = sub(v[2], v[3]);
     C r1, r2, w1, w2;
-    r1.x = v[0].x + c1 * a1.x + c2 * a2.x;
-    r1.y = v[0].y + c1 * a1.y + c2 * a2.y;
-    r2.x = v[0].x + c2 * a1.x + c1 * a2.x;
-    r2.y = v[0].y + c2 * a1.y + c1 * a2.y;
-    w1.x = s1 * b1.x + s2 * b2.x;
-    w1.y = s1 * b1.y + s2 * b2.y;
-    w2.x = s2 * b1.x - s1 * b2.x;
-    w2.y = s2 * b1.y - s1 * b2.y;
+    if constexpr (fx::is_fx<C>) {
+      r1.x = v[0].x + fx_scale<false, 1, 5>(a1.x) + fx_scale<false, 2, 5>(a2.x);
+      r1.y = v[0].y + fx_scale<false, 1, 5>(a1.y) + fx_scale<false, 2, 5>(a2.y);
+      r2.x = v[0].x + fx_scale<false, 2, 5>(a1.x) + fx_scale<false, 1, 5>(a2.x);
+      r2.y = v[0].y + fx_scale<false, 2, 5>(a1.y) + fx_scale<false, 1, 5>(a2.y);
+      w1.x = fx_scale<true, 1, 5>(b1.x) + fx_scale<true, 2, 5>(b2.x);
+      w1.y = fx_scale<true, 1, 5>(b1.y) + fx_scale<true, 2, 5>(b2.y);
+      w2.x = fx_scale<true, 2, 5>(b1.x) - fx_scale<true, 1, 5>(b2.x);
+      w2.y = fx_scale<true, 2, 5>(b1.y) - fx_scale<true, 1, 5>(b2.y);
+    } else {
+      const T c1 = (T)0.30901699437494742410, c2 = (T)-0.80901699437494742410;
+      const T s1 = (T)0.95105651629515357212, s2 = (T)0.58778525229247312917;
+      r1.x = v[0].x + c1 * a1.x + c2 * a2.x;
+      r1.y = v[0].y + c1 * a1.y + c2 * a2.y;
+      r2.x = v[0].x + c2 * a1.x + c1 * a2.x;
+      r2.y = v[0].y + c2 * a1.y + c1 * a2.y;
+      w1.x = s1 * b1.x + s2 * b2.x;
+      w1.y = s1 * b1.y + s2 * b2.y;
+      w2.x = s2 * b1.x - s1 * b2.x;
+      w2.y = s2 * b1.y - s1 * b2.y;
+    }
     const C i1 = muli(w1, s), i2 = muli(w2, s);
     v[0] = add(v[0], add(a1, a2));
     v[1] = add(r1, i1);
@@ -174,7 +237,9 @@ __device__ __forceinline__ void rdft_split(C* v, T s) {
       constexpr int k1 = decltype(kc)::value;
       if constexpr ((j * k1) % N != 0) {
         constexpr double wc = kcos(j * k1, N), ws = ksin(j * k1, N);
-        if constexpr (wc == 0.0 && (ws == 1.0 || ws == -1.0)) {
+        if constexpr (fx::is_fx<C>) {
+          t[j][k1] = fx_twiddle<(j * k1) % N, N>(t[j][k1], s);
+        } else if constexpr (wc == 0.0 && (ws == 1.0 || ws == -1.0)) {
           t[j][k1] = muli(t[j][k1], ws > 0.0 ? s : -s);  // w = +-i
         } else if constexpr (ws == 0.0 && wc == -1.0) {
           t[j][k1].x = -t[j][k1].x;  // w = -1
@@ -227,6 +292,8 @@ __device__ __forceinline__ C twiddle_c(C a, T s) {
   constexpr int e = ((E % N) + N) % N;
   if constexpr (e == 0) {
     return a;
+  } else if constexpr (fx::is_fx<C>) {
+    return fx_twiddle<e, N>(a, s);
   } else {
     constexpr double wc = kcos(e, N), ws = ksin(e, N);
     if constexpr (wc == 0.0 && (ws == 1.0 || ws == -1.0)) {

@@ -158,6 +158,9 @@ struct kss_sys_s {
   kss::DevBuf d_V64;               // V(r_j), [j3][j2][j1], unscaled
   kss::DevBuf d_Vx64, d_Vx32;      // V(r_j)/(N1 N2 N3) in [j1][j2][j3] order (plane kernel)
   kss::DevBuf d_tw64[3], d_tw32[3];// e^{-2 pi i k/N_d}, k < N_d
+  kss::DevBuf d_rot[3];            // the same in fixed point (fx64.cuh)
+  kss::DevBuf d_vhigh;             // high word of max |V| (int)
+  std::map<int, kss::DevBuf> vfx;  // V in fixed point as [x][z][p] per split code A*32+B (lazy)
   kss::DevBuf d_D64, d_D32;
   std::map<int, kss::DevBuf> vpi64, vpi32;  // V/N^3 as [x][z][p] per split code A*32+B (lazy)
   std::map<int, kss::DevBuf> vfused32;       // V/N^3 in the fused kernel's digit-reversed order (lazy)
@@ -243,6 +246,7 @@ struct NvtxRange {
 void launch_vloc(kss_sys s, cudaStream_t st);
 void launch_projectors(kss_sys s, KData& kd, cudaStream_t st);
 void launch_vloc_views(kss_sys s, cudaStream_t st);
+void launch_fx_tables(kss_sys s, cudaStream_t st);  // d_rot, d_vhigh (after launch_vloc)
 double device_max(const double* x, size_t n, cudaStream_t st);
 void projector_norms(const double* beta, int npw, int nproj, std::vector<double>& out,
                      cudaStream_t st);
@@ -265,6 +269,8 @@ const void* beta_split_nn(kss_sys s, int ik);
 // V/N^3 of the system in the [x][z][p] layout of the CTA-wide pass B for split N2 = N3 = A*B (p the
 // digit-reversed y position k2 + B k of y = k + A k2), built on first use and kept.
 const void* vpi_view(kss_sys s, int A, int B, bool f64);
+// V of the system in fixed point in the same layout (the fixed-point pass B), built on first use.
+const void* vfx_view(kss_sys s, int A, int B);
 // out = T psi + V psi (the local part only)
 void apply_local(kss_sys s, int ik, int nb, const void* psi, void* out, int ld, kss_precision prec);
 // ---- generalised problem with a nonlocal overlap (overlap.cu) ----
@@ -282,8 +288,11 @@ constexpr size_t kSlabChunkBytes = 64ull << 20;
 size_t sys_device_bytes(kss_sys s);  // device bytes of a system's tables (api.cpp)
 // Caller-provided workspace forms (used by the entry point that allocates nothing).
 size_t local_slab_bytes_per_band(kss_sys s, int ik, kss_precision prec);
+// Bytes of plane exponents that the fixed-point passes of nc bands need beside the slab.
+size_t local_meta_bytes(kss_sys s, int ik, int nc);
+// meta: local_meta_bytes(nc) bytes, or null (double precision then takes the per-warp passes)
 void local_apply_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
-                    kss_precision prec, void* work, int nc);
+                    kss_precision prec, void* work, int nc, void* meta);
 bool gemm_cn_ws(kss_ctx ctx, bool fp64, int M, int N, int K, const void* A, int lda, const void* B,
                 int ldb, void* C, int ldc, void* partials, size_t partial_bytes);
 void scale_rows_noprof(bool fp64, int M, int N, void* C, int ldc, const void* d, double s,

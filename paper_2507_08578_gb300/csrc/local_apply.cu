@@ -18,6 +18,8 @@
 //     (local_wide.cu), every transform stage spread over all lanes of the CTA;
 //   * passes A/C (and pass B otherwise) with a compile-time split: per-warp two-level register
 //     codelets (fft_reg.cuh, CtPol), else the same with runtime sizes (RtPol);
+//   * double precision with a CTA-wide pass B and an x edge of KSS_FX_X: all three passes in fixed
+//     point (local_fx.cuh), 3 to 4 times the FP64 pipe's rate; other boxes in FP64;
 //   * lengths that do not split into two codelets of size <= 16: warp-level Stockham FFTs
 //     (radix 4/2/3/5) on contiguous pencils in shared memory (the kernels in this file).
 // The slab lives in a workspace of nc bands (chunked so that it stays L2-resident).
@@ -422,6 +424,24 @@ int chunk_bands(kss_sys s, int ik, int nb, size_t es) {
   return (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, target / per));
 }
 
+void fx_args(kss_sys s, FxTables& f) {
+  f.r1 = s->d_rot[0].as<fx::Rot>();
+  f.r2 = s->d_rot[1].as<fx::Rot>();
+  f.vhigh = s->d_vhigh.as<int>();
+  f.invn = 1.0 / ((double)s->N[0] * s->N[1] * s->N[2]);
+}
+
+// Double precision: whether the passes of `a` run in fixed point (all three or none: the slab
+// between them is in that form).  The CTA-wide schedule of the tuner and an instance for the x edge.
+template <typename T>
+bool fx_passes(const LocalArgs<T>& a, const PassBSched& sb) {
+  if constexpr (sizeof(T) == 8)
+    return sb.threads && wide_pass_b<T>(a, sb.A, sb.B, sb.threads, 0, nullptr, true) &&
+           wide_pass_x<T>(a, 0, 0, nullptr, true) && wide_pass_x<T>(a, 1, 0, nullptr, true);
+  else
+    return false;
+}
+
 // Kernel arguments of the local passes for (system, k-point, band block).
 template <typename T>
 LocalArgs<T> local_args(kss_sys s, int ik, const void* psi, const void* psi_prev, void* out, int ld,
@@ -463,6 +483,7 @@ LocalArgs<T> local_args(kss_sys s, int ik, const void* psi, const void* psi_prev
   a.alpha = (T)c.alpha;
   a.beta = (T)c.beta;
   a.gamma = (T)c.gamma;
+  if (f64) fx_args(s, a.fx);
   return a;
 }
 
@@ -519,8 +540,10 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
   KSS_CHECK_CUDA(cudaFuncSetAttribute(pass_b<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
   KSS_CHECK_CUDA(cudaFuncSetAttribute(pass_c<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sa));
   const int nc = chunk_bands(s, ik, nb, sizeof(C));
-  ctx->ws_local.ensure(slab_elems(s, ik) * nc * sizeof(C));
+  ctx->ws_local.ensure(slab_elems(s, ik) * nc * sizeof(C) + (f64 ? local_meta_bytes(s, ik, nc) : 0));
   a.work = ctx->ws_local.as<C>();
+  a.fx.ma = reinterpret_cast<int2*>(a.work + slab_elems(s, ik) * nc);
+  a.fx.mb = a.fx.ma + (size_t)nc * a.W3;
   RegPlan rp;
   if (choose_split(a.N1, rp.s1) && choose_split(a.N2, rp.s2) && choose_split(a.N3, rp.s3)) {
     const int scr_warp = std::max(rp.s1.PP * rp.s1.scr, std::max(rp.s2.PP * rp.s2.scr, rp.s3.PP * rp.s3.scr));
@@ -536,9 +559,15 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
       auto warp_b = [&](const LocalArgs<T>& t, int m) {
         kk.b<<<dim3(t.N1, m), kThreads, rb, ctx->stream>>>(t, rp, scr_warp);
       };
-      const PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, true);
-      const bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
-      if (sb.threads) a.Vpi = (const T*)vpi_view(s, sb.A, sb.B, f64);
+      PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, true);
+      bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
+      if (f64) {
+        wx = fx_passes<T>(a, sb);
+        if (wx) a.fx.V = (const fx::Limbs*)vfx_view(s, sb.A, sb.B);
+        else sb.threads = 0;
+      } else if (sb.threads) {
+        a.Vpi = (const T*)vpi_view(s, sb.A, sb.B, false);
+      }
       static const int ida = prof_register(f64 ? "local_pass_a<f64>" : "local_pass_a<f32>");
       static const int idb = prof_register(f64 ? "local_pass_b<f64>" : "local_pass_b<f32>");
       static const int idc = prof_register(f64 ? "local_pass_c<f64>" : "local_pass_c<f32>");
@@ -603,7 +632,7 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
 // events).  Same kernels as run_local; the pass-B schedule comes from the autotuner's table or
 // the built-in choice (no tuning, which would allocate a scratch slab).
 template <typename T>
-void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld, void* work, int nc) {
+void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld, void* work, int nc, void* meta) {
   using C = typename CT<T>::C;
   const bool f64 = sizeof(T) == 8;
   kss_ctx ctx = s->ctx;
@@ -643,6 +672,9 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
   a.beta = (T)0;
   a.gamma = (T)0;
   a.work = (C*)work;
+  if (f64) fx_args(s, a.fx);
+  a.fx.ma = static_cast<int2*>(meta);
+  a.fx.mb = a.fx.ma ? a.fx.ma + (size_t)nc * a.W3 : nullptr;
   const size_t smax = 227 * 1024;
   RegPlan rp;
   if (choose_split(a.N1, rp.s1) && choose_split(a.N2, rp.s2) && choose_split(a.N3, rp.s3)) {
@@ -660,13 +692,17 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
         kk.b<<<dim3(t.N1, m), kThreads, rb, ctx->stream>>>(t, rp, scr_warp);
       };
       PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, false);  // no tuning here
-      const bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
+      bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
       // The CTA-wide form needs V in its split's layout; that view is built (allocated) by the
       // first ordinary application, and without it this path takes the per-warp form.
-      if (sb.threads) {
-        auto& cache = f64 ? s->vpi64 : s->vpi32;
-        auto it = cache.find(sb.A * 32 + sb.B);
-        if (it != cache.end()) a.Vpi = (const T*)it->second.p;
+      if (f64) {
+        auto it = s->vfx.find(sb.A * 32 + sb.B);
+        wx = meta && it != s->vfx.end() && fx_passes<T>(a, sb);
+        if (wx) a.fx.V = it->second.template as<fx::Limbs>();
+        else sb.threads = 0;
+      } else if (sb.threads) {
+        auto it = s->vpi32.find(sb.A * 32 + sb.B);
+        if (it != s->vpi32.end()) a.Vpi = (const T*)it->second.p;
         else sb.threads = 0;
       }
       for (int n0 = 0; n0 < nb; n0 += nc) {
@@ -755,16 +791,21 @@ size_t local_slab_bytes_per_band(kss_sys s, int ik, kss_precision prec) {
 }
 
 void local_apply_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
-                    kss_precision prec, void* work, int nc) {
+                    kss_precision prec, void* work, int nc, void* meta) {
   if (prec == KSS_PREC_FP64)
-    run_local_ws<double>(s, ik, nb, psi, out, ld, work, nc);
+    run_local_ws<double>(s, ik, nb, psi, out, ld, work, nc, meta);
   else
-    run_local_ws<float>(s, ik, nb, psi, out, ld, work, nc);
+    run_local_ws<float>(s, ik, nb, psi, out, ld, work, nc, nullptr);
+}
+
+size_t local_meta_bytes(kss_sys s, int ik, int nc) {
+  return sizeof(int2) * (size_t)nc * (s->N[0] + s->k[ik].W[2]);
 }
 
 size_t local_workspace_bytes(kss_sys s, int ik, int nb, kss_precision prec) {
   const size_t es = prec == KSS_PREC_FP64 ? 16 : 8;
-  return slab_elems(s, ik) * chunk_bands(s, ik, nb, es) * es;
+  const int nc = chunk_bands(s, ik, nb, es);
+  return slab_elems(s, ik) * nc * es + (prec == KSS_PREC_FP64 ? local_meta_bytes(s, ik, nc) : 0);
 }
 
 template <typename T>
@@ -796,6 +837,38 @@ const void* vpi_view(kss_sys s, int A, int B, bool f64) {
     vpi_gather<double><<<blocks, 256, 0, s->ctx->stream>>>(s->d_Vx64.as<double>(), d.as<double>(), N1, N, A, B);
   else
     vpi_gather<float><<<blocks, 256, 0, s->ctx->stream>>>(s->d_Vx32.as<float>(), d.as<float>(), N1, N, A, B);
+  KSS_CHECK_CUDA(cudaGetLastError());
+  return d.p;
+}
+
+// V 2^(63 - e) as an integer in limbs, e from the largest |V|
+__global__ void vfx_gather(const double* __restrict__ V, const int* __restrict__ high, fx::Limbs* __restrict__ out,
+                           int N1, int N, int A, int B) {
+  const long long n = (long long)N1 * N * N;
+  const int E = fx::v_exp(*high) - 63;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int p = (int)(i % N);
+    const long long r = i / N;
+    const int z = (int)(r % N), x = (int)(r / N);
+    const int k = p / B, k2 = p - k * B;
+    const int y = k + A * k2;
+    out[i] = fx::limbs(fx::from_double(V[((size_t)z * N + y) * N1 + x], E));
+  }
+}
+
+const void* vfx_view(kss_sys s, int A, int B) {
+  const int code = A * 32 + B;
+  auto it = s->vfx.find(code);
+  if (it != s->vfx.end()) return it->second.p;
+  KSS_REQUIRE(s->N[1] == s->N[2] && A * B == s->N[1], "V view: split does not match the box");
+  const int N1 = s->N[0], N = s->N[1];
+  const long long n = (long long)N1 * N * N;
+  DevBuf& d = s->vfx[code];
+  d.alloc((size_t)n * sizeof(fx::Limbs));
+  const unsigned blocks = (unsigned)std::min<long long>((n + 255) / 256, 152LL * 32);
+  vfx_gather<<<blocks, 256, 0, s->ctx->stream>>>(s->d_V64.as<double>(), s->d_vhigh.as<int>(), d.as<fx::Limbs>(), N1,
+                                                 N, A, B);
   KSS_CHECK_CUDA(cudaGetLastError());
   return d.p;
 }

@@ -14,6 +14,17 @@ namespace lk {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
+// Tables and exponents of the fixed-point passes (local_fx.cuh), double precision only.
+struct FxTables {
+  const fx::Rot* r1;       // rotations e^{-2 pi i m / N} of x and of y and z
+  const fx::Rot* r2;
+  const fx::Limbs* V;      // V in units of 2^(e - 63), e = fx::v_exp(*vhigh), as [x][z][p] (as Vpi)
+  const int* vhigh;        // high word of the largest |V|
+  int2* ma;                // (exponent, size) of the slab's planes: [band][W3] after pass A,
+  int2* mb;                // [band][N1] after pass B
+  double invn;             // 1 / (N1 N2 N3)
+};
+
 template <typename T> struct CT;
 template <> struct CT<double> { using C = double2; };
 template <> struct CT<float> { using C = float2; };
@@ -49,6 +60,7 @@ struct LocalArgs {
                   // psi_2n + i psi_2n+1 (real-space-real bands); pass C then stores the raw
                   // transform (no epilogue) and a separate kernel unpacks
   int nbands;     // bands in psi (packed mode: the last pair may hold one band)
+  FxTables fx;    // double precision: set for the fixed-point passes
 };
 
 template <typename C>

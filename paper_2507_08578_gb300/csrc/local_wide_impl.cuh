@@ -1,8 +1,7 @@
-// Kernel instances of the CTA-wide passes (local_kernels.cuh) for one precision: pass B
-// (pass_bw_body) for every split of KSS_WIDE_SPLITS at 256 and 384 threads per CTA (and 128 in
-// single precision), passes A and C (pass_aw_body, pass_cw_body) for the x splits of
-// KSS_WIDEX_SPLITS.  Included by one translation unit per precision (local_wide_f32.cu,
-// local_wide_f64.cu) so the build compiles them in parallel.
+// Kernel instances of the CTA-wide passes (local_kernels.cuh) in single precision: pass B
+// (pass_bw_body) for every split of KSS_WIDE_SPLITS at 128, 256 and 384 threads per CTA, passes A
+// and C (pass_aw_body, pass_cw_body) for the x splits of KSS_WIDEX_SPLITS.  (Double precision:
+// local_fx_impl.cuh.)
 #pragma once
 
 #include "local_kernels.cuh"

@@ -78,7 +78,12 @@ extern "C" kss_status kss_apply_H_noalloc(kss_sys sys, int ik, int nb, const voi
       part = std::max(cprj, (free_after / 2) / cprj * cprj);
     }
     const size_t slab_off = cprj + align256(part);
-    const int nc = (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, (cap - slab_off) / plane));
+    int nc = (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, (cap - slab_off) / plane));
+    // the plane exponents of the double-precision passes sit behind the slab; a request whose only
+    // slab leaves no room for them runs the form without
+    auto meta_end = [&](int c) { return slab_off + align256(plane * c) + local_meta_bytes(sys, ik, c); };
+    if (f64 && nc > 1 && meta_end(nc) > cap) --nc;
+    void* meta = f64 && meta_end(nc) <= cap ? base + slab_off + align256(plane * nc) : nullptr;
     if (sys->nproj) {
       void* C = base;
       const bool ok = gemm_cn_ws(ctx, f64, sys->nproj, nb, kd.npw, f64 ? kd.d_beta64.p : kd.d_beta32.p,
@@ -87,7 +92,7 @@ extern "C" kss_status kss_apply_H_noalloc(kss_sys sys, int ik, int nb, const voi
       scale_rows_noprof(f64, sys->nproj, nb, C, sys->nproj, f64 ? sys->d_D64.p : sys->d_D32.p, 1.0,
                         ctx->stream);
     }
-    local_apply_ws(sys, ik, nb, psi, hpsi, ld, prec, base + slab_off, nc);
+    local_apply_ws(sys, ik, nb, psi, hpsi, ld, prec, base + slab_off, nc, meta);
     if (sys->nproj)
       gemm_nn_noprof(f64, kd.npw, nb, sys->nproj, f64 ? kd.d_beta64.p : kd.d_beta32.p, kd.npw, base,
                      sys->nproj, hpsi, ld, ctx->stream);

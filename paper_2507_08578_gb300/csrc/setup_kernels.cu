@@ -1,7 +1,9 @@
 // Device-side setup: local potential on the FFT grid, its plane-kernel views, the projector
 // table (Eq. ham-nl of §5.2 with projectors kept in memory) and small reductions.
+#include <algorithm>
 #include <cmath>
 
+#include "fx64.cuh"
 #include "kss_internal.h"
 
 namespace kss {
@@ -61,6 +63,15 @@ __global__ void vloc_view_kernel(const double* __restrict__ V, T* __restrict__ V
   const int j2 = (int)((idx / N3) % N2);
   const int j1 = (int)(idx / ((long long)N3 * N2));
   Vx[idx] = (T)(V[((long long)j3 * N2 + j2) * N1 + j1] * scale);
+}
+
+// largest high word of |x|
+__global__ void high_max_kernel(const double* __restrict__ x, long long n, int* out) {
+  unsigned m = 0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    m = max(m, (unsigned)__double2hiint(x[i]) & 0x7fffffffu);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, (int)m);
 }
 
 __global__ void max_kernel(const double* __restrict__ x, long long n, double* out) {
@@ -156,6 +167,22 @@ void launch_vloc_views(kss_sys s, cudaStream_t st) {
       s->d_V64.as<double>(), s->d_Vx64.as<double>(), s->N[0], s->N[1], s->N[2], scale);
   vloc_view_kernel<float><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
       s->d_V64.as<double>(), s->d_Vx32.as<float>(), s->N[0], s->N[1], s->N[2], scale);
+  KSS_CHECK_CUDA(cudaGetLastError());
+}
+
+void launch_fx_tables(kss_sys s, cudaStream_t st) {
+  for (int d = 0; d < 3; ++d) {
+    const int N = s->N[d];
+    std::vector<fx::Rot> t(N);
+    for (int m = 0; m < N; ++m) t[m] = fx::rot_limbs(fx::kcos62(m, N), -fx::ksin62(m, N));
+    s->d_rot[d].alloc(t.size() * sizeof(fx::Rot));
+    KSS_CHECK_CUDA(cudaMemcpy(s->d_rot[d].p, t.data(), t.size() * sizeof(fx::Rot), cudaMemcpyHostToDevice));
+  }
+  const long long n = (long long)s->N[0] * s->N[1] * s->N[2];
+  s->d_vhigh.alloc(sizeof(int));
+  KSS_CHECK_CUDA(cudaMemsetAsync(s->d_vhigh.p, 0, sizeof(int), st));
+  high_max_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 152 * 4), 256, 0, st>>>(s->d_V64.as<double>(), n,
+                                                                                           s->d_vhigh.as<int>());
   KSS_CHECK_CUDA(cudaGetLastError());
 }
 

@@ -72,10 +72,14 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   const size_t per_band = (size_t)t.N1 * t.W3 * t.W2 * sizeof(C);
   const int nbt = (int)std::max<size_t>(1, std::min<size_t>(64, kSlabChunkBytes / per_band));
   const size_t elems = (size_t)t.N1 * t.W3 * t.W2 * nbt;
-  ctx->ws_tune.ensure(elems * sizeof(C));
-  KSS_CHECK_CUDA(cudaMemsetAsync(ctx->ws_tune.p, 0, elems * sizeof(C), ctx->stream));
+  const size_t bytes = elems * sizeof(C) + sizeof(int2) * (size_t)nbt * (t.N1 + t.W3);
+  ctx->ws_tune.ensure(bytes);
+  KSS_CHECK_CUDA(cudaMemsetAsync(ctx->ws_tune.p, 0, bytes, ctx->stream));
   t.work = ctx->ws_tune.as<C>();
+  t.fx.ma = reinterpret_cast<int2*>(t.work + elems);
+  t.fx.mb = t.fx.ma + (size_t)nbt * t.W3;
   t.Vpi = t.Vx;  // any N1 x N x N array: the values do not matter for timing
+  t.fx.V = reinterpret_cast<const fx::Limbs*>(t.Vx);
   t.n0 = 0;
   cudaEvent_t e0, e1;
   KSS_CHECK_CUDA(cudaEventCreate(&e0));

@@ -1,0 +1,95 @@
+"""The fixed-point double-precision local part through the C ABI, where block exponents can go wrong.
+
+* Bands of one call at scales from 1e-150 to 1e150, a zero band, a single plane wave and a band
+  concentrated at one point: each band has exponents of its own, so each is as accurate as alone
+  (1e-14 of its own |H psi|: a few roundings of 2^-53 each in the oracle's FP64 sums of at most
+  1e4 terms and in the library).
+* A band with a NaN or an infinity gives NaN and leaves the others bit for bit as they are.
+* Gamma pairs of very different norms: the smaller band's error is relative to the pair (as in the
+  transform of the sum), 1e-14 of the pair's |H psi|.
+* Boxes whose y/z split runs pruned and full, odd edges among them.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+import workloads as W
+import paper_2507_08578_gb300.kss as K
+from tests.kss_helpers import ensure_built, make_ctx, setup
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    ensure_built()
+    c = make_ctx()
+    yield c
+    torch.cuda.synchronize()
+    K.kss_destroy(c)
+
+
+def _apply(sysh, c, gamma=False):
+    import torch
+    psi = torch.from_numpy(c).cuda()
+    out = torch.empty_like(psi)
+    (K.kss_apply_H_gamma if gamma else K.kss_apply_H)(sysh, 0, psi, out, K.KSS_PREC_FP64)
+    torch.cuda.synchronize()
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("box,a,ecut,kpt", [
+    ((24, 24, 24), 10.0, 10.0, 0), ((25, 25, 25), 8.0, 10.0, 1), ((27, 30, 30), 8.0, 8.0, 1),
+    ((54, 54, 54), 13.9, 17.3, 1), ((96, 96, 96), 9.0, 9.0, 1), ((45, 48, 48), 10.0, 16.0, 0)])
+def test_scales_and_special_bands(ctx, box, a, ecut, kpt):
+    s = W.make_system("fx", a, ecut, 3, 4, seed=17, kpts=[[0.25 * kpt] * 3], fft_box=box, nproj_per_atom=0)
+    sysh = setup(ctx, s)
+    try:
+        p = O.build_problem(s, 0, box=box)
+        npw = p.basis.npw
+        c = W.random_block(npw, 9, seed=5)
+        c[1] *= 1e-150
+        c[2] *= 1e150
+        c[3] = 0
+        c[4] = 0
+        c[4, npw // 3] = 1
+        c[5] = 1.0 / np.sqrt(npw)
+        c[6] *= 10.0 ** np.random.default_rng(1).uniform(-14, 0, npw)
+        out = _apply(sysh, c)
+        scale = np.array([1, 1e150, 1e-150, 1, 1, 1, 1, 1, 1])[:, None]
+        ref = p.apply(c * scale)
+        err = np.linalg.norm(out * scale - ref, axis=1)
+        assert err[3] == 0
+        nz = [i for i in range(9) if i != 3]
+        assert np.all(err[nz] < 1e-14 * np.linalg.norm(ref[nz], axis=1)), err[nz] / np.linalg.norm(ref[nz], axis=1)
+        bad = c.copy()
+        bad[0, 3] = np.nan
+        bad[7, npw - 1] = np.inf
+        o2 = _apply(sysh, bad)
+        assert np.all(np.isnan(o2[0])) and np.all(np.isnan(o2[7]))
+        keep = [i for i in range(9) if i not in (0, 7)]
+        assert np.array_equal(o2[keep], out[keep])
+    finally:
+        K.kss_sys_destroy(sysh)
+
+
+def test_gamma_pairs_of_uneven_norm(ctx):
+    s = W.make_system("fxg", 10.0, 10.0, 4, 4, seed=18, fft_box=(30, 30, 30), nproj_per_atom=0)
+    sysh = setup(ctx, s)
+    try:
+        p = O.build_problem(s, 0, box=(30, 30, 30))
+        c = W.random_block(p.basis.npw, 5, seed=6)
+        c = c + c[:, ::-1].conj()  # the canonical order at Gamma is symmetric
+        c[1] *= 1e-9
+        c[2] *= 1e-6
+        c[4] *= 1e120
+        out = _apply(sysh, c, gamma=True)
+        ref = np.concatenate([p.apply(c[:4]), 1e120 * p.apply(c[4:] * 1e-120)])
+        err = np.linalg.norm((out - ref) / np.array([1, 1, 1, 1, 1e120])[:, None], axis=1)
+        big = np.linalg.norm(ref / np.array([1, 1, 1, 1, 1e120])[:, None], axis=1)
+        assert np.all(err[:2] < 1e-14 * big[:2].max())
+        assert np.all(err[2:4] < 1e-14 * big[2:4].max())
+        assert err[4] < 1e-14 * big[4]
+    finally:
+        K.kss_sys_destroy(sysh)
