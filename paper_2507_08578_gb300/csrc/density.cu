@@ -11,6 +11,7 @@
 
 #include "density.h"
 #include "kss_internal.h"
+#include "local_wide.h"
 
 namespace kss {
 
@@ -209,15 +210,15 @@ void density_t(kss_sys s, int ik, int nb, const void* psi, int ld, const double*
   int resident = 1;
   if (!(s->N[1] == s->N[2] && choose_split(s->N[1], sp)))
     fail(KSS_ENOTSUP, "kss_density_accumulate needs N2 == N3 with a two-codelet split");
-  {
-    LocalArgs<T> probe{};
-    probe.N1 = s->N[0];
-    probe.N2 = s->N[1];
-    probe.N3 = s->N[2];
-    probe.W3 = s->k[ik].W[2];
-    if (!pass_d<T>(probe, sp.A, sp.B, 0, 1, nullptr, nullptr, nullptr, true, &resident))
-      fail(KSS_ENOTSUP, "no density kernel instance for this FFT length / window");
-  }
+  const LocalArgs<T> args = density_args<T>(s, ik, psi, ld);
+  // double precision: in fixed point where the x edge and the box have instances (20 bohr cell, 512
+  // bands: 9.8 ms, 33.9 on the FP64 pipe)
+  bool fx = false;
+  if constexpr (sizeof(T) == 8)
+    fx = wide_pass_x<T>(args, 0, 0, nullptr, true) &&
+         density_pass_fx(args, sp.A, sp.B, 0, 1, nullptr, nullptr, nullptr, &resident);
+  if (!fx && !pass_d<T>(args, sp.A, sp.B, 0, 1, nullptr, nullptr, nullptr, true, &resident))
+    fail(KSS_ENOTSUP, "no density kernel instance for this FFT length / window");
   const int N1 = s->N[0], N2 = s->N[1], N3 = s->N[2];
   const int cap = std::max(1, ctx->nsm) * std::max(1, resident);
   // Band groups of a chunk of m bands: G maximising (fill of the last wave of N1*G CTAs) x
@@ -243,8 +244,15 @@ void density_t(kss_sys s, int ik, int nb, const void* psi, int ld, const double*
                                  ctx->stream));
   KSS_CHECK_CUDA(cudaMemsetAsync(ctx->ws_rho.p, 0, (size_t)G * N1 * N2 * N3 * sizeof(double), ctx->stream));
   static const int idd = prof_register(sizeof(T) == 8 ? "density_pass<f64>" : "density_pass<f32>");
-  pass_a_chunks<T>(s, ik, nb, psi, ld, [&](const LocalArgs<T>& a, int m) {
+  pass_a_chunks<T>(s, ik, nb, args, fx, [&](const LocalArgs<T>& a, int m) {
     ProfScope ps(ctx, idd);
+    if constexpr (sizeof(T) == 8) {
+      if (fx) {
+        density_pass_fx(a, sp.A, sp.B, m, groups(m), ctx->ws_occ.as<double>(), ctx->ws_rho.as<double>(), ctx->stream,
+                        nullptr);
+        return;
+      }
+    }
     pass_d<T>(a, sp.A, sp.B, m, groups(m), ctx->ws_occ.as<double>(), ctx->ws_rho.as<double>(), ctx->stream, false);
   });
   static const int idr = prof_register("density_reduce");

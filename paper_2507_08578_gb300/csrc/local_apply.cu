@@ -753,11 +753,17 @@ template void warp_pass_b<double>(kss_ctx, const LocalArgs<double>&, int);
 template void warp_pass_b<float>(kss_ctx, const LocalArgs<float>&, int);
 
 template <typename T>
-void pass_a_chunks(kss_sys s, int ik, int nb, const void* psi, int ld,
+LocalArgs<T> density_args(kss_sys s, int ik, const void* psi, int ld) {
+  return local_args<T>(s, ik, psi, nullptr, nullptr, ld, ChebCoef{1.0, 0.0, 0.0});
+}
+template LocalArgs<double> density_args<double>(kss_sys, int, const void*, int);
+template LocalArgs<float> density_args<float>(kss_sys, int, const void*, int);
+
+template <typename T>
+void pass_a_chunks(kss_sys s, int ik, int nb, LocalArgs<T> a, bool fx,
                    const std::function<void(const LocalArgs<T>&, int)>& after) {
   using C = typename CT<T>::C;
   kss_ctx ctx = s->ctx;
-  LocalArgs<T> a = local_args<T>(s, ik, psi, nullptr, nullptr, ld, ChebCoef{1.0, 0.0, 0.0});
   RegPlan rp;
   if (!(choose_split(a.N1, rp.s1) && choose_split(a.N2, rp.s2) && choose_split(a.N3, rp.s3)))
     fail(KSS_ENOTSUP, "FFT length without a two-codelet split");
@@ -765,25 +771,27 @@ void pass_a_chunks(kss_sys s, int ik, int nb, const void* psi, int ld,
   const size_t ra = sizeof(C) * ((size_t)a.N1 + (size_t)a.W2 * a.N1p + (size_t)kWarps * scr_warp);
   if (ra > 227 * 1024) fail(KSS_ENOTSUP, "FFT box too large for the shared-memory pencil tiles");
   const PassKernels<T> kk = pick_kernels<T>(rp);
-  KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ra));
+  if (!fx) KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ra));
   const int nc = chunk_bands(s, ik, nb, sizeof(C));
-  ctx->ws_local.ensure(slab_elems(s, ik) * nc * sizeof(C));
+  ctx->ws_local.ensure(slab_elems(s, ik) * nc * sizeof(C) + (fx ? local_meta_bytes(s, ik, nc) : 0));
   a.work = ctx->ws_local.as<C>();
+  if (fx) a.fx.ma = reinterpret_cast<int2*>(a.work + slab_elems(s, ik) * nc);
   static const int ida = prof_register(sizeof(T) == 8 ? "local_pass_a<f64>" : "local_pass_a<f32>");
   for (int n0 = 0; n0 < nb; n0 += nc) {
     const int m = std::min(nc, nb - n0);
     a.n0 = n0;
     {
       ProfScope ps(ctx, ida);
-      kk.a<<<dim3(a.W3, m), kThreads, ra, ctx->stream>>>(a, rp, scr_warp);
+      if (fx) wide_pass_x<T>(a, 0, m, ctx->stream, false);
+      else kk.a<<<dim3(a.W3, m), kThreads, ra, ctx->stream>>>(a, rp, scr_warp);
     }
     after(a, m);
   }
   KSS_CHECK_CUDA(cudaGetLastError());
 }
-template void pass_a_chunks<double>(kss_sys, int, int, const void*, int,
+template void pass_a_chunks<double>(kss_sys, int, int, LocalArgs<double>, bool,
                                     const std::function<void(const LocalArgs<double>&, int)>&);
-template void pass_a_chunks<float>(kss_sys, int, int, const void*, int,
+template void pass_a_chunks<float>(kss_sys, int, int, LocalArgs<float>, bool,
                                    const std::function<void(const LocalArgs<float>&, int)>&);
 
 size_t local_slab_bytes_per_band(kss_sys s, int ik, kss_precision prec) {

@@ -177,28 +177,51 @@ struct FxB {
   }
 };
 
+// Shared memory of a plane's y and z transforms (pass B, density).
+template <int A, int B>
+struct FxPlane {
+  using G = FxB<A, B>;
+  Rot* tw;
+  Cx* Q;      // W3 rows (z in the sphere window) x N (y)
+  Cx* Z;      // N columns (y position) x N (z)
+  int* zmap;
+  int* rs;    // shift of each row at the load
+  int* word;  // sizes after each of 8 stages, top exponent, bad
+  __device__ FxPlane(const LocalArgs<double>& a, unsigned char* sm) {
+    tw = reinterpret_cast<Rot*>(sm);
+    Q = reinterpret_cast<Cx*>(tw + G::N);
+    Z = Q + a.W3 * G::QS;
+    zmap = reinterpret_cast<int*>(Z + G::N * G::ZS);
+    rs = zmap + G::N;
+    word = rs + a.W3;
+  }
+  // the rotations and the window's z map, once per CTA
+  __device__ void tables(const LocalArgs<double>& a) const {
+    for (int i = threadIdx.x; i < G::N; i += blockDim.x) tw[i] = a.fx.r2[i];
+    for (int z = threadIdx.x; z < G::N; z += blockDim.x) {
+      int u = (z - a.lo3) % G::N;
+      if (u < 0) u += G::N;
+      zmap[z] = u < a.W3 ? u : -1;
+    }
+  }
+};
+
+// Slab plane (x, nl) through the y transform and the first stage of the z transform: Z ready for its
+// DFT-B stage (in that stage's range), values v 2^E.  Returns E; bad: the band is not finite.
 template <int A, int B, int CW>
-__device__ __forceinline__ void fx_pass_b(const LocalArgs<double>& a, int x, int nl) {
+__device__ __forceinline__ int fx_inverse(const LocalArgs<double>& a, int x, int nl, const FxPlane<A, B>& s,
+                                          bool& bad) {
   using G = FxB<A, B>;
   constexpr int N = G::N, QS = G::QS, ZS = G::ZS;
   constexpr unsigned MW = fftr::edge_mask<A, CW>(), MF = fftr::full_mask<A>();
   constexpr int kWin = fx::kLimit(popcount_mask<A>(MW));
-  extern __shared__ __align__(16) unsigned char smraw[];
-  Rot* tw = reinterpret_cast<Rot*>(smraw);
-  Cx* Q = reinterpret_cast<Cx*>(tw + N);         // W3 rows (z in the sphere window) x N (y)
-  Cx* Z = Q + a.W3 * QS;                         // N columns (y position) x N (z)
-  int* zmap = reinterpret_cast<int*>(Z + N * ZS);
-  int* rs = zmap + N;                            // shift of each row at the load
-  int* word = rs + a.W3;                  // sizes after each of 8 stages, top exponent, bad
+  const Rot* tw = s.tw;
+  Cx *Q = s.Q, *Z = s.Z;
+  const int* zmap = s.zmap;
+  int *rs = s.rs, *word = s.word;
   const int tid = threadIdx.x, NT = blockDim.x;
   const int W3 = a.W3, W2 = a.W2;
   if (tid < 10) word[tid] = tid == 8 ? INT_MIN / 2 : 0;
-  for (int i = tid; i < N; i += NT) tw[i] = a.fx.r2[i];
-  for (int z = tid; z < N; z += NT) {
-    int u = (z - a.lo3) % N;
-    if (u < 0) u += N;
-    zmap[z] = u < W3 ? u : -1;
-  }
   for (int i = tid; i < W3 * QS; i += NT) Q[i] = Cx{0, 0};
   const int2* ma = a.fx.ma + (size_t)nl * W3;
   __syncthreads();
@@ -210,9 +233,9 @@ __device__ __forceinline__ void fx_pass_b(const LocalArgs<double>& a, int x, int
   }
   __syncthreads();
   constexpr int kLoad = kWin - 1;  // leaves the shift after the first stage to the exception
-  const bool bad = word[9] != 0;
+  bad = word[9] != 0;
   int E = (word[8] == INT_MIN / 2 ? 0 : word[8]) - kLoad;
-  Cx* slab = reinterpret_cast<Cx*>(a.work) + ((size_t)nl * a.N1 + x) * W3 * W2;
+  const Cx* slab = reinterpret_cast<const Cx*>(a.work) + ((size_t)nl * a.N1 + x) * W3 * W2;
   const fftr::FastDiv dw2(W2), dw3(W3);
   for (int i = tid; i < W3 * W2; i += NT) {
     const int u3 = dw2(i), u2 = i - u3 * W2;
@@ -298,9 +321,29 @@ __device__ __forceinline__ void fx_pass_b(const LocalArgs<double>& a, int x, int
     mag.put(word + 2);
   }
   __syncthreads();
-  // ---- z, inverse stage 2, x V / 2 ----
   sh = refit(Z, N * ZS, fx::mag_bits(word[2]), fx::kLimit(B));
-  E += 1 + sh;
+  return E + sh;
+}
+
+template <int A, int B, int CW>
+__device__ __forceinline__ void fx_pass_b(const LocalArgs<double>& a, int x, int nl) {
+  using G = FxB<A, B>;
+  constexpr int N = G::N, QS = G::QS, ZS = G::ZS;
+  constexpr unsigned MW = fftr::edge_mask<A, CW>(), MF = fftr::full_mask<A>();
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const FxPlane<A, B> pl(a, smraw);
+  const Rot* tw = pl.tw;
+  Cx *Q = pl.Q, *Z = pl.Z;
+  const int* zmap = pl.zmap;
+  int* word = pl.word;
+  const int tid = threadIdx.x, NT = blockDim.x;
+  const int W3 = a.W3, W2 = a.W2;
+  const fftr::FastDiv dw2(W2), dw3(W3);
+  pl.tables(a);
+  bool bad;
+  int E = fx_inverse<A, B, CW>(a, x, nl, pl, bad) + 1;  // V / 2
+  int sh;
+  // ---- z, inverse stage 2, x V / 2 ----
   {
     fx::Mag mag;
     const fx::Limbs* vp = a.fx.V + (size_t)x * N * N;
@@ -425,6 +468,7 @@ __device__ __forceinline__ void fx_pass_b(const LocalArgs<double>& a, int x, int
     mag.put(word + 7);
   }
   __syncthreads();
+  Cx* slab = reinterpret_cast<Cx*>(a.work) + ((size_t)nl * a.N1 + x) * W3 * W2;
   for (int i = tid; i < W3 * W2; i += NT) {
     const int u3 = dw2(i), u2 = i - u3 * W2;
     slab[i] = Q[u3 * QS + fftr::wrap_add(a.lo2, u2, N)];

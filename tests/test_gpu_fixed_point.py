@@ -93,3 +93,42 @@ def test_gamma_pairs_of_uneven_norm(ctx):
         assert err[4] < 1e-14 * big[4]
     finally:
         K.kss_sys_destroy(sysh)
+
+
+@pytest.mark.parametrize("box,a,ecut,kpt", [((24, 24, 24), 10.0, 10.0, 0), ((25, 25, 25), 8.0, 10.0, 1),
+                                            ((45, 48, 48), 10.0, 16.0, 0), ((96, 96, 96), 9.0, 9.0, 1)])
+def test_density_scales_and_special_bands(ctx, box, a, ecut, kpt):
+    """Bands at scales whose squares leave single weights and densities in range: w |psi|^2 of each
+    is of order one, so the sum is as accurate as in the oracle (1e-13 of its maximum: roundings of
+    2^-53 of |psi| in sums of at most 1e4 terms, twice that in the square)."""
+    import torch
+    s = W.make_system("fx", a, ecut, 3, 4, seed=17, kpts=[[0.25 * kpt] * 3], fft_box=box, nproj_per_atom=0)
+    sysh = setup(ctx, s)
+    try:
+        b = O.make_basis(s.lattice, s.ecut, s.kpts[0], box)
+        _, vol = O.reciprocal_lattice(s.lattice)
+        c = W.random_block(b.npw, 7, seed=5) / np.sqrt(b.npw)
+        c[3] = 0
+        c[4] = 0
+        c[4, b.npw // 3] = 1  # one plane wave: a constant density
+        c[5] = 1.0 / b.npw    # a peak at the origin
+        w = np.array([1.0, 0.7, 1.3, 2.0, 1.0, 0.5, -0.25])
+        scale = np.array([1, 1e-150, 1e150, 1, 1, 1, 1])
+
+        def rho_of(c, w):
+            rho = torch.zeros(tuple(reversed(box)), dtype=torch.float64, device="cuda")
+            K.kss_density_accumulate(sysh, 0, torch.from_numpy(c).cuda(), w, rho)
+            torch.cuda.synchronize()
+            return rho.cpu().numpy()
+
+        got = rho_of(c * scale[:, None], w / scale ** 2)
+        ref = O.density(c, b, w, vol)
+        assert np.max(np.abs(got - ref)) < 1e-13 * np.max(ref), np.max(np.abs(got - ref)) / np.max(ref)
+        assert np.all(rho_of(c[3:4], w[3:4]) == 0)
+        one = rho_of(c[4:5], w[4:5])
+        assert np.max(np.abs(one - 1.0 / vol)) < 1e-14 / vol
+        bad = c.copy()
+        bad[6, 0] = np.inf
+        assert np.all(np.isnan(rho_of(bad, w)))
+    finally:
+        K.kss_sys_destroy(sysh)
