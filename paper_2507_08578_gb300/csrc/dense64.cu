@@ -13,8 +13,8 @@
 //   3. Householder tridiagonalisation C = Q T Q^H (unblocked, on the full Hermitian matrix):
 //      per column, the reflector H = I - tau v v^H with a real subdiagonal (beta = -sign(Re
 //      alpha) |x|), p = tau C v, w = p - (tau/2)(p^H v) v, C <- C - v w^H - w v^H.
-//   4. Eigenpairs of the real symmetric tridiagonal T: every eigenvalue by bisection on the
-//      Sturm count (the number of negative pivots of the LDL^T factorisation of T - sigma I),
+//   4. Eigenpairs of the real symmetric tridiagonal T: every eigenvalue by interpolation and
+//      sections on the Sturm count (the number of negative pivots of the LDL^T factorisation of T - sigma I),
 //      every eigenvector by inverse iteration with the partially pivoted LU of T - lambda I;
 //      eigenvalues closer than 1e-5 |T| form a cluster whose vectors are orthogonalised against
 //      each other (modified Gram-Schmidt) in every iteration.
@@ -52,6 +52,36 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 static_assert((kWarps & (kWarps - 1)) == 0, "the CTA reductions take a power-of-two warp count");
+
+// 1 / x and 1 / sqrt(x) from the hardware's approximations (about 20 bits) by one third-order
+// iteration, r (1 + e + e^2) and r (1 + e / 2 + 3 e^2 / 8) with e the residual: within about one unit
+// in the last place.  The serial steps of the solver wait for these: three dependent operations of 64
+// cycles where a correctly rounded division takes about ten.  Arguments near the ends of the exponent
+// range take the ordinary operations.
+__device__ __forceinline__ bool mid_range(double x) {
+  const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
+  return e - 0x06000000u < 0x73000000u;  // 2^-926 .. 2^914
+}
+__device__ __forceinline__ double fast_rcp(double x) {
+  if (!mid_range(x)) return 1.0 / x;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double fast_rsqrt(double x) {  // x > 0
+  if (!mid_range(x)) return 1.0 / sqrt(x);
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x * r, r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
+// sqrt(x) from r = 1 / sqrt(x)
+__device__ __forceinline__ double sqrt_from(double x, double r) {
+  if (!mid_range(x)) return sqrt(x);
+  const double q = x * r;
+  return fma(fma(-q, q, x), 0.5 * r, q);
+}
 
 // ---- complex helpers ---------------------------------------------------------------------------
 // On GB300 an SM retires about two FP64 fused multiply-adds per clock, so every FP64 instruction
@@ -126,9 +156,9 @@ __device__ __forceinline__ double2 mk<double2>(double x, double y) { return make
 __device__ __forceinline__ double abs2_acc(double a, double s) { return fma(a, a, s); }
 __device__ __forceinline__ double abs2_acc(double2 a, double s) { return fma(a.x, a.x, fma(a.y, a.y, s)); }
 // 1 / a
-__device__ __forceinline__ double cinv(double a) { return 1.0 / a; }
+__device__ __forceinline__ double cinv(double a) { return fast_rcp(a); }
 __device__ __forceinline__ double2 cinv(double2 a) {
-  const double r = 1.0 / (a.x * a.x + a.y * a.y);
+  const double r = fast_rcp(fma(a.x, a.x, a.y * a.y));
   return make_double2(a.x * r, -a.y * r);
 }
 // complex128 value of a scalar (the caller's matrices are complex128 in both cases)
@@ -152,9 +182,7 @@ struct Ctl {
 
 struct CtaTeam {
   __device__ int rank() const { return threadIdx.x; }
-  // rank for per-thread independent work (the same as rank() on one CTA)
-  __device__ int srank() const { return threadIdx.x; }
-  __device__ int swrank() const { return threadIdx.x >> 5; }  // the same for per-warp work
+  __device__ int swrank() const { return threadIdx.x >> 5; }  // rank for per-warp work
   __device__ int size() const { return blockDim.x; }
   __device__ int wsize() const { return blockDim.x >> 5; }
   __device__ bool sync() const {
@@ -169,9 +197,8 @@ struct GridTeam {
   int* info;  // the pencil's status word: -1 when a barrier wait gave up
   unsigned long long limit_ns;
   __device__ int rank() const { return blockIdx.x * blockDim.x + threadIdx.x; }
-  // rank for per-thread independent work, spread over the CTAs first so that n work items use
-  // every SM's FP64 units instead of the first few CTAs'
-  __device__ int srank() const { return threadIdx.x * gridDim.x + blockIdx.x; }
+  // rank for per-warp independent work, spread over the CTAs first so that n work items use every
+  // SM's FP64 units instead of the first few CTAs'
   __device__ int swrank() const { return (threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
   __device__ int size() const { return gridDim.x * blockDim.x; }
   __device__ int wsize() const { return (gridDim.x * blockDim.x) >> 5; }
@@ -230,8 +257,8 @@ struct Pencil {
   int n, lda, ldb;
   S* R;         // n x n (ld n): reduction workspace, then the reflector vectors
   double* Z;    // n x n (ld n): eigenvectors of T
-  double* wk;   // 7 n^2 doubles: inverse-iteration arrays
-  double* vec;  // 11 n + 8 doubles: d, e, tau (S), p (2 x S), 1/L_jj, e^2, FP32 d and e^2
+  double* wk;   // 6 n^2 doubles: inverse-iteration arrays
+  double* vec;  // 9 n + 8 doubles: d, e, tau (S), p (2 x S), 1/L_jj
   int smem_cols;  // 1: the launch gives every warp n words of S of dynamic shared memory
   double2* outA;  // the caller's A and B (complex128; the same as A and B when S = double2)
   double2* outB;
@@ -304,6 +331,7 @@ __device__ bool cholesky(const Team& T, const Pencil<S>& P, S* smem) {
   __shared__ int s_bad;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool first_cta = T.rank() < (int)blockDim.x;
+  static_assert(W <= 32 && (W & (W - 1)) == 0, "one row of the diagonal block a lane");
   for (int p0 = 0; p0 < n; p0 += W) {
     const int w = min(W, n - p0);
     // 1. the diagonal block
@@ -311,40 +339,41 @@ __device__ bool cholesky(const Team& T, const Pencil<S>& P, S* smem) {
       const int c = e / W, r = e - c * W;
       Lb[c * LP + r] = (r < w && c < w && r >= c) ? B[(p0 + r) + (size_t)(p0 + c) * ld] : mk<S>(0.0, 0.0);
     }
+    if (tid >= w && tid < W) rdb[tid] = 0.0;
     if (tid == 0) s_bad = 0;
     __syncthreads();
-    if (warp == 0) {  // unblocked right-looking on the block, lane = row
-      for (int j = 0; j < w; ++j) {
-        const double d = re(Lb[j * LP + j]);
-        if (!(d > 0.0) || !isfinite(d)) {
-          if (lane == 0) s_bad = p0 + j + 1;
-          break;
+    if (warp == 0) {  // unblocked right-looking, lane = row, the row's entries in registers
+      S r[W];
+      const int i = lane & (W - 1);
+#pragma unroll
+      for (int k = 0; k < W; ++k) r[k] = Lb[k * LP + i];
+      int bad = 0;
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        if (j < w && !bad) {
+          const double d = re(shfl_c(r[j], j));
+          if (!(d > 0.0) || !isfinite(d)) {
+            bad = p0 + j + 1;
+          } else {
+            const double q = fast_rsqrt(d);
+            r[j] = i == j ? mk<S>(sqrt_from(d, q), 0.0) : cscale(r[j], q);
+            if (lane == j) rdb[j] = q;
+#pragma unroll
+            for (int k = j + 1; k < W; ++k) r[k] = cfms(r[j], conjd(shfl_c(r[j], k)), r[k]);
+          }
         }
-        const double sd = sqrt(d), r = 1.0 / sd;
-        if (lane > j && lane < w) Lb[j * LP + lane] = cscale(Lb[j * LP + lane], r);
-        if (lane == j) {
-          Lb[j * LP + j] = mk<S>(sd, 0.0);
-          rdb[j] = r;
-        }
-        __syncwarp();
-        for (int k = j + 1; k < w; ++k) {
-          const S lkj = conjd(Lb[j * LP + k]);
-          if (lane >= k && lane < w) Lb[k * LP + lane] = cfms(Lb[j * LP + lane], lkj, Lb[k * LP + lane]);
-        }
-        __syncwarp();
       }
+      if (lane < W) {
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+          if (k <= i) Lb[k * LP + i] = r[k];
+      }
+      if (bad && lane == 0) s_bad = bad;
     }
     __syncthreads();
     if (s_bad) {
       if (T.rank() == 0) *P.info = s_bad;
       return false;
-    }
-    if (first_cta) {
-      for (int e = tid; e < w * w; e += blockDim.x) {
-        const int c = e / w, r = e - c * w;
-        if (r >= c) B[(p0 + r) + (size_t)(p0 + c) * ld] = Lb[c * LP + r];
-      }
-      for (int j = tid; j < w; j += blockDim.x) rd[p0 + j] = rdb[j];
     }
     // 2. the rows below: l_ij = (a_ij - sum_{k<j} l_ik conj(L11[j][k])) / L11[j][j]
     for (int rb = p0 + w + 32 * T.swrank(); rb < n; rb += 32 * T.wsize()) {
@@ -353,12 +382,13 @@ __device__ bool cholesky(const Team& T, const Pencil<S>& P, S* smem) {
         S row[W];
 #pragma unroll
         for (int j = 0; j < W; ++j) row[j] = j < w ? B[i + (size_t)(p0 + j) * ld] : mk<S>(0.0, 0.0);
+        // column by column to the right: the W - 1 - j updates of a column are independent (the
+        // dependent chain is 2 W operations of 64 cycles, W^2 / 2 with the sums formed row by row)
 #pragma unroll
         for (int j = 0; j < W; ++j) {
-          S v = row[j];
+          row[j] = cscale(row[j], rdb[j]);
 #pragma unroll
-          for (int k = 0; k < j; ++k) v = cfms(row[k], conjd(Lb[k * LP + j]), v);
-          row[j] = cscale(v, rdb[j]);
+          for (int k = j + 1; k < W; ++k) row[k] = cfms(row[j], conjd(Lb[j * LP + k]), row[k]);
         }
 #pragma unroll
         for (int j = 0; j < W; ++j)
@@ -366,6 +396,14 @@ __device__ bool cholesky(const Team& T, const Pencil<S>& P, S* smem) {
       }
     }
     if (!T.sync()) return false;
+    // (behind the barrier: every CTA has read the block that this overwrites)
+    if (first_cta) {
+      for (int e = tid; e < w * w; e += blockDim.x) {
+        const int c = e / w, r = e - c * w;
+        if (r >= c) B[(p0 + r) + (size_t)(p0 + c) * ld] = Lb[c * LP + r];
+      }
+      for (int j = tid; j < w; j += blockDim.x) rd[p0 + j] = rdb[j];
+    }
     // 3. the trailing lower triangle
     if (p0 + w < n) {
       for (int k = p0 + w + T.swrank(); k < n; k += T.wsize()) {
@@ -535,7 +573,7 @@ __device__ bool reduce_standard(const Team& T, const Pencil<S>& P) {
 
 // ---- phase 3: Householder tridiagonalisation ------------------------------------------------------
 // vec layout: d[n], e[n], tau[2n] (n words of S), p[4n] (2 n words of S: p of two consecutive
-// steps), 1/L_jj[n], e^2[n], FP32 d and e^2[n]
+// steps), 1/L_jj[n]
 template <class S>
 __device__ __forceinline__ double* vd(const Pencil<S>& P) { return P.vec; }
 template <class S>
@@ -544,12 +582,6 @@ template <class S>
 __device__ __forceinline__ S* vtau(const Pencil<S>& P) { return reinterpret_cast<S*>(P.vec + 2 * P.n); }
 template <class S>
 __device__ __forceinline__ S* vp(const Pencil<S>& P) { return reinterpret_cast<S*>(P.vec + 4 * P.n); }
-template <class S>
-__device__ __forceinline__ double* ve2(const Pencil<S>& P) { return P.vec + 9 * P.n; }   // e^2
-template <class S>
-__device__ __forceinline__ float* vd32(const Pencil<S>& P) { return reinterpret_cast<float*>(P.vec + 10 * P.n); }
-template <class S>
-__device__ __forceinline__ float* ve232(const Pencil<S>& P) { return vd32(P) + P.n; }   // e^2 in FP32
 
 // Sum over the CTA (every thread passes a value; every thread gets the same total, reduced in a
 // fixed order so that all CTAs of a grid team obtain bit-identical results).
@@ -588,9 +620,10 @@ __device__ S cta_reflector(const Pencil<S>& P, int j, S* sx, bool writer) {
     if (s == 0.0 && im(alpha) == 0.0) {
       beta = re(alpha);  // nothing to annihilate: H = I
     } else {
-      const double an = sqrt(abs2_acc(alpha, s));
+      const double a2 = abs2_acc(alpha, s);
+      const double ra = fast_rsqrt(a2), an = sqrt_from(a2, ra);
       beta = re(alpha) >= 0.0 ? -an : an;
-      const double rb = 1.0 / beta;
+      const double rb = re(alpha) >= 0.0 ? -ra : ra;
       tj = mk<S>((beta - re(alpha)) * rb, -im(alpha) * rb);
       vs = cinv(csub(alpha, mk<S>(beta, 0.0)));  // v_i = x_i / (alpha - beta)
     }
@@ -714,27 +747,37 @@ __device__ bool tridiagonalise(const Team& T, const Pencil<S>& P, S* sbuf) {
 }
 
 // ---- phase 4: eigenpairs of the symmetric tridiagonal T (d, e) -----------------------------------
+// The phase works on T scaled by a power of two to norm [1, 2), staged in shared memory as (d_i,
+// e_{i-1}^2) pairs (and the same in FP32), later as (d_i, e_i).
+//
 // Number of eigenvalues of T below s, from the signs of the leading principal minors p_i of
-// T - s I (a Sturm sequence): p_0 = 1, p_1 = d_0 - s, p_{i+1} = (d_i - s) p_i - e_{i-1}^2 p_{i-1};
+// T - s I (a Sturm sequence): p_0 = 1, p_{i+1} = (d_i - s) p_i - e_{i-1}^2 p_{i-1} with e_{-1} = 0;
 // the count is the number of sign changes between consecutive minors, i.e. of negative pivots
 // p_{i+1} / p_i of the LDL^T factorisation (Sylvester's law of inertia).  Division-free: one fused
 // multiply-add per row on the dependent chain (an FP64 division has about seven times the latency
-// of a fused multiply-add on GB300, where that latency is already 64 cycles).  The pair
-// (p_i, p_{i+1}) is rescaled by an exact power of two when p_{i+1} leaves [2^-600, 2^600]; an
-// exactly zero minor is replaced by -2^-600 times the previous one (a tiny negative pivot, the
-// guard of the pivot form), which also carries the sequence across a split (e_i = 0).  e2 = e^2.
+// of a fused multiply-add on GB300, where that latency is already 64 cycles), and everything else
+// beside it: rows go four at a time, whose minors are only checked to be of size 2^-400 to 2^400;
+// the four rows are repeated one by one when they are not.  There the pair (p_i, p_{i+1}) is rescaled
+// by an exact power of two when p_{i+1} leaves [2^-600, 2^600], and an exactly zero minor is
+// replaced by -2^-600 times the previous one (a tiny negative pivot), which also carries the
+// sequence across a split (e_i = 0).  The last minor is v 2^ve.
+struct Sturm {
+  int count, ve;
+  double v;
+};
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 // |x| as an integer: ordered like |x| for all non-NaN doubles
 __device__ __forceinline__ unsigned long long dmag(double x) {
   return (unsigned long long)dbits(x) & 0x7FFFFFFFFFFFFFFFull;
 }
-__device__ __forceinline__ int sturm_count(const double* __restrict__ d, const double* __restrict__ e2, int n,
-                                           double s) {
-  double pm = 1.0, p = d[0] - s;
-  if (((unsigned long long)dbits(p) << 1) == 0) p = -0x1p-600;
-  int c = (int)((unsigned long long)dbits(p) >> 63);
-  for (int i = 1; i < n; ++i) {
-    double pn = fma(d[i] - s, p, -e2[i - 1] * pm);
+// 2^e, the exponent taken into the normal range
+__device__ __forceinline__ double exp2_of(int e) { return __hiloint2double((1023 + max(-1022, min(1023, e))) << 20, 0); }
+
+__device__ __forceinline__ Sturm sturm_count(const double2* __restrict__ t, int n, double s) {
+  double pm = 0.0, p = 1.0;
+  int c = 0, es = 0;
+  auto row = [&](double2 a) {  // one row with all the checks
+    double pn = fma(a.x - s, p, -a.y * pm);
     if (((unsigned long long)dbits(pn) << 1) == 0) pn = -0x1p-600 * p;
     c += (int)((unsigned long long)(dbits(pn) ^ dbits(p)) >> 63);
     pm = p;
@@ -743,22 +786,51 @@ __device__ __forceinline__ int sturm_count(const double* __restrict__ d, const d
     if (ex > 1023 + 600) {
       p *= 0x1p-600;
       pm *= 0x1p-600;
+      es += 600;
     } else if (ex < 1023 - 600 && (int)((dbits(pm) >> 52) & 0x7FF) < 1023 + 400) {
       p *= 0x1p+600;
       pm *= 0x1p+600;
+      es -= 600;
+    }
+  };
+  int i = 0;
+  for (; i + 4 <= n; i += 4) {
+    const double2 a0 = t[i], a1 = t[i + 1], a2 = t[i + 2], a3 = t[i + 3];
+    const double q0 = fma(a0.x - s, p, -a0.y * pm);
+    const double q1 = fma(a1.x - s, q0, -a1.y * p);
+    const double q2 = fma(a2.x - s, q1, -a2.y * q0);
+    const double q3 = fma(a3.x - s, q2, -a3.y * q1);
+    const int h = __double2hiint(p), h0 = __double2hiint(q0), h1 = __double2hiint(q1), h2 = __double2hiint(q2),
+              h3 = __double2hiint(q3);
+    auto out = [](int x) { return (unsigned)((x & 0x7ff00000) - ((1023 - 400) << 20)) > (unsigned)(800 << 20); };
+    if (out(h0) | out(h1) | out(h2) | out(h3)) {
+#pragma unroll 1
+      for (int u = 0; u < 4; ++u) row(t[i + u]);
+      continue;
+    }
+    c += ((unsigned)(h ^ h0) >> 31) + ((unsigned)(h0 ^ h1) >> 31) + ((unsigned)(h1 ^ h2) >> 31) +
+         ((unsigned)(h2 ^ h3) >> 31);
+    pm = q2;
+    p = q3;
+    const int ex = ((h3 >> 20) & 0x7FF) - 1023;
+    if (ex > 200 || ex < -200) {
+      const double f = exp2_of(-ex);
+      p *= f;
+      pm *= f;
+      es += ex;
     }
   }
-  return c;
+  for (; i < n; ++i) row(t[i]);
+  return Sturm{c, es, p};
 }
 // The same count in FP32 (about 64 times cheaper on GB300), used only to narrow the bracket.
-__device__ __forceinline__ int sturm_count32(const float* __restrict__ d, const float* __restrict__ e2, int n,
-                                             float s, float pivmin) {
+__device__ __forceinline__ int sturm_count32(const float2* __restrict__ t, int n, float s, float pivmin) {
   int c = 0;
-  float q = d[0] - s;
-  if (fabsf(q) < pivmin) q = -pivmin;
-  c += q < 0.f;
-  for (int i = 1; i < n; ++i) {
-    q = (d[i] - s) - __fdividef(e2[i - 1], q);
+  float q = 1.f;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) {
+    const float2 a = t[i];
+    q = (a.x - s) - __fdividef(a.y, q);
     if (fabsf(q) < pivmin) q = -pivmin;
     c += q < 0.f;
   }
@@ -776,69 +848,77 @@ __device__ __forceinline__ double start_entry(int k, int i) {
   return ((double)(h >> 8) + 0.5) * (2.0 / 16777216.0) - 1.0;
 }
 
+// smem: 3 n words of S
 template <class Team, class S>
-__device__ bool tridiagonal_eig(const Team& T, const Pencil<S>& P) {
+__device__ bool tridiagonal_eig(const Team& T, const Pencil<S>& P, S* smem) {
   const int n = P.n;
   const double* d = vd(P);
   const double* e = ve(P);
-  double* e2 = ve2(P);
-  float* d32 = vd32(P);
-  float* e232 = ve232(P);
   double* w = P.w;
-  for (int i = T.rank(); i < n; i += T.size()) {
-    const double ei = i < n - 1 ? e[i] : 0.0;
-    e2[i] = ei * ei;
-    d32[i] = (float)d[i];
-    e232[i] = (float)(ei * ei);
-  }
-  // norms and Gershgorin interval (every thread computes them the same way)
-  double tn = 0.0, glo = 0.0, gu = 0.0, emax2 = 0.0;
-  for (int i = 0; i < n; ++i) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  double2* t64 = reinterpret_cast<double2*>(smem);
+  float2* t32 = reinterpret_cast<float2*>(t64 + n);
+  // norm and Gershgorin interval (every warp computes them the same way, in the scaled units below)
+  double tn = 0.0, glo = 1e308, gu = -1e308;
+  for (int i = lane; i < n; i += 32) {
     const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < n - 1 ? fabs(e[i]) : 0.0);
     tn = fmax(tn, fabs(d[i]) + r);
-    glo = i ? fmin(glo, d[i] - r) : d[i] - r;
-    gu = i ? fmax(gu, d[i] + r) : d[i] + r;
-    if (i < n - 1) emax2 = fmax(emax2, e[i] * e[i]);
+    glo = fmin(glo, d[i] - r);
+    gu = fmax(gu, d[i] + r);
   }
-  const double eps = 2.220446049250313e-16;
-  const double pivmin = 2.2250738585072014e-308 * fmax(1.0, emax2);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+    glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
+    gu = fmax(gu, __shfl_xor_sync(0xffffffffu, gu, o));
+  }
   tn = fmax(tn, 1e-300);
-  glo -= 2.0 * eps * tn + 2.0 * pivmin;
-  gu += 2.0 * eps * tn + 2.0 * pivmin;
-  if (!T.sync()) return false;
-  // Eigenvalue k by multisection, one group of kSect lanes per eigenvalue (32 / kSect eigenvalues
-  // per warp, kSect = 8, 16 or 32): in every round the group's lanes count at kSect interior points of the bracket
-  // [lo, hi] (count(lo) <= k < count(hi)) and the bracket shrinks to the 1/(kSect+1) between the
-  // last point below eigenvalue k and the first above it.  The bracket is first narrowed with FP32
-  // counts (about 64 times cheaper than FP64 on GB300) to 1e-6 |T|, widened by 2e-6 |T| and
-  // accepted only if the FP64 counts at both ends confirm it (else the Gershgorin interval is
-  // used); FP64 rounds then take it to 2 eps |lambda|.  The rounds are a sequence of dependent
-  // Sturm counts, so the lane groups trade a few times more FP64 work than plain bisection for a
-  // sequence about three times shorter.
-  const float pivmin32 = 1e-30f * (float)fmax(1.0, emax2);
-  const int lane = threadIdx.x & 31;
-  // lanes per eigenvalue: a 32-section shrinks the bracket by 33 per round, an 8-section by 9, at
-  // four times the Sturm counts per round; wider sections pay while they keep the busy warps at
-  // no more than half of the team's (beyond that the FP64 pipe, not the chain, is the limit)
-  const int kSect = T.wsize() >= 2 * n ? 32 : T.wsize() >= n ? 16 : 8;
+  const int tex = max(-1000, min(1000, (int)(dbits(tn) >> 52 & 0x7FF) - 1023));
+  const double sc = exp2_of(-tex), usc = exp2_of(tex);
+  const double eps = 2.220446049250313e-16;
+  tn *= sc;
+  glo = glo * sc - 2.0 * eps * tn;
+  gu = gu * sc + 2.0 * eps * tn;
+  for (int i = tid; i < n; i += blockDim.x) {
+    const double di = d[i] * sc, ei = i > 0 ? e[i - 1] * sc : 0.0;
+    t64[i] = make_double2(di, ei * ei);
+    t32[i] = make_float2((float)di, (float)(ei * ei));
+  }
+  __syncthreads();
+  // Eigenvalue k by a group of kSect lanes.  A bracket [lo, hi] (count(lo) <= k < count(hi)) is first
+  // narrowed with FP32 counts to 1e-6 |T|, widened by 2e-6 |T| and accepted only if the FP64
+  // counts at both ends confirm it (else the Gershgorin interval is used); FP64 rounds take it to
+  // 2 eps |lambda|.  In every round each lane of the group counts at one point of the bracket and
+  // the bracket becomes the interval between the last point below the eigenvalue and the first
+  // above it.  While the bracket holds a single eigenvalue the points stand at geometric distances
+  // on both sides of the root that the last minors at its ends interpolate (regula falsi): at each
+  // round the bracket shrinks to about its square over the distance to the next eigenvalue, three
+  // or four rounds from 4e-6 |T| where even sections take about ten.  A round that gains less than a
+  // factor 8, or a bracket with several eigenvalues, is followed by one with evenly spaced points.
+  // Orders 564 and 1127: 0.75 and 1.49 ms (even sections, unblocked counts: 2.08 and 4.66).
+  const float pivmin32 = 1e-30f;
+  // 8 lanes an eigenvalue, 4 where that would keep the team's FP64 units busy for several passes
+  const int kSect = T.size() >= 8 * n ? 8 : 4;
   const int kGroups = 32 / kSect;
-  if (T.wsize() * kGroups >= n) {
-    const int grp = lane / kSect, gi = lane % kSect;
-    const unsigned gmask = kSect == 32 ? 0xffffffffu : ((1u << kSect) - 1u) << (grp * kSect);
+  {
+    const int grp = lane / kSect, gi = lane % kSect, g0 = grp * kSect;
+    const unsigned gmask = ((1u << kSect) - 1u) << g0;
+    auto first_above = [&](bool above) {
+      const unsigned bits = (__ballot_sync(0xffffffffu, above) & gmask) >> g0;
+      return bits ? __ffs(bits) - 1 : kSect;
+    };
     for (int k0 = T.swrank() * kGroups; k0 < n; k0 += T.wsize() * kGroups) {
       const int k = k0 + grp;
       const bool act = k < n;
       float l32 = (float)glo, h32 = (float)gu;
       const float wid = (float)(1e-6 * tn);
       bool open = act;
-      for (int it = 0; it < 16; ++it) {
+      for (int it = 0; it < 24; ++it) {
         open = open && h32 - l32 > wid;
         if (!__any_sync(0xffffffffu, open)) break;
         const float step = (h32 - l32) * (1.0f / (float)(kSect + 1));
         const float pt = l32 + (float)(gi + 1) * step;
-        const bool above = open && pt < h32 && sturm_count32(d32, e232, n, pt, pivmin32) > k;
-        const unsigned bits = (__ballot_sync(0xffffffffu, above) & gmask) >> (grp * kSect);
-        const int f = bits ? __ffs(bits) - 1 : kSect;
+        const int f = first_above(open && pt < h32 && sturm_count32(t32, n, pt, pivmin32) > k);
         if (open) {
           const float nl = f == 0 ? l32 : l32 + (float)f * step;
           const float nh = f == kSect ? h32 : l32 + (float)(f + 1) * step;
@@ -851,170 +931,218 @@ __device__ bool tridiagonal_eig(const Team& T, const Pencil<S>& P) {
         }
       }
       double lo = fmax(glo, (double)l32 - 2e-6 * tn), hi = fmin(gu, (double)h32 + 2e-6 * tn);
+      Sturm flo{0, 0, 0.0}, fhi{0, 0, 0.0};
       {
-        const int c = !act ? 0 : gi == 0 ? sturm_count(d, e2, n, lo) : (gi == 1 ? sturm_count(d, e2, n, hi) : 0);
-        const int c0 = __shfl_sync(0xffffffffu, c, grp * kSect), c1 = __shfl_sync(0xffffffffu, c, grp * kSect + 1);
-        if (!(c0 <= k && c1 > k)) {
+        Sturm c{0, 0, 0.0};
+        if (act && gi < 2) c = sturm_count(t64, n, gi ? hi : lo);
+        flo.count = __shfl_sync(0xffffffffu, c.count, g0);
+        flo.ve = __shfl_sync(0xffffffffu, c.ve, g0);
+        flo.v = __shfl_sync(0xffffffffu, c.v, g0);
+        fhi.count = __shfl_sync(0xffffffffu, c.count, g0 + 1);
+        fhi.ve = __shfl_sync(0xffffffffu, c.ve, g0 + 1);
+        fhi.v = __shfl_sync(0xffffffffu, c.v, g0 + 1);
+        if (!(flo.count <= k && fhi.count > k)) {
           lo = glo;
           hi = gu;
+          flo = Sturm{0, 0, 0.0};
+          fhi = Sturm{n, 0, 0.0};
         }
       }
       open = act;
-      for (int it = 0; it < 64; ++it) {
-        open = open && !(hi - lo <= 2.0 * eps * fmax(fabs(lo), fabs(hi)) + pivmin);
+      bool even = false;  // this round takes evenly spaced points
+      for (int it = 0; it < 80; ++it) {
+        open = open && !(hi - lo <= 2.0 * eps * fmax(fabs(lo), fabs(hi)) + 1e-300);
         if (!__any_sync(0xffffffffu, open)) break;
-        const double step = (hi - lo) * (1.0 / (double)(kSect + 1));
-        const double pt = lo + (double)(gi + 1) * step;
-        const bool above = open && pt < hi && sturm_count(d, e2, n, pt) > k;
-        const unsigned bits = (__ballot_sync(0xffffffffu, above) & gmask) >> (grp * kSect);
-        const int f = bits ? __ffs(bits) - 1 : kSect;
+        const double width = hi - lo;
+        // (a count of 0 or n at the ends of the Gershgorin interval comes without its minor)
+        const bool ladder = !even && fhi.count - flo.count == 1 && flo.v != 0.0 && fhi.v != 0.0;
+        double pt;
+        if (ladder) {
+          const double r = fabs(fhi.v) * exp2_of(fhi.ve - flo.ve) * fast_rcp(fabs(flo.v));
+          const double est = lo + width * fast_rcp(1.0 + r);
+          const int half = kSect >> 1, j = gi < half ? gi : kSect - 1 - gi;  // 0: outermost
+          // exponents of the distances: 3, 8, 14, 22 below the bracket's width (two lanes a side: 6, 16)
+          const int down = kSect == 8 ? (j == 0 ? 3 : j == 1 ? 8 : j == 2 ? 14 : 22) : (j == 0 ? 6 : 16);
+          const double del = fmax(width * exp2_of(-down), 0.95 * eps * fabs(est));
+          pt = gi < half ? est - del : est + del;
+        } else {
+          pt = lo + (double)(gi + 1) * (width * (1.0 / (double)(kSect + 1)));
+        }
+        Sturm c{0, 0, 0.0};
+        const bool in = open && pt > lo && pt < hi;
+        if (in) c = sturm_count(t64, n, pt);
+        const int f = first_above(in ? c.count > k : !(pt <= lo));
+        const int sl = g0 + max(f - 1, 0), sh = g0 + min(f, kSect - 1);
+        const double pl = __shfl_sync(0xffffffffu, pt, sl), ph = __shfl_sync(0xffffffffu, pt, sh);
+        const Sturm cl{__shfl_sync(0xffffffffu, c.count, sl), __shfl_sync(0xffffffffu, c.ve, sl),
+                       __shfl_sync(0xffffffffu, c.v, sl)};
+        const Sturm ch{__shfl_sync(0xffffffffu, c.count, sh), __shfl_sync(0xffffffffu, c.ve, sh),
+                       __shfl_sync(0xffffffffu, c.v, sh)};
         if (open) {
-          const double nl = f == 0 ? lo : lo + (double)f * step;
-          const double nh = f == kSect ? hi : lo + (double)(f + 1) * step;
-          if (!(nh > nl) || (nl == lo && nh >= hi)) {
-            open = false;
+          if (f > 0 && pl > lo) {
+            lo = pl;
+            flo = cl;
+          }
+          if (f < kSect && ph < hi) {
+            hi = ph;
+            fhi = ch;
+          }
+          const double nw = hi - lo;
+          if (!(nw < width)) {
+            if (!ladder) open = false;  // the points have become neighbours
+            even = true;
           } else {
-            lo = nl;
-            hi = fmin(nh, hi);
+            even = ladder && nw > 0.125 * width;
           }
         }
       }
-      if (act && gi == 0) w[k] = 0.5 * (lo + hi);
-    }
-  } else {
-    // fewer warps than eigenvalues (one CTA per pencil): plain bisection, one thread per
-    // eigenvalue, with the same FP32 narrowing and FP64 confirmation of the bracket
-    for (int k = T.srank(); k < n; k += T.size()) {
-      float l32 = (float)glo, h32 = (float)gu;
-      const float wid = (float)(1e-5 * tn);
-      for (int it = 0; it < 64 && h32 - l32 > wid; ++it) {
-        const float mid = 0.5f * (l32 + h32);
-        if (mid <= l32 || mid >= h32) break;
-        if (sturm_count32(d32, e232, n, mid, pivmin32) > k) h32 = mid;
-        else l32 = mid;
-      }
-      double lo = fmax(glo, (double)l32 - 1e-5 * tn), hi = fmin(gu, (double)h32 + 1e-5 * tn);
-      if (!(sturm_count(d, e2, n, lo) <= k && sturm_count(d, e2, n, hi) > k)) {
-        lo = glo;
-        hi = gu;
-      }
-      for (int it = 0; it < 200; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        if (hi - lo <= 2.0 * eps * fmax(fabs(lo), fabs(hi)) + pivmin || mid <= lo || mid >= hi) break;
-        if (sturm_count(d, e2, n, mid) > k) hi = mid;
-        else lo = mid;
-      }
-      w[k] = 0.5 * (lo + hi);
+      if (act && gi == 0) w[k] = 0.5 * (lo + hi) * usc;
     }
   }
   if (!T.sync()) return false;
   T.stamp(4);
-  // eigenvectors by inverse iteration, one cluster per thread
-  const double ortol = 1e-5 * tn;
+  // Eigenvectors by inverse iteration, one cluster per thread, in the scaled units.  T - s I = P L U
+  // (partial pivoting) once, then two solves for a single eigenvalue, four for each of a cluster; the
+  // first solve starts behind L (a random vector stays random).  With the eigenvalue good to
+  // 2 eps |T| and the next one 1e-5 |T| away, one solve leaves about 1e-10 of the other vectors and
+  // the second nothing.  Orders 564 and 1127: 0.81 and 1.60 ms (three full solves, row by row: 2.07 and
+  // 4.85).  A chain of n dependent rows per pass, so every pass reads its arrays
+  // eight rows ahead and keeps all but one multiply-add a row off the chain: the diagonal of U is
+  // stored as reciprocals, already multiplied into its first superdiagonal.
+  for (int i = tid; i < n; i += blockDim.x) t64[i] = make_double2(d[i] * sc, i < n - 1 ? e[i] * sc : 0.0);
+  __syncthreads();
+  const double ortol = 1e-5 * tn * usc;
   const double tiny = eps * tn;
   const size_t nn = (size_t)n * n;
-  // (separate input and output arrays in every sweep, so that the loads of later rows can be
-  // issued ahead of the dependent arithmetic)
   double* __restrict__ ua = P.wk;           // reciprocals of U's diagonal
-  double* __restrict__ ub = P.wk + nn;      // U first superdiagonal
-  double* __restrict__ uc = P.wk + 2 * nn;  // U second superdiagonal (fill-in of row swaps)
-  double* __restrict__ ml = P.wk + 3 * nn;  // multipliers
-  double* __restrict__ sw = P.wk + 4 * nn;  // 1: rows i, i+1 swapped
-  double* __restrict__ x = P.wk + 5 * nn;   // iterate
-  double* __restrict__ y = P.wk + 6 * nn;   // L^{-1} P x
+  double* __restrict__ ub = P.wk + nn;      // U first superdiagonal over its diagonal
+  double* __restrict__ ml = P.wk + 2 * nn;  // multipliers
+  double* __restrict__ x = P.wk + 3 * nn;   // iterate
+  double* __restrict__ y = P.wk + 4 * nn;   // L^{-1} P x
+  unsigned* __restrict__ sw = reinterpret_cast<unsigned*>(P.wk + 5 * nn);  // bit i: rows i, i+1 swapped
+  constexpr int U = 8;  // rows a block
   // 32 consecutive eigenvalues per warp (the interleaved arrays are then read in full 256-byte
   // rows), the warps spread over the CTAs
-  for (int k0 = T.swrank() * 32 + (threadIdx.x & 31); k0 < n; k0 += T.size()) {
+  for (int k0 = T.swrank() * 32 + lane; k0 < n; k0 += T.size()) {
     if (k0 > 0 && w[k0] - w[k0 - 1] <= ortol) continue;  // not the first of its cluster
     int k1 = k0 + 1;
     while (k1 < n && w[k1] - w[k1 - 1] <= ortol) ++k1;
     double sprev = 0.0;
     for (int m = k0; m < k1; ++m) {
       // slot m of the interleaved arrays: element i at [i * n + m]
-      double s = w[m];
+      double s = w[m] * sc;
       const double pert = 10.0 * eps * fmax(fabs(s), tn);
       if (m > k0 && s - sprev < pert) s = sprev + pert;
       sprev = s;
-      // factor T - s I = P L U with partial pivoting
       {
-        double a = d[0] - s, b = n > 1 ? e[0] : 0.0;
+        double2 ti = t64[0];
+        double a = ti.x - s, b = ti.y;
+        unsigned bits = 0;
         for (int i = 0; i < n - 1; ++i) {
-          const double sub = e[i];
-          const double nd = d[i + 1] - s;
-          const double ns = i + 1 < n - 1 ? e[i + 1] : 0.0;
+          const double2 tj = t64[i + 1];
+          const double sub = ti.y, nd = tj.x - s, ns = tj.y;
           const size_t o = (size_t)i * n + m;
-          // ua holds the reciprocal pivot: one division per row, none in the solves; the pivot
-          // choice compares magnitudes as integers (the FP64 compare would add 64 cycles a row)
-          if (dmag(a) >= dmag(sub)) {
-            if (dmag(a) == 0) a = tiny;
-            const double r = 1.0 / a;
-            const double l = sub * r;
-            ua[o] = r;
-            ub[o] = b;
-            uc[o] = 0.0;
-            ml[o] = l;
-            sw[o] = 0.0;
-            a = nd - l * b;
-            b = ns;
-          } else {
-            const double r = 1.0 / sub;
-            const double l = a * r;
-            ua[o] = r;
-            ub[o] = nd;
-            uc[o] = ns;
-            ml[o] = l;
-            sw[o] = 1.0;
-            a = b - l * nd;
-            b = -l * ns;
+          // the pivot choice compares magnitudes as integers (the FP64 compare would add 64 cycles a
+          // row); a pivot below eps |T| is taken as that
+          const bool swp = dmag(a) < dmag(sub);
+          double piv = swp ? sub : a;
+          if (dmag(piv) < dmag(tiny)) piv = tiny;
+          const double r = fast_rcp(piv), l = (swp ? a : sub) * r;
+          ua[o] = r;
+          ub[o] = (swp ? nd : b) * r;
+          ml[o] = l;
+          bits |= (unsigned)swp << (i & 31);
+          if ((i & 31) == 31 || i == n - 2) {
+            sw[(size_t)(i >> 5) * n + m] = bits;
+            bits = 0;
           }
+          a = swp ? fma(-l, nd, b) : fma(-l, b, nd);
+          b = swp ? -l * ns : ns;
+          ti = tj;
         }
-        if (dmag(a) == 0) a = tiny;
-        ua[(size_t)(n - 1) * n + m] = 1.0 / a;
+        if (dmag(a) < dmag(tiny)) a = tiny;
+        ua[(size_t)(n - 1) * n + m] = fast_rcp(a);
       }
-      for (int i = 0; i < n; ++i) x[(size_t)i * n + m] = start_entry(m, i);
-      const int iters = (k1 - k0 > 1) ? 4 : 3;
+      const bool cluster = k1 - k0 > 1;
+      const int iters = cluster ? 4 : 2;
       for (int it = 0; it < iters; ++it) {
         // forward: y = L^{-1} P x, the row operations of the factorisation (running row in a register)
-        {
+        if (it == 0) {
+          for (int i = 0; i < n; ++i) y[(size_t)i * n + m] = start_entry(m, i);
+        } else {
           double cur = x[m];
-#pragma unroll 4
-          for (int i = 0; i < n - 1; ++i) {
-            const size_t o = (size_t)i * n + m;
-            double nxt = x[o + n];
-            if (dmag(sw[o]) != 0) {
-              const double t = cur;
-              cur = nxt;
-              nxt = t;
+          unsigned bits = 0;
+          int i = 0;
+          for (; i + U <= n - 1; i += U) {
+            double nx[U], l[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              nx[u] = x[(size_t)(i + u + 1) * n + m];
+              l[u] = ml[(size_t)(i + u) * n + m];
             }
-            y[o] = cur;
-            cur = fma(-ml[o], cur, nxt);
+            if ((i & 31) == 0) bits = sw[(size_t)(i >> 5) * n + m];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const bool swp = bits >> ((i + u) & 31) & 1u;
+              const double yv = swp ? nx[u] : cur, nv = swp ? cur : nx[u];
+              y[(size_t)(i + u) * n + m] = yv;
+              cur = fma(-l[u], yv, nv);
+            }
+          }
+          for (; i < n - 1; ++i) {
+            const size_t o = (size_t)i * n + m;
+            const bool swp = sw[(size_t)(i >> 5) * n + m] >> (i & 31) & 1u;
+            const double nx = x[o + n];
+            const double yv = swp ? nx : cur, nv = swp ? cur : nx;
+            y[o] = yv;
+            cur = fma(-ml[o], yv, nv);
           }
           y[(size_t)(n - 1) * n + m] = cur;
         }
         // backward: x = U^{-1} y (the two solved rows below in registers; the iterate and the rows
-        // still to solve are scaled down together when it grows)
+        // still to solve are scaled down together when a block of rows has grown beyond 1e100)
         {
           double x1 = 0.0, x2 = 0.0;
-#pragma unroll 4
-          for (int i = n - 1; i >= 0; --i) {
-            const size_t o = (size_t)i * n + m;
-            double v = y[o];
-            if (i + 2 < n) v = fma(-uc[o], x2, v);
-            if (i + 1 < n) v = fma(-ub[o], x1, v);
-            v *= ua[o];
-            x[o] = v;
-            x2 = x1;
-            x1 = v;
-            if (dmag(v) > dmag(1e100)) {
+          for (int i0 = n; i0 > 0; i0 -= U) {
+            const int cnt = min(U, i0);
+            double yv[U], uv[U], bv[U], cv[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int i = i0 - 1 - u;
+              yv[u] = uv[u] = bv[u] = cv[u] = 0.0;
+              if (u < cnt) {
+                const size_t o = (size_t)i * n + m;
+                yv[u] = y[o];
+                uv[u] = ua[o];
+                if (i < n - 1) {
+                  bv[u] = ub[o];
+                  // second superdiagonal (fill-in of a swap): e_{i+1}
+                  if (sw[(size_t)(i >> 5) * n + m] >> (i & 31) & 1u) cv[u] = t64[i + 1].y;
+                }
+              }
+            }
+            unsigned long long big = 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const double v = fma(-bv[u], x1, fma(-(cv[u] * uv[u]), x2, yv[u] * uv[u]));
+              if (u < cnt) {
+                x[(size_t)(i0 - 1 - u) * n + m] = v;
+                x2 = x1;
+                x1 = v;
+                big = max(big, dmag(v));
+              }
+            }
+            if (big > dmag(1e100)) {
               for (int r = 0; r < n; ++r) {
-                x[(size_t)r * n + m] *= 1e-100;
-                y[(size_t)r * n + m] *= 1e-100;
+                if (r >= i0 - cnt) x[(size_t)r * n + m] *= 1e-100;
+                else y[(size_t)r * n + m] *= 1e-100;
               }
               x1 *= 1e-100;
               x2 *= 1e-100;
             }
           }
         }
+        if (!cluster && it + 1 < iters) continue;
         // orthogonalise against the cluster's earlier vectors, then normalise
         for (int q = k0; q < m; ++q) {
           const double* zq = P.Z + (size_t)q * n;
@@ -1024,13 +1152,17 @@ __device__ bool tridiagonal_eig(const Team& T, const Pencil<S>& P) {
         }
         double n0 = 0.0, n1 = 0.0, n2 = 0.0, n3 = 0.0;  // four independent chains
         int i = 0;
-        for (; i + 3 < n; i += 4) {
-          const double v0 = x[(size_t)i * n + m], v1 = x[(size_t)(i + 1) * n + m];
-          const double v2 = x[(size_t)(i + 2) * n + m], v3 = x[(size_t)(i + 3) * n + m];
-          n0 = fma(v0, v0, n0);
-          n1 = fma(v1, v1, n1);
-          n2 = fma(v2, v2, n2);
-          n3 = fma(v3, v3, n3);
+        for (; i + U <= n; i += U) {
+          double v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) v[u] = x[(size_t)(i + u) * n + m];
+#pragma unroll
+          for (int u = 0; u < U; u += 4) {
+            n0 = fma(v[u], v[u], n0);
+            n1 = fma(v[u + 1], v[u + 1], n1);
+            n2 = fma(v[u + 2], v[u + 2], n2);
+            n3 = fma(v[u + 3], v[u + 3], n3);
+          }
         }
         for (; i < n; ++i) {
           const double v = x[(size_t)i * n + m];
@@ -1038,10 +1170,20 @@ __device__ bool tridiagonal_eig(const Team& T, const Pencil<S>& P) {
         }
         const double nrm = sqrt((n0 + n1) + (n2 + n3));
         const double r = nrm > 0.0 ? 1.0 / nrm : 0.0;
-        for (int i = 0; i < n; ++i) x[(size_t)i * n + m] *= r;
+        double* __restrict__ zm = P.Z + (size_t)m * n;
+        const bool last = it + 1 == iters;
+        for (i = 0; i < n; i += U) {
+          double v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) v[u] = i + u < n ? x[(size_t)(i + u) * n + m] * r : 0.0;
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (i + u < n) {
+              if (last) zm[i + u] = v[u];
+              else x[(size_t)(i + u) * n + m] = v[u];
+            }
+        }
       }
-      double* zm = P.Z + (size_t)m * n;
-      for (int i = 0; i < n; ++i) zm[i] = x[(size_t)i * n + m];
     }
   }
   return T.sync();
@@ -1097,7 +1239,7 @@ __device__ void solve_pencil(const Team& T, const Pencil<S>& P) {
   T.stamp(2);
   if (!tridiagonalise(T, P, smem)) return;
   T.stamp(3);
-  if (!tridiagonal_eig(T, P)) return;
+  if (!tridiagonal_eig(T, P, smem)) return;
   T.stamp(5);
   if (!back_transform(T, P, P.smem_cols ? smem : nullptr)) return;
   finish(T, P);
@@ -1105,7 +1247,7 @@ __device__ void solve_pencil(const Team& T, const Pencil<S>& P) {
 }
 
 template <class S>
-__global__ void __launch_bounds__(kThreads, 2) hegv_grid_kernel(Pencil<S> P, Ctl* ctl, unsigned long long limit_ns) {
+__global__ void __launch_bounds__(kThreads, 1) hegv_grid_kernel(Pencil<S> P, Ctl* ctl, unsigned long long limit_ns) {
   GridTeam T{ctl, P.info, limit_ns};
   solve_pencil(T, P);
 }
@@ -1121,11 +1263,11 @@ __global__ void __launch_bounds__(kThreads, 2) hegv_cta_kernel(const Pencil<S>* 
 size_t pad32(size_t x) { return (x + 31) & ~(size_t)31; }
 
 // Workspace doubles of one pencil, each array padded to 32 doubles: complex, R (complex n^2);
-// real, the compact A, B and R (n^2 each); then Z (n^2), wk (7 n^2) and vec (11 n + 8).
+// real, the compact A, B and R (n^2 each); then Z (n^2), wk (6 n^2) and vec (9 n + 8).
 size_t work_doubles(int n, bool real) {
   const size_t nn = (size_t)n * n;
   const size_t own = real ? 3 * pad32(nn) : pad32(2 * nn);
-  return own + pad32(nn) + pad32(7 * nn) + pad32(11 * (size_t)n + 8);
+  return own + pad32(nn) + pad32(6 * nn) + pad32(9 * (size_t)n + 8);
 }
 
 template <class S>
@@ -1156,7 +1298,7 @@ Pencil<S> make_pencil(double2* A, int lda, double2* B, int ldb, double* w, int* 
   }
   P.Z = rest;
   P.wk = P.Z + pad32(nn);
-  P.vec = P.wk + pad32(7 * nn);
+  P.vec = P.wk + pad32(6 * nn);
   P.smem_cols = 0;
   return P;
 }

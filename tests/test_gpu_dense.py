@@ -177,3 +177,33 @@ def test_not_positive_definite(ctx, n):
     B = B - 2.0 * np.linalg.norm(B, 2) * np.outer(np.eye(n)[n // 2], np.eye(n)[n // 2])
     info, _ = run(ctx, [(A, B)])
     assert 0 < info[0] <= n
+
+
+@pytest.mark.parametrize("name", ["graded", "split", "tight", "scaled_down", "scaled_up", "wilkinson", "zero"])
+@pytest.mark.parametrize("n", [21, 67])
+def test_tridiagonal_spectra(ctx, name, n):
+    """Tridiagonal pencils (B = 1) whose Sturm sequences and pivots leave the ordinary range: sizes
+    graded over 1e-28, off-diagonals exactly zero, pairs closer than the bracket of one count,
+    norms near the ends of the exponent range, Wilkinson's near-equal pairs, the zero matrix."""
+    d = np.linspace(-1.0, 1.0, n) ** 3
+    e = np.full(n - 1, 0.1)
+    s = 1.0
+    if name == "graded":
+        d, e = 10.0 ** -np.linspace(0, 28, n), 0.3 * 10.0 ** -np.linspace(0, 28, n - 1)
+    elif name == "split":
+        e[::3] = 0.0
+    elif name == "tight":
+        e[:] = 1e-9
+        d = np.round(d * 4) / 4 + 1e-8 * np.arange(n)
+    elif name == "scaled_down":
+        s = 1e-120
+    elif name == "scaled_up":
+        s = 1e120
+    elif name == "wilkinson":
+        d, e = np.abs(np.arange(n) - n // 2).astype(float), np.ones(n - 1)
+    elif name == "zero":
+        d, e = 0 * d, 0 * e
+    A = (np.diag(d) + np.diag(e, 1) + np.diag(e, -1)).astype(np.complex128)
+    info, [(w, X)] = run(ctx, [(A * s, np.eye(n, dtype=np.complex128))], real=True)
+    assert info[0] == 0
+    check(A, np.eye(n, dtype=np.complex128), w / s, X)
