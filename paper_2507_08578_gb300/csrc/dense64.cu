@@ -24,9 +24,9 @@
 // Real symmetric pencils (the Gamma point) run the same phases in real arithmetic on compact real
 // copies of the lower triangles: a quarter of the FP64 operations of the O(n^3) phases.
 //
-// Parallel organisation.  The same phase code runs on a "team": either one CTA (many small
-// pencils, one CTA each, barrier = __syncthreads) or a whole cooperative grid (one large pencil,
-// barrier = a grid barrier of this file with a bounded wait).  Work that is independent per
+// Parallel organisation.  The same phase code runs on a "team": one CTA (barrier = __syncthreads) or
+// a cluster of up to eight per pencil of a batch (barrier = the cluster's), or a whole cooperative grid
+// (one large pencil, barrier = a grid barrier of this file with a bounded wait).  Work that is independent per
 // column (the triangular solves, the reflector applications, the inverse iterations) needs no
 // team barrier: one warp owns a column and each lane owns the rows r = lane (mod 32), so values
 // written by one lane are read back only by that lane and everything else travels by shuffles.
@@ -187,6 +187,21 @@ struct CtaTeam {
   __device__ int wsize() const { return blockDim.x >> 5; }
   __device__ bool sync() const {
     __syncthreads();
+    return true;
+  }
+  __device__ void stamp(int) const {}
+};
+
+// The CTAs of one thread-block cluster: barriers in hardware (all CTAs of a cluster are resident), which
+// also order the CTAs' global writes.
+struct ClusterTeam {
+  int crank, csize;
+  __device__ int rank() const { return crank * blockDim.x + threadIdx.x; }
+  __device__ int swrank() const { return (threadIdx.x >> 5) * csize + crank; }
+  __device__ int size() const { return csize * blockDim.x; }
+  __device__ int wsize() const { return csize * (blockDim.x >> 5); }
+  __device__ bool sync() const {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
     return true;
   }
   __device__ void stamp(int) const {}
@@ -1260,6 +1275,13 @@ __global__ void __launch_bounds__(kThreads, 2) hegv_cta_kernel(const Pencil<S>* 
   solve_pencil(T, P);
 }
 
+template <class S>
+__global__ void __launch_bounds__(kThreads, 2) hegv_cluster_kernel(const Pencil<S>* __restrict__ items, int csize) {
+  const Pencil<S> P = items[blockIdx.x / csize];
+  ClusterTeam T{(int)blockIdx.x % csize, csize};
+  solve_pencil(T, P);
+}
+
 size_t pad32(size_t x) { return (x + 31) & ~(size_t)31; }
 
 // Workspace doubles of one pencil, each array padded to 32 doubles: complex, R (complex n^2);
@@ -1318,6 +1340,16 @@ size_t dyn_smem_bytes(int n, size_t ws) {
 }
 constexpr int kMaxN = 4608;  // 3 n complex words must fit in shared memory (221 KB)
 
+// CTAs per pencil of a batch, a portable cluster at most.  A pencil's serial steps leave most of an SM
+// idle and several short waves even out uneven orders, so the line lies at six CTAs per SM (pencils of
+// order 20 to 141; 12 of them on 1, 2, 4, 8 CTAs each: 25.6, 13.7, 7.9, 5.1 ms; 217 of them: 28.0, 18.5,
+// 14.5, 18.2 ms).  At least four columns a CTA.
+int cluster_size(kss_ctx ctx, int count, int nmax) {
+  int c = 8;
+  while (c > 1 && ((long long)count * c > 6LL * std::max(ctx->nsm, 1) || 4 * c > nmax)) c /= 2;
+  return c;
+}
+
 template <class S>
 void launch_cta(kss_ctx ctx, std::vector<Pencil<S>>& small, size_t items_offset, const char* name) {
   if (small.empty()) return;
@@ -1331,9 +1363,26 @@ void launch_cta(kss_ctx ctx, std::vector<Pencil<S>>& small, size_t items_offset,
   for (auto& P : small) P.smem_cols = col_smem_bytes(nmax, sizeof(S)) ? 1 : 0;
   Pencil<S>* d_items = reinterpret_cast<Pencil<S>*>(static_cast<char*>(ctx->dense_items.p) + items_offset);
   KSS_CHECK_CUDA(cudaMemcpyAsync(d_items, small.data(), small.size() * sizeof(Pencil<S>), cudaMemcpyHostToDevice, st));
-  KSS_CHECK_CUDA(cudaFuncSetAttribute(hegv_cta_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   ProfScope ps(ctx, prof_register(name));
-  hegv_cta_kernel<S><<<(unsigned)small.size(), kThreads, sm, st>>>(d_items, (int)small.size());
+  const int csize = cluster_size(ctx, (int)small.size(), nmax);
+  if (csize == 1) {
+    KSS_CHECK_CUDA(cudaFuncSetAttribute(hegv_cta_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    hegv_cta_kernel<S><<<(unsigned)small.size(), kThreads, sm, st>>>(d_items, (int)small.size());
+  } else {
+    KSS_CHECK_CUDA(cudaFuncSetAttribute(hegv_cluster_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)csize;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(small.size() * csize));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    KSS_CHECK_CUDA(cudaLaunchKernelEx(&cfg, hegv_cluster_kernel<S>, (const Pencil<S>*)d_items, csize));
+  }
   KSS_CHECK_CUDA(cudaGetLastError());
 }
 

@@ -207,3 +207,18 @@ def test_tridiagonal_spectra(ctx, name, n):
     info, [(w, X)] = run(ctx, [(A * s, np.eye(n, dtype=np.complex128))], real=True)
     assert info[0] == 0
     check(A, np.eye(n, dtype=np.complex128), w / s, X)
+
+
+@pytest.mark.parametrize("count,n,real", [(3, 33, False), (150, 21, True), (150, 18, False), (400, 9, False), (1000, 5, True)])
+def test_batches_on_clusters(ctx, count, n, real):
+    """Batches whose pencils run on 8, 4, 2 and 1 CTAs each, one of them not positive definite: it
+    stops alone, the others are solved."""
+    ps = [pencil(n - i % 3, seed=300 + i % 7, real=real) for i in range(count)]
+    bad = count // 2
+    A, B = ps[bad]
+    ps[bad] = (A, B - 3.0 * np.linalg.norm(B, 2) * np.eye(B.shape[0]))
+    info, out = run(ctx, ps, real=real)
+    assert info[bad] == 1 and np.all(np.delete(info, bad) == 0)
+    for i in list(range(0, count, max(1, count // 12))) + [count - 1]:
+        if i != bad:
+            check(*ps[i], *out[i])
