@@ -645,6 +645,10 @@ void oz_gemm_cn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const 
                 bool f64out, int digits) {
   if (M <= 0 || N <= 0) return;
   KSS_REQUIRE(K > 0, "digit-product GEMM: K = 0");
+  if (f64in && f64out && digits <= 0 && small_product_cn(M, N, K)) {
+    small_gemm_cn(ctx, M, N, K, A, lda, B, ldb, C, ldc, ar, ai, br, bi, tag);
+    return;
+  }
   const int S = digits > 0 ? digits : (f64in ? 7 : 4);
   OzOperand a;
   if (a_pre) {
@@ -664,6 +668,10 @@ void oz_gemm_nn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const 
                 bool f64out, int digits) {
   if (M <= 0 || N <= 0) return;
   KSS_REQUIRE(K > 0, "digit-product GEMM: K = 0");
+  if (f64in && f64out && digits <= 0 && small_product_nn(M, N, K)) {
+    small_gemm_nn(ctx, M, N, K, A, lda, B, ldb, C, ldc, ar, ai, br, bi, tag);
+    return;
+  }
   const int S = digits > 0 ? digits : (f64in ? 7 : 4);
   OzOperand a;
   if (a_pre) {

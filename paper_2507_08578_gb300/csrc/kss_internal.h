@@ -413,6 +413,16 @@ OzOperand oz_prepare(kss_ctx ctx, OzKind kind, int n, int K, const void* src, lo
 // digits: exact products of the FP32 values to 28 bits of the row scales; with 7: to 49 bits);
 // f64out: complex128 C, else complex64.  a_pre: A already in digit form (static operands), else
 // prepared here.
+// Small complex128 products on the FP64 pipe (gemm_small.cu): which sizes they take, and the products.
+// The first form scales row i of the sum by row_scale[i] s when row_scale is given.
+bool small_product_cn(int M, int N, int K);
+bool small_product_nn(int M, int N, int K);
+void small_gemm_cn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc,
+                   double ar, double ai, double br, double bi, const char* tag, const double* row_scale = nullptr,
+                   double s = 1.0);
+void small_gemm_nn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc,
+                   double ar, double ai, double br, double bi, const char* tag);
+// (complex128 products of small sizes go to the functions above)
 void oz_gemm_cn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc,
                 double ar, double ai, double br, double bi, const char* tag, const OzOperand* a_pre = nullptr,
                 bool f64in = true, bool f64out = true, int digits = 0);

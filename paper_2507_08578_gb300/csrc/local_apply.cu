@@ -940,7 +940,11 @@ void apply_h(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev, v
   // Nonlocal, first half: projector coefficients C = beta^H psi, scaled to alpha * D * C.
   if (s->nproj) {
     ctx->ws_cprj.ensure((size_t)s->nproj * nb * es);
-    if (f64)
+    const bool small = f64 && small_product_cn(s->nproj, nb, kd.npw);
+    if (small)
+      small_gemm_cn(ctx, s->nproj, nb, kd.npw, kd.d_beta64.p, kd.npw, psi, ld, ctx->ws_cprj.p, s->nproj, 1.0, 0.0, 0.0,
+                    0.0, "cprj", s->d_D64.as<double>(), c.alpha);
+    else if (f64)
       oz_gemm_cn(ctx, s->nproj, nb, kd.npw, kd.d_beta64.p, kd.npw, psi, ld, ctx->ws_cprj.p, s->nproj, 1.0, 0.0,
                  0.0, 0.0, "cprj", &beta_oz_cn(s, ik));
     else if (c.fp32_proj)
@@ -949,8 +953,8 @@ void apply_h(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev, v
     else
       tc_gemm_cn_split(ctx, s->nproj, nb, kd.npw, beta_split_cn(s, ik), psi, ld, ctx->ws_cprj.p, s->nproj,
                        1.0, 0.0, 0.0, 0.0, "cprj");
-    scale_rows(ctx, f64, s->nproj, nb, ctx->ws_cprj.p, s->nproj, f64 ? s->d_D64.p : s->d_D32.p,
-               c.alpha);
+    if (!small)
+      scale_rows(ctx, f64, s->nproj, nb, ctx->ws_cprj.p, s->nproj, f64 ? s->d_D64.p : s->d_D32.p, c.alpha);
   }
   if (f64)
     run_local<double>(s, ik, nb, psi, psi_prev, out, ld, c);
@@ -960,7 +964,7 @@ void apply_h(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev, v
   if (s->nproj) {
     if (f64)
       oz_gemm_nn(ctx, kd.npw, nb, s->nproj, kd.d_beta64.p, kd.npw, ctx->ws_cprj.p, s->nproj, out, ld, 1.0, 0.0,
-                 1.0, 0.0, "nonlocal", &beta_oz_nn(s, ik));
+                 1.0, 0.0, "nonlocal", small_product_nn(kd.npw, nb, s->nproj) ? nullptr : &beta_oz_nn(s, ik));
     else if (c.fp32_proj)
       gemm_nn(ctx, false, kd.npw, nb, s->nproj, kd.d_beta32.p, kd.npw, ctx->ws_cprj.p, s->nproj, out, ld, 1.0, 0.0,
               1.0, 0.0, "nonlocal");

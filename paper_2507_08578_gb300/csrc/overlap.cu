@@ -47,7 +47,7 @@ void proj_cn(kss_ctx ctx, bool f64, kss_sys s, int ik, int nb, const void* psi, 
   const int nproj = s->nproj;
   if (f64)
     oz_gemm_cn(ctx, nproj, nb, kd.npw, kd.d_beta64.p, kd.npw, psi, ld, out, nproj, 1, 0, 0, 0, tag,
-               &beta_oz_cn(s, ik));
+               small_product_cn(nproj, nb, kd.npw) ? nullptr : &beta_oz_cn(s, ik));
   else
     tc_gemm_cn_split(ctx, nproj, nb, kd.npw, beta_split_cn(s, ik), psi, ld, out, nproj, 1, 0, 0, 0, tag);
 }
@@ -57,7 +57,7 @@ void proj_nn(kss_ctx ctx, bool f64, kss_sys s, int ik, int nb, const void* coef,
   const int nproj = s->nproj;
   if (f64)
     oz_gemm_nn(ctx, kd.npw, nb, nproj, kd.d_beta64.p, kd.npw, coef, nproj, out, ld, 1, 0, 1, 0, tag,
-               &beta_oz_nn(s, ik));
+               small_product_nn(kd.npw, nb, nproj) ? nullptr : &beta_oz_nn(s, ik));
   else
     tc_gemm_nn_split(ctx, kd.npw, nb, nproj, beta_split_nn(s, ik), coef, nproj, out, ld, 1, 0, 1, 0, tag);
 }

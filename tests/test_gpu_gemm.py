@@ -206,3 +206,23 @@ def test_split_bf16_every_form(ctx, op, M, N, Kd):
                 assert err < 1e-4, (form, sp, err)
     finally:
         K.kss_autotune_clear()
+
+
+@pytest.mark.parametrize("op,M,N,Kd", [(0, 1, 1, 1), (0, 16, 8, 16), (0, 17, 9, 17), (0, 33, 7, 5000), (0, 250, 260, 3),
+                                       (0, 2, 3, 60000), (1, 1, 1, 1), (1, 32, 4, 8), (1, 33, 5, 255), (1, 3, 1000, 256),
+                                       (1, 40000, 2, 7)])
+@pytest.mark.parametrize("alpha,beta", [(1.0, 0.0), (1.0, 1.0), (0.6 + 0.3j, -0.4 + 0.2j)])
+def test_small_fp64_products(ctx, op, M, N, Kd, alpha, beta):
+    """Small complex128 products (edges of their tiles, of the K split and of the sizes they take): each
+    entry within the rounding bound of two sums of K complex terms, (4 K + 16) 2^-53 sum |a| |b|."""
+    import torch
+    rng = np.random.default_rng(M + 3 * N + Kd)
+    A = crand(rng, (M, Kd)) if op == 0 else crand(rng, (Kd, M))
+    B, C0 = crand(rng, (N, Kd)), crand(rng, (N, M))
+    Am = A.conj() if op == 0 else A.T
+    ref = alpha * (Am @ B.T) + beta * C0.T
+    tA, tB, tC = (torch.from_numpy(x).cuda() for x in (A, B, C0))
+    K.kss_gemm(ctx, op, tA, tB, tC, alpha, beta, K.KSS_PREC_FP64)
+    torch.cuda.synchronize()
+    bound = (4 * Kd + 16) * 2.0 ** -53 * (abs(alpha) * (np.abs(Am) @ np.abs(B.T)) + abs(beta) * np.abs(C0.T))
+    assert np.all(np.abs(tC.cpu().numpy().T - ref) <= 2 * bound)
