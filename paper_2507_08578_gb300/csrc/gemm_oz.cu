@@ -16,8 +16,8 @@
 //     same p + q form one "group" whose weight is a single power of two;
 //   * within a chunk of 384 BF16 along K every group sum is an integer below 2^24 (at most 7
 //     pairs of |d d'| <= 2^13 per K entry), so FP32 accumulation in TMEM is exact; after each
-//     chunk the seven group sums are read back, combined in double-float (two FP32 words) and
-//     added to FP64 accumulators in registers; the row exponents are applied at the end.
+//     chunk the seven group sums are read back and added, weighted, to two 64-bit integers per output
+//     (exact); the sum and the row exponents become a double once, at the end.
 //
 // Complex -> real as in the split-BF16 kernel: the B rows hold interleaved (re, im) pairs along K
 // and each complex row of A becomes two real rows on the A side ((re, im) and (-im, re) for
@@ -28,9 +28,14 @@
 // when the tiles do not fill the SMs); warp 0 lane 0 feeds a 2-stage TMA ring (each stage the 7
 // digit tiles of A, 128 x 32 BF16, and of B, 64 x 32 BF16, 64-byte swizzle), warp 1 lane 0
 // issues tcgen05.mma (M = 128, N = 64, K = 16; 28 per 16-wide slice) into 7 TMEM accumulators of
-// 64 columns, warps 2-5 drain the accumulators chunk by chunk.  Every wait is bounded; on time-out
+// 64 columns, warps 2-9 drain the accumulators chunk by chunk.  Every wait is bounded; on time-out
 // the kernel raises the error flag shared with the split-BF16 kernel, drains its own copies,
 // frees TMEM and returns.
+//
+// What bounds it: the MMAs' operand reads from shared memory (6 KB per 128 x 64 x 16 MMA, 48 cycles where
+// the multiplication takes 32).  Measured, per product with its operands prepared: 564 x 564 x 34181
+// 2.47 ms, 34181 x 564 x 256 accumulated 1.92, 256 x 564 x 34181 1.00 (drains in FP64, an epilogue in FP64
+// on every other lane: 3.40, 2.98, 1.25).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -51,7 +56,8 @@ constexpr int NG = 7;                                // digit-pair groups g = p 
 constexpr uint32_t ATILE = TM * TK * 2;              // 8 KB
 constexpr uint32_t BTILE = TN * TK * 2;              // 4 KB
 constexpr int CHUNK = 12;                            // k-blocks per exact chunk (384 BF16 of K)
-constexpr int kOzThreads = 192;
+constexpr int kOzThreads = 320;
+constexpr int kSplitKb = 8192 * CHUNK;               // most k-blocks of one split (sums below 2^50)
 constexpr uint32_t kTmemCols = 512;                  // 7 groups x 64 columns, rounded up
 constexpr unsigned long long kWaitNs = 2000000000ull;
 
@@ -96,10 +102,6 @@ __device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, cons
   return true;
 }
 
-__device__ __forceinline__ double pow2(int e) {  // 2^e for |e| < 1000, exactly
-  return __longlong_as_double((long long)(1023 + e) << 52);
-}
-
 template <int SA, int SB, typename CT>
 __global__ void __launch_bounds__(kOzThreads, 1)
 oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int rowsA,
@@ -131,7 +133,7 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       mbar_init(smem_u32(&empty[s]), 1);
     }
     mbar_init(smem_u32(accf), 1);
-    mbar_init(smem_u32(acce), 4);
+    mbar_init(smem_u32(acce), 8);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -210,12 +212,16 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                      : "memory");
     }
   } else if (warp >= 2) {
-    // Epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (accumulator rows).
-    const int quarter = warp & 3;
+    // Epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (accumulator rows), warps 2-5 columns 0-31
+    // and warps 6-9 columns 32-63.  The group sums are integers below 2^24; their weighted sums over
+    // all chunks are kept exactly in two 64-bit integers, groups 0-2 in units of 2^-28 and groups 3-6
+    // in units of 2^-56 (FP64 sums would hold the FP64 pipe for half as long as a chunk's MMAs).
+    constexpr int TC = TN / 2;
+    const int quarter = warp & 3, colh = ((warp - 2) >> 2) * TC;
     const int row = tm * TM + quarter * 32 + lane;
-    double acc[TN];
+    long long a1[TC], a2[TC];
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[j] = 0.0;
+    for (int j = 0; j < TC; ++j) a1[j] = a2[j] = 0;
     bool ok = true;
     for (int c = 0; c < nchunks; ++c) {
       ok = wait_or_fail(smem_u32(accf), c & 1, vfail);
@@ -226,74 +232,67 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-      for (int c0 = 0; c0 < TN; c0 += 16) {
-        float hi[16], lo[16];
+      for (int c0 = 0; c0 < TC; c0 += 8) {
+        uint32_t r[NG][8];
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
-          uint32_t r[16];
-          const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(g * TN + c0);
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-              : "r"(taddr));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          // group g weighs 2^{-7 g} relative to group 0 (exact in FP32); double-float sum
-          const float sc = __int_as_float((127 - 7 * g) << 23);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float v = __uint_as_float(r[j]) * sc;
-            if (g == 0) {
-              hi[j] = v;
-              lo[j] = 0.f;
-            } else {
-              const float s = hi[j] + v;
-              const float bb = s - hi[j];
-              const float e = (hi[j] - (s - bb)) + (v - bb);
-              hi[j] = s;
-              lo[j] += e;
-            }
-          }
+          const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(g * TN + colh + c0);
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                       : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
+                         "=r"(r[g][6]), "=r"(r[g][7])
+                       : "r"(taddr));
         }
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[c0 + j] += (double)hi[j] + (double)lo[j];
+        for (int j = 0; j < 8; ++j) {
+          int v[NG];
+#pragma unroll
+          for (int g = 0; g < NG; ++g) v[g] = __float2int_rn(__uint_as_float(r[g][j]));
+          a1[c0 + j] += (long long)v[0] * (1 << 14) + (long long)(v[1] * 128 + v[2]);
+          a2[c0 + j] += (long long)v[3] * (1 << 21) + (long long)v[4] * (1 << 14) + (long long)(v[5] * 128 + v[6]);
+        }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(acce));
     }
-    if (ok && nkb > 0) {
-      // value = acc * 2^{ea + eb - 14} (the 2^-14 of group 0)
-      const int er = row < Mr ? ea[row] - 14 : 0;
-      const int col0 = tn * TN;
-      if (part) {
-        double* P = part + (size_t)blockIdx.y * Nr * Mr;
+    if (ok && nkb > 0 && row < Mr) {
+      const int er = ea[row], col0 = tn * TN + colh;
+      const bool cplx = ai != 0.0 || bi != 0.0;
+      using R = decltype(CT{}.x);
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-          const int col = col0 + j;
-          if (row < Mr && col < Nr) P[(size_t)col * Mr + row] = acc[j] * pow2(er + eb[col]);
+      for (int j = 0; j < TC; ++j) {
+        const int col = col0 + j;
+        if (col >= Nr) break;
+        // value a1 2^(E - 28) + a2 2^(E - 56), both put into the fraction of a number with that unit (a1
+        // around 1.5 2^52: below 2^50 for as many chunks as a split takes), whose exponent also takes E
+        // as far as it fits; rounded once
+        const int E = er + eb[col], Ec = max(-980, min(980, E));
+        const long long hi = a1[j] + (a2[j] >> 28), lo = a2[j] & ((1LL << 28) - 1);
+        const long long b1 = ((long long)(1023 + 52 - 28 + Ec) << 52) + (1LL << 51);
+        const long long b2 = (long long)(1023 + 52 - 56 + Ec) << 52;
+        double v = (__longlong_as_double(b1 + hi) - __longlong_as_double(b1 + (1LL << 24))) +
+                   __longlong_as_double(b2 + lo);
+        if (E != Ec) v = ldexp(v, E - Ec);
+        if (part) {
+          part[((size_t)blockIdx.y * Nr + col) * Mr + row] = v;
+          continue;
         }
-      } else {
-        // fused complex result: accumulator row 2i is Re C(i, col), row 2i + 1 is Im C(i, col)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-          const int col = col0 + j;
-          const double v = (row < Mr && col < Nr) ? acc[j] * pow2(er + eb[col]) : 0.0;
-          const double w = __shfl_down_sync(0xffffffffu, v, 1);
-          if (!(lane & 1) && row < Mr && col < Nr) {
-            CT* dst = C + (size_t)col * ldc + (row >> 1);
-            double ox = ar * v - ai * w, oy = ar * w + ai * v;
-            if (br != 0.0 || bi != 0.0) {
-              const CT q = *dst;
-              ox += br * (double)q.x - bi * (double)q.y;
-              oy += br * (double)q.y + bi * (double)q.x;
-            }
-            CT o;
-            o.x = ox;
-            o.y = oy;
-            *dst = o;
+        // row 2i is Re C(i, col), row 2i + 1 is Im C(i, col): consecutive words of C
+        R* dst = reinterpret_cast<R*>(C + (size_t)col * ldc) + row;
+        double o = ar == 1.0 ? v : ar * v;
+        if (cplx) {  // (Mr is even: both rows of a pair are here)
+          const double w = __shfl_xor_sync(__activemask(), v, 1);
+          o = (row & 1) ? o + ai * w : o - ai * w;
+          if (br != 0.0 || bi != 0.0) {
+            const double q = *dst, p = dst[(row & 1) ? -1 : 1];
+            __syncwarp(__activemask());
+            o += (row & 1) ? br * q + bi * p : br * q - bi * p;
           }
+        } else if (br != 0.0) {
+          o = br == 1.0 ? o + (double)*dst : fma(br, (double)*dst, o);
         }
+        *dst = (R)o;
       }
     }
   }
@@ -370,47 +369,55 @@ template <> struct Real<double2> { using T = double; };
 template <> struct Real<float2> { using T = float; };
 
 // K-major complex source (column c: K values at src + c ld) -> digit planes [S][rows][KT] of
-// interleaved (re, im) pairs, one warp per column.  pair = 1 (the A operand of A^H B): row 2c holds
+// interleaved (re, im) pairs, one CTA per column (a warp per column left most SMs idle below a
+// thousand columns), two neighbouring values a thread.  pair = 1 (the A operand of A^H B): row 2c holds
 // (re, im) and row 2c + 1 (-im, re), both with the column's exponent.
 template <int S, typename CS>
-__global__ void oz_prep_k(const CS* __restrict__ src, long long ld, int K, int ncols, int KT,
-                          __nv_bfloat16* __restrict__ dst, int rows, int* __restrict__ erow, int pair) {
+__global__ void oz_prep_k(const CS* __restrict__ src, long long ld, int K, int KT, __nv_bfloat16* __restrict__ dst,
+                          int rows, int* __restrict__ erow, int pair) {
   using R = typename Real<CS>::T;
-  const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (c >= ncols) return;
+  __shared__ unsigned long long red[32];
+  const int c = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const CS* x = src + (size_t)c * ld;
   unsigned long long mx = 0;
-  for (int k = lane; k < K; k += 32) {
+#pragma unroll 4
+  for (int k = tid; k < K; k += nt) {
     const CS v = x[k];
     const unsigned long long a = Bits<R>::of(v.x) & Bits<R>::kAbs;
     const unsigned long long b = Bits<R>::of(v.y) & Bits<R>::kAbs;
     mx = a > mx ? a : mx;
     mx = b > mx ? b : mx;
   }
-  const int e = row_exponent<R>(warp_max_u64(mx));
+  mx = warp_max_u64(mx);
+  if ((tid & 31) == 0) red[tid >> 5] = mx;
+  __syncthreads();
+  mx = warp_max_u64((tid & 31) < nt / 32 ? red[tid & 31] : 0);
+  const int e = row_exponent<R>(mx);
   const int r0 = pair ? 2 * c : c;
-  if (lane == 0) {
+  if (tid == 0) {
     erow[r0] = e;
     if (pair) erow[r0 + 1] = e;
   }
   const size_t plane = (size_t)rows * KT;
-  for (int k = lane; k < KT / 2; k += 32) {
-    R re = 0, im = 0;
-    if (k < K) {
-      const CS v = x[k];
-      re = v.x;
-      im = v.y;
+  __nv_bfloat16* o0 = dst + (size_t)r0 * KT;
+  for (int k = 2 * tid; k < KT / 2; k += 2 * nt) {  // KT / 2 is a multiple of 16
+    CS v[2];
+    float dr[2][S], di[2][S];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      v[u].x = v[u].y = 0;
+      if (k + u < K) v[u] = x[k + u];
+      digits<S>(v[u].x, e, dr[u]);
+      digits<S>(v[u].y, e, di[u]);
     }
-    float dr[S], di[S];
-    digits<S>(re, e, dr);
-    digits<S>(im, e, di);
 #pragma unroll
     for (int p = 0; p < S; ++p) {
-      __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(dst + p * plane + (size_t)r0 * KT);
-      o[k] = __floats2bfloat162_rn(dr[p], di[p]);
+      __nv_bfloat162 q[2] = {__floats2bfloat162_rn(dr[0][p], di[0][p]), __floats2bfloat162_rn(dr[1][p], di[1][p])};
+      *reinterpret_cast<uint2*>(o0 + p * plane + 2 * k) = *reinterpret_cast<uint2*>(q);
       if (pair) {
-        __nv_bfloat162* o1 = reinterpret_cast<__nv_bfloat162*>(dst + p * plane + (size_t)(r0 + 1) * KT);
-        o1[k] = __floats2bfloat162_rn(-di[p], dr[p]);
+        q[0] = __floats2bfloat162_rn(-di[0][p], dr[0][p]);
+        q[1] = __floats2bfloat162_rn(-di[1][p], dr[1][p]);
+        *reinterpret_cast<uint2*>(o0 + KT + p * plane + 2 * k) = *reinterpret_cast<uint2*>(q);
       }
     }
   }
@@ -551,7 +558,7 @@ void launch_oz(kss_ctx ctx, const OzOperand& a, const OzOperand& b, int M, int N
   // One product with `splits` K-splits into C (ldc, alpha, beta).
   auto launch = [&](int splits, CT* Cd, int ldd, double br_, double bi_, bool prof) {
     int kps = (kb_total + splits - 1) / splits;
-    kps = ((kps + CHUNK - 1) / CHUNK) * CHUNK;
+    kps = std::min(((kps + CHUNK - 1) / CHUNK) * CHUNK, kSplitKb);
     splits = (kb_total + kps - 1) / kps;
     if (splits > 1) ctx->oz_part.ensure((size_t)splits * Mr * Nr * sizeof(double));
     const bool fused = splits == 1;
@@ -617,8 +624,10 @@ void prepare_as(kss_ctx ctx, OzKind kind, int n, int K, const CS* src, long long
     oz_exp_m<CS><<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(src, ld, n, K, o.e);
     oz_prep_m<S, CS><<<g, dim3(32, 8), 0, ctx->stream>>>(src, ld, n, K, o.KT, o.planes, o.rows, o.e);
   } else {
-    oz_prep_k<S, CS><<<(unsigned)((n + 7) / 8), 256, 0, ctx->stream>>>(src, ld, K, n, o.KT, o.planes, o.rows, o.e,
-                                                                      kind == OZ_CN_A ? 1 : 0);
+    // wide CTAs where the columns alone would leave SMs short of threads
+    const int nt = n < 3 * std::max(ctx->nsm, 1) && K > 2048 ? 768 : 256;
+    oz_prep_k<S, CS><<<(unsigned)n, nt, 0, ctx->stream>>>(src, ld, K, o.KT, o.planes, o.rows, o.e,
+                                                          kind == OZ_CN_A ? 1 : 0);
   }
 }
 
