@@ -33,7 +33,7 @@ using fftr::Split;
 // Shared memory of the CTA-wide pass B for box length N and sphere window W3.
 size_t wide_b_smem(int N, int W3, size_t es) {
   const size_t P = (size_t)((N + 1) | 1);  // the odd pitches of the CTA-wide form
-  return es * ((size_t)N + (size_t)W3 * P + (size_t)N * P) + sizeof(int) * N;
+  return es * (2 * (size_t)N + (size_t)W3 * P + (size_t)N * P) + sizeof(int) * N;
 }
 
 bool has_ct(int code) {
@@ -286,6 +286,7 @@ void BatchEngine::prepare_t() {
   // form with its split code).
   std::vector<std::pair<long long, int>> key(n);
   std::vector<PassBSched> bs(n);
+  std::vector<char> pruned(n, 0);  // the window fits the pruned form of the CTA-wide pass B
   for (int u = 0; u < n; ++u) {
     const RegPlanHost& p = plans[u];
     int c1 = -1, c23 = -1;
@@ -296,10 +297,11 @@ void BatchEngine::prepare_t() {
     RegPlan rp;
     std::memcpy(&rp, &p, sizeof(RegPlan));
     bs[u] = pass_b_schedule<T>(ctx, au, rp.s2, true);
-    if (bs[u].threads && (!group_kernel_w<T>(bs[u].A, bs[u].B, bs[u].threads) ||
+    pruned[u] = bs[u].threads && pruned_w<T>(au, bs[u].A, bs[u].B);
+    if (bs[u].threads && (!group_kernel_w<T>(bs[u].A, bs[u].B, bs[u].threads, pruned[u]) ||
                           wide_b_smem(au.N2, au.W3, es) > 227 * 1024 || au.N2 != au.N3))
       bs[u].threads = 0;
-    const long long k2 = bs[u].threads ? 10001 + (long long)(bs[u].A * 32 + bs[u].B) * 3 + bs[u].threads / 128 - 1
+    const long long k2 = bs[u].threads ? 10001 + ((long long)(bs[u].A * 32 + bs[u].B) * 3 + bs[u].threads / 128 - 1) * 2 + pruned[u]
                                        : (long long)(c23 + 1);
     key[u] = {(long long)(c1 + 1) * 100000 + k2, u};
     if (sizeof(T) == 4 && fused_code(units[u]->sys)) key[u].first = -100000 + fused_code(units[u]->sys);
@@ -320,7 +322,7 @@ void BatchEngine::prepare_t() {
     const int c23 = (p.s2.A == p.s3.A && p.s2.B == p.s3.B && has_ct(p.s2.A * 32 + p.s2.B)) ? p.s2.A * 32 + p.s2.B : -1;
     const PassBSched& b = bs[u];
     if (classes.empty() || i == 0 || key[i].first != key[i - 1].first) {
-      classes.push_back(PassClass{c1, b.threads ? -1 : c23, i, 0, 0, 0, 0, 0, 0, b.A, b.B, b.threads});
+      classes.push_back(PassClass{c1, b.threads ? -1 : c23, i, 0, 0, 0, 0, 0, 0, b.A, b.B, b.threads, pruned[u] != 0});
       if (key[i].first < 0) classes.back().fcode = (int)(key[i].first + 100000);
     }
     PassClass& pc = classes.back();
@@ -368,7 +370,7 @@ void BatchEngine::prepare_t() {
     }
     want(group_kernel<T, 0>(pc.code1), pc.smem_ac);
     want(group_kernel<T, 2>(pc.code1), pc.smem_ac);
-    if (pc.wnt) want(group_kernel_w<T>(pc.wa, pc.wb, pc.wnt), pc.smem_bw);
+    if (pc.wnt) want(group_kernel_w<T>(pc.wa, pc.wb, pc.wnt, pc.wpruned), pc.smem_bw);
     else want(group_kernel<T, 1>(pc.code23), pc.smem_b);
   }
   for (const auto& kv : need)
@@ -589,7 +591,7 @@ void BatchEngine::launch_filter_t() {
       if (pc.fcode) continue;
       ProfScope ps(ctx, idb);
       if (pc.wnt)
-        group_kernel_w<T>(pc.wa, pc.wb, pc.wnt)<<<pc.blocks_b, pc.wnt, pc.smem_bw, ctx->stream>>>(it, pc.count, scr_warp);
+        group_kernel_w<T>(pc.wa, pc.wb, pc.wnt, pc.wpruned)<<<pc.blocks_b, pc.wnt, pc.smem_bw, ctx->stream>>>(it, pc.count, scr_warp);
       else
         group_kernel<T, 1>(pc.code23)<<<pc.blocks_b, kThreads, pc.smem_b, ctx->stream>>>(it, pc.count, scr_warp);
     }

@@ -53,8 +53,8 @@ __global__ void __launch_bounds__(kThreads) group_pass(const LocalItem<T>* __res
 }
 
 // Pass B of a class with a common compile-time y/z split, in the CTA-wide form.
-template <typename T, int A, int B, int NT>
-__global__ void __launch_bounds__(NT) group_passw(const LocalItem<T>* __restrict__ items, int n, int) {
+template <typename T, int A, int B, int CW>
+__global__ void __launch_bounds__(kWideThreads) group_passw(const LocalItem<T>* __restrict__ items, int n, int) {
   __shared__ LocalArgs<T> sa;
   __shared__ int s_local, s_idle;
   if (threadIdx.x == 0) {
@@ -66,17 +66,22 @@ __global__ void __launch_bounds__(NT) group_passw(const LocalItem<T>* __restrict
   __syncthreads();
   if (s_idle) return;
   const int local = s_local;
-  pass_bw_body<T, A, B, NT>(sa, local % sa.N1, local / sa.N1);
+  pass_bw_body<T, A, B, CW>(sa, local % sa.N1, local / sa.N1);
 }
 
 template <typename T>
 using GroupKernel = void (*)(const LocalItem<T>*, int, int);
 
-// Grouped CTA-wide pass B for split (A, B) at nt threads (128 in single precision, 256 or 384);
-// nullptr when no instance
-// exists.  Instances live in batch_wide_f32.cu / batch_wide_f64.cu.
+// Grouped CTA-wide pass B for split (A, B) at nt threads (128 in single precision, 256 or 384), in the
+// form pruned to the sphere's window or the full one; nullptr when no instance exists.  pruned_w:
+// whether the pruned form covers a unit's window.  Instances live in batch_wide_f32.cu / batch_wide_f64.cu.
 template <typename T>
-GroupKernel<T> group_kernel_w(int A, int B, int nt);
+GroupKernel<T> group_kernel_w(int A, int B, int nt, bool pruned);
+template <typename T>
+bool pruned_w(const LocalArgs<T>& a, int A, int B) {
+  const int cw = wide_prune_cw(A, B, a.lo2, a.W2, a.lo3, a.W3);
+  return cw > 0 && cw <= wide_edge(A);
+}
 
 }  // namespace bk
 }  // namespace kss

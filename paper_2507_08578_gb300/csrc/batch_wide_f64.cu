@@ -1,17 +1,17 @@
-// Grouped CTA-wide pass B instances of the batch engine, double precision: every split
-// of KSS_WIDE_SPLITS at 256 and 384 threads per CTA.
+// Grouped CTA-wide pass B instances of the batch engine, double precision: every split of
+// KSS_WIDE_SPLITS, full and pruned to the sphere's window.
 #include "batch_kernels.cuh"
 
 namespace kss {
 namespace bk {
 
 template <>
-GroupKernel<double> group_kernel_w<double>(int A, int B, int nt) {
+GroupKernel<double> group_kernel_w<double>(int A, int B, int nt, bool pruned) {
   if (nt != 256 && nt != 384) return nullptr;
   switch (A * 32 + B) {
 #define KSS_CASE(x, y) \
   case x * 32 + y:     \
-    return nt == 256 ? group_passw<double, x, y, 256> : group_passw<double, x, y, 384>;
+    return pruned ? group_passw<double, x, y, wide_edge(x)> : group_passw<double, x, y, 0>;
     KSS_WIDE_SPLITS(KSS_CASE)
 #undef KSS_CASE
     default:

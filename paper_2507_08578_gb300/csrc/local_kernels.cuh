@@ -521,7 +521,10 @@ __device__ __forceinline__ void pass_c_body(const LocalArgs<T>& a, const RegPlan
 // a column holds (to read V).  The z columns of the whole plane live in a second buffer Z, so the
 // inverse z transform reads the sphere window rows of Q (zeros elsewhere) and the forward one
 // writes only the window rows back.  Requires N2 == N3 == A * B.
-constexpr int kWideThreads = 384;  // 12 warps: 96-point stages split into whole rounds of tasks
+constexpr int kWideThreads = 384;  // the most a launch uses: 96-point stages split into whole rounds of tasks
+// Edge width of the pruned instance of a DFT-A stage, 0 when there is nothing to prune: what a box of the
+// default size leaves (N >= 4 max|m| + 1, so |m| < N / 4).
+constexpr int wide_edge(int A) { return 2 * ((A + 3) / 4) < A ? (A + 3) / 4 : 0; }
 
 template <typename T, int A, int B>
 struct WideB {
@@ -529,9 +532,26 @@ struct WideB {
   static constexpr int QS = (N + 1) | 1;  // odd row / column pitches: with the index along the
   static constexpr int ZS = (N + 1) | 1;  // pitch fastest across lanes, no shared-memory bank conflicts
   static size_t smem(int W3) {
-    return sizeof(typename CT<T>::C) * ((size_t)N + (size_t)W3 * QS + (size_t)N * ZS) + sizeof(int) * N;
+    return sizeof(typename CT<T>::C) * (2 * (size_t)N + (size_t)W3 * QS + (size_t)N * ZS) + sizeof(int) * N;
   }
 };
+
+// The n twiddles of one task, consecutive in a table whose rows are 16-byte aligned for even n: two
+// single-precision values a load.
+template <int n, typename C>
+__device__ __forceinline__ void load_twiddles(const C* row, C (&w)[n]) {
+  if constexpr (sizeof(C) == 8 && n % 2 == 0) {
+#pragma unroll
+    for (int k = 0; k < n; k += 2) {
+      const float4 q = *reinterpret_cast<const float4*>(row + k);
+      w[k] = make_float2(q.x, q.y);
+      w[k + 1] = make_float2(q.z, q.w);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < n; ++k) w[k] = row[k];
+  }
+}
 
 // Pruned stages (CW > 0): the window rows of y and z (the sphere's extent, about 0.4 N) occupy,
 // in the strided index r + B i of a DFT-A stage, only the first CW and the last CW values of i, so
@@ -539,50 +559,69 @@ struct WideB {
 // stages compute only those outputs (the others are discarded): fftr::rdft_m with the edge mask.
 // Valid when B CW exceeds the window's largest index and is at least its most negative index's
 // magnitude along both y and z (wide_prune_cw); CW = 0 is the full transform.
-template <typename T, int A, int B, int NT = kWideThreads, int CW = 0>
+//
+// What bounds it in single precision: issue slots, of which the FP32 arithmetic takes a third.  So
+// the twiddles of a task lie side by side in two tables, the window rows of the pruned form are at
+// constant offsets from one pointer (no table of rows), and the slab is read and written a row per
+// warp.  Measured, 564 bands at 96 points: 1.70 -> 1.62 ms; filter of a batch of 12 units of 27 to 60
+// points, pruned there too: 136 -> 126 ms.
+template <typename T, int A, int B, int CW = 0>
 __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int nl) {
   using C = typename CT<T>::C;
   using G = WideB<T, A, B>;
   constexpr int N = G::N, QS = G::QS, ZS = G::ZS;
   constexpr unsigned MW = fftr::edge_mask<A, CW>(), MF = fftr::full_mask<A>();
   extern __shared__ __align__(16) unsigned char smraw[];
-  C* tw = reinterpret_cast<C*>(smraw);  // e^{-2 pi i m / N}, m < N
-  C* Q = tw + N;                        // W3 rows (z in the sphere window) x N (y)
-  C* Z = Q + a.W3 * QS;                 // N columns (y position) x N (z)
-  int* zmap = reinterpret_cast<int*>(Z + N * ZS);
-  const int tid = threadIdx.x;
-  const int W3 = a.W3, W2 = a.W2;
-  for (int i = tid; i < N; i += NT) tw[i] = a.tw2[i];
-  for (int z = tid; z < N; z += NT) {
-    int u = (z - a.lo3) % N;
-    if (u < 0) u += N;
-    zmap[z] = u < W3 ? u : -1;
+  C* twi = reinterpret_cast<C*>(smraw);  // [r < B][k < A]: e^{+2 pi i r k / N} of the inverse stages
+  C* twf = twi + N;                      // [k < A][q < B]: e^{-2 pi i k q / N} of the forward stages
+  C* Q = twf + N;                        // W3 rows (z in the sphere window) x N (y)
+  C* Z = Q + a.W3 * QS;                  // N columns (y position) x N (z)
+  int* zmap = reinterpret_cast<int*>(Z + N * ZS);  // full form only
+  const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
+  const int W3 = a.W3, W2 = a.W2, lo3 = a.lo3;
+  for (int i = tid; i < N; i += NT) {
+    const int r = i / A, k = i - r * A, k2 = i / B, q = i - k2 * B;
+    C w = a.tw2[r * k];
+    w.y = -w.y;
+    twi[i] = w;
+    twf[i] = a.tw2[k2 * q];
   }
-  for (int i = tid; i < W3 * QS; i += NT) Q[i] = C{0, 0};
-  __syncthreads();
+  if constexpr (CW == 0) {
+    for (int z = tid; z < N; z += NT) {
+      int u = (z - lo3) % N;
+      if (u < 0) u += N;
+      zmap[z] = u < W3 ? u : -1;
+    }
+  }
   C* slab = a.work + ((size_t)nl * a.N1 + x) * W3 * W2;
-  const fftr::FastDiv dw2(W2), dw3(W3);
-  for (int i = tid; i < W3 * W2; i += NT) {
-    const int u3 = dw2(i), u2 = i - u3 * W2;
-    Q[u3 * QS + fftr::wrap_add(a.lo2, u2, N)] = slab[i];
+  const fftr::FastDiv dw3(W3);
+  // a warp per row: the window's values in place, zeros around them
+#pragma unroll 2
+  for (int u3 = warp; u3 < W3; u3 += nw) {
+    const C* src = slab + u3 * W2;
+#pragma unroll
+    for (int y0 = 0; y0 < N; y0 += 32) {
+      const int y = y0 + lane;
+      int u2 = y - a.lo2;
+      if (u2 < 0) u2 += N;
+      else if (u2 >= N) u2 -= N;
+      if (y < N) Q[u3 * QS + y] = u2 < W2 ? src[u2] : C{0, 0};
+    }
   }
   __syncthreads();
   // ---- y, inverse ----
   for (int t = tid; t < W3 * B; t += NT) {
     const int r = dw3(t), u = t - r * W3;  // rows fastest across lanes
     C* row = Q + u * QS + r;
-    C v[A];
+    C v[A], w[A];
+    load_twiddles(twi + r * A, w);
     fftr::static_for<0, A>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
       if constexpr (MW >> i & 1u) v[i] = row[B * i];
     });
     fftr::rdft_m<A, MW, MF>(v, (T)1);
 #pragma unroll
-    for (int k = 1; k < A; ++k) {
-      C w = tw[r * k];
-      w.y = -w.y;
-      v[k] = fftr::mul(v[k], w);
-    }
+    for (int k = 1; k < A; ++k) v[k] = fftr::mul(v[k], w[k]);
 #pragma unroll
     for (int k = 0; k < A; ++k) row[B * k] = v[k];
   }
@@ -598,24 +637,30 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
     for (int j = 0; j < B; ++j) row[j] = v[j];
   }
   __syncthreads();
+  // Window row of z = r + B i, as a row of Q relative to row r - lo3 (pruned form: the first CW
+  // values of i are z >= 0, the last CW are z - N; the window straddles 0).
+  auto wrow = [](int i) { return B * i - (2 * i >= A ? N : 0); };
   // ---- z, inverse stage 1 (column p of the plane; only window rows are nonzero) ----
   for (int t = tid; t < N * B; t += NT) {
     const int r = t / N, p = t - r * N;
-    C v[A];
+    C v[A], w[A];
+    load_twiddles(twi + r * A, w);
+    const int u0 = r - lo3;
+    const C* q0 = Q + u0 * QS + p;
     fftr::static_for<0, A>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
       if constexpr (MW >> i & 1u) {
-        const int u = zmap[r + B * i];
-        v[i] = u >= 0 ? Q[u * QS + p] : C{0, 0};
+        if constexpr (CW > 0) {
+          v[i] = (unsigned)(u0 + wrow(i)) < (unsigned)W3 ? q0[wrow(i) * QS] : C{0, 0};
+        } else {
+          const int u = zmap[r + B * i];
+          v[i] = u >= 0 ? Q[u * QS + p] : C{0, 0};
+        }
       }
     });
     fftr::rdft_m<A, MW, MF>(v, (T)1);
 #pragma unroll
-    for (int k = 1; k < A; ++k) {
-      C w = tw[r * k];
-      w.y = -w.y;
-      v[k] = fftr::mul(v[k], w);
-    }
+    for (int k = 1; k < A; ++k) v[k] = fftr::mul(v[k], w[k]);
     C* col = Z + p * ZS + r;
 #pragma unroll
     for (int k = 0; k < A; ++k) col[B * k] = v[k];
@@ -639,8 +684,10 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
       v[k2].y *= vv;
     }
     fftr::rdft<B>(v, (T)-1);
+    C w[B];
+    load_twiddles(twf + k * B, w);
 #pragma unroll
-    for (int q = 1; q < B; ++q) v[q] = fftr::mul(v[q], tw[k * q]);
+    for (int q = 1; q < B; ++q) v[q] = fftr::mul(v[q], w[q]);
 #pragma unroll
     for (int q = 0; q < B; ++q) col[q] = v[q];
   }
@@ -653,11 +700,17 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = col[B * m];
     fftr::rdft_m<A, MF, MW>(v, (T)-1);
+    const int u0 = q - lo3;
+    C* q0 = Q + u0 * QS + p;
     fftr::static_for<0, A>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
       if constexpr (MW >> k & 1u) {
-        const int u = zmap[q + B * k];
-        if (u >= 0) Q[u * QS + p] = v[k];
+        if constexpr (CW > 0) {
+          if ((unsigned)(u0 + wrow(k)) < (unsigned)W3) q0[wrow(k) * QS] = v[k];
+        } else {
+          const int u = zmap[q + B * k];
+          if (u >= 0) Q[u * QS + p] = v[k];
+        }
       }
     });
   }
@@ -666,12 +719,13 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
   for (int t = tid; t < W3 * A; t += NT) {
     const int r = dw3(t), u = t - r * W3;
     C* row = Q + u * QS + B * r;
-    C v[B];
+    C v[B], w[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = row[j];
     fftr::rdft<B>(v, (T)-1);
+    load_twiddles(twf + r * B, w);
 #pragma unroll
-    for (int q = 1; q < B; ++q) v[q] = fftr::mul(v[q], tw[r * q]);
+    for (int q = 1; q < B; ++q) v[q] = fftr::mul(v[q], w[q]);
 #pragma unroll
     for (int q = 0; q < B; ++q) row[q] = v[q];
   }
@@ -689,9 +743,9 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
     });
   }
   __syncthreads();
-  for (int i = tid; i < W3 * W2; i += NT) {
-    const int u3 = dw2(i), u2 = i - u3 * W2;
-    slab[i] = Q[u3 * QS + fftr::wrap_add(a.lo2, u2, N)];
+  for (int u3 = warp; u3 < W3; u3 += nw) {
+    C* dst = slab + u3 * W2;
+    for (int u2 = lane; u2 < W2; u2 += 32) dst[u2] = Q[u3 * QS + fftr::wrap_add(a.lo2, u2, N)];
   }
 }
 
