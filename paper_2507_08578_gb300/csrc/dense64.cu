@@ -319,132 +319,148 @@ __device__ void finish(const Team&, const Pencil<double2>&) {}
 template <class S>
 __device__ __forceinline__ double* vrdiag(const Pencil<S>& P) { return P.vec + 8 * P.n; }
 
-// Panel width of the blocked Cholesky: 16 columns (one row of the panel lives in a thread's
-// registers while it is solved against the diagonal block).
-template <class S> __host__ __device__ constexpr int chol_panel() { return 16; }
+// Panel width of the blocked Cholesky.
+constexpr int kPanel = 16;
 // Shared memory of the blocked Cholesky: the diagonal block (pitch panel + 1) and its 1 / L[j][j].
 template <class S> __host__ __device__ constexpr size_t chol_smem() {
-  return sizeof(S) * (size_t)chol_panel<S>() * (chol_panel<S>() + 1) + sizeof(double) * chol_panel<S>();
+  return sizeof(S) * (size_t)kPanel * (kPanel + 1) + sizeof(double) * kPanel;
 }
 
 // Blocked right-looking Cholesky B = L L^H in panels of W columns, two team barriers per panel:
 //   1. every CTA factors the W x W diagonal block in its own shared memory (the same arithmetic
-//      in every CTA, so the copies agree bit for bit; the team's first CTA writes it back);
-//   2. the rows below it are solved against it, L21 = A21 L11^{-H} (one warp per 32 rows, one
-//      row per lane, its W entries in registers): no barrier between the rows;
-//   3. barrier; the trailing lower triangle is updated, A22 -= L21 L21^H (one warp per column,
-//      one row per lane, the column's W factors broadcast once); barrier.
+//      in every CTA, so the copies agree bit for bit; the team's first CTA writes it back), one
+//      entry of the triangle per thread;
+//   2. the rows below it are solved against it, L21 = A21 L11^{-H}, four rows a warp: eight groups of
+//      lanes hold two columns each and pass every finished column on by shuffles;
+//   3. barrier; the trailing lower triangle is updated, A22 -= L21 L21^H, a warp per 32 rows of
+//      one column, one row per lane, the column's W factors broadcast once; barrier.
+// What bounds it: a warp's FP64 instruction takes 64 cycles of its quarter of the SM, so each step is
+// spread until no warp has a long list of them, and the update's tasks are equal (columns of
+// the triangle in pairs of constant length).  Cycles per panel (diagonal / rows / update), order 564
+// complex: 23k / 11k / 18k (one warp, 32 rows a warp, a warp a column: 53k / 35k / 48k); 1127 real:
+// 19k / 5k / 18k (26k / 11k / 33k).
 // Returns false when the solve stops (non-positive pivot: *info set; or an abandoned barrier).
 template <class Team, class S>
 __device__ bool cholesky(const Team& T, const Pencil<S>& P, S* smem) {
-  constexpr int W = chol_panel<S>(), LP = W + 1;
+  constexpr int W = kPanel, LP = W + 1;
+  static_assert(W == 16, "the lane maps below");
   const int n = P.n, ld = P.ldb;
   S* B = P.B;
   double* rd = vrdiag(P);
   S* Lb = smem;  // diagonal block, column-major with pitch LP
   double* rdb = reinterpret_cast<double*>(Lb + W * LP);
   __shared__ int s_bad;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const bool first_cta = T.rank() < (int)blockDim.x;
-  static_assert(W <= 32 && (W & (W - 1)) == 0, "one row of the diagonal block a lane");
+  // entry (di, dk), di >= dk, of thread tid < W (W + 1) / 2: columns of the triangle one after another
+  int di = tid, dk = 0;
+  while (dk < W && di >= W - dk) {
+    di -= W - dk;
+    ++dk;
+  }
+  di += dk;
+  const bool mine = dk < W;
+  const int nwt = (W * (W + 1) / 2 + 31) / 32;  // warps with entries
   for (int p0 = 0; p0 < n; p0 += W) {
     const int w = min(W, n - p0);
     // 1. the diagonal block
-    for (int e = tid; e < W * W; e += blockDim.x) {
-      const int c = e / W, r = e - c * W;
-      Lb[c * LP + r] = (r < w && c < w && r >= c) ? B[(p0 + r) + (size_t)(p0 + c) * ld] : mk<S>(0.0, 0.0);
-    }
-    if (tid >= w && tid < W) rdb[tid] = 0.0;
+    if (tid < W) rdb[tid] = 0.0;
     if (tid == 0) s_bad = 0;
+    S c = mk<S>(0.0, 0.0);
+    if (mine) {
+      if (di < w) c = B[(p0 + di) + (size_t)(p0 + dk) * ld];
+      Lb[dk * LP + di] = c;
+    }
     __syncthreads();
-    if (warp == 0) {  // unblocked right-looking, lane = row, the row's entries in registers
-      S r[W];
-      const int i = lane & (W - 1);
-#pragma unroll
-      for (int k = 0; k < W; ++k) r[k] = Lb[k * LP + i];
-      int bad = 0;
-#pragma unroll
-      for (int j = 0; j < W; ++j) {
-        if (j < w && !bad) {
-          const double d = re(shfl_c(r[j], j));
-          if (!(d > 0.0) || !isfinite(d)) {
-            bad = p0 + j + 1;
-          } else {
-            const double q = fast_rsqrt(d);
-            r[j] = i == j ? mk<S>(sqrt_from(d, q), 0.0) : cscale(r[j], q);
-            if (lane == j) rdb[j] = q;
-#pragma unroll
-            for (int k = j + 1; k < W; ++k) r[k] = cfms(r[j], conjd(shfl_c(r[j], k)), r[k]);
-          }
+    for (int j = 0; j < w; ++j) {
+      const double d = re(Lb[j * LP + j]);
+      const bool bad = !(d > 0.0) || !isfinite(d);
+      if (bad && tid == 0) s_bad = p0 + j + 1;
+      if (bad) break;  // the same in every thread
+      if (mine && dk == j) {
+        const double q = fast_rsqrt(d);
+        if (di == j) {  // (the block keeps the pivot, which other threads may still read)
+          c = mk<S>(sqrt_from(d, q), 0.0);
+          rdb[j] = q;
+        } else {
+          Lb[j * LP + di] = c = cscale(c, q);
         }
       }
-      if (lane < W) {
-#pragma unroll
-        for (int k = 0; k < W; ++k)
-          if (k <= i) Lb[k * LP + i] = r[k];
+      __syncthreads();
+      if ((tid >> 5) < nwt) {
+        if (mine && dk > j) {
+          c = cfms(Lb[j * LP + di], conjd(Lb[j * LP + dk]), c);
+          if (di == dk) Lb[dk * LP + di] = c;  // the pivots to come
+        }
       }
-      if (bad && lane == 0) s_bad = bad;
+      __syncthreads();
     }
     __syncthreads();
     if (s_bad) {
       if (T.rank() == 0) *P.info = s_bad;
       return false;
     }
-    // 2. the rows below: l_ij = (a_ij - sum_{k<j} l_ik conj(L11[j][k])) / L11[j][j]
-    for (int rb = p0 + w + 32 * T.swrank(); rb < n; rb += 32 * T.wsize()) {
-      const int i = rb + lane;
+    // 2. the rows below: column by column, the rest of the row updated with each finished column
+    for (int rb = p0 + w + 4 * T.swrank(); rb < n; rb += 4 * T.wsize()) {
+      const int i = rb + (lane & 3), cg = lane >> 2;  // columns cg and cg + 8
+      S r0 = mk<S>(0.0, 0.0), r1 = r0;
       if (i < n) {
-        S row[W];
+        if (cg < w) r0 = B[i + (size_t)(p0 + cg) * ld];
+        if (cg + 8 < w) r1 = B[i + (size_t)(p0 + cg + 8) * ld];
+      }
 #pragma unroll
-        for (int j = 0; j < W; ++j) row[j] = j < w ? B[i + (size_t)(p0 + j) * ld] : mk<S>(0.0, 0.0);
-        // column by column to the right: the W - 1 - j updates of a column are independent (the
-        // dependent chain is 2 W operations of 64 cycles, W^2 / 2 with the sums formed row by row)
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-          row[j] = cscale(row[j], rdb[j]);
-#pragma unroll
-          for (int k = j + 1; k < W; ++k) row[k] = cfms(row[j], conjd(Lb[j * LP + k]), row[k]);
+      for (int j = 0; j < W; ++j) {
+        const S f = cscale(shfl_c(j < 8 ? r0 : r1, (lane & 3) | (j & 7) << 2), rdb[j]);
+        if (j < 8) {
+          if (cg == j) r0 = f;
+          else if (cg > j) r0 = cfms(f, conjd(Lb[j * LP + cg]), r0);
+          r1 = cfms(f, conjd(Lb[j * LP + cg + 8]), r1);
+        } else {
+          if (cg == j - 8) r1 = f;
+          else if (cg > j - 8) r1 = cfms(f, conjd(Lb[j * LP + cg + 8]), r1);
         }
-#pragma unroll
-        for (int j = 0; j < W; ++j)
-          if (j < w) B[i + (size_t)(p0 + j) * ld] = row[j];
+      }
+      if (i < n) {
+        if (cg < w) B[i + (size_t)(p0 + cg) * ld] = r0;
+        if (cg + 8 < w) B[i + (size_t)(p0 + cg + 8) * ld] = r1;
       }
     }
     if (!T.sync()) return false;
     // (behind the barrier: every CTA has read the block that this overwrites)
     if (first_cta) {
-      for (int e = tid; e < w * w; e += blockDim.x) {
-        const int c = e / w, r = e - c * w;
-        if (r >= c) B[(p0 + r) + (size_t)(p0 + c) * ld] = Lb[c * LP + r];
-      }
+      if (mine && di < w) B[(p0 + di) + (size_t)(p0 + dk) * ld] = c;
       for (int j = tid; j < w; j += blockDim.x) rd[p0 + j] = rdb[j];
     }
-    // 3. the trailing lower triangle
-    if (p0 + w < n) {
-      for (int k = p0 + w + T.swrank(); k < n; k += T.wsize()) {
-        S f[W];
-        const S mine = lane < w ? conjd(B[k + (size_t)(p0 + lane) * ld]) : mk<S>(0.0, 0.0);
-#pragma unroll
-        for (int j = 0; j < W; ++j) f[j] = shfl_c(mine, j);
-        S* __restrict__ ck = B + (size_t)k * ld;
-        // two rows per lane and two partial sums per row: four independent accumulation chains
-        for (int i = k + lane; i < n; i += 64) {
-          const int i2 = i + 32;
-          S a0 = mk<S>(0.0, 0.0), a1 = a0, c0 = a0, c1 = a0;
-#pragma unroll
-          for (int j = 0; j < W; j += 2) {
-            const S* pj = B + (size_t)(p0 + j) * ld;
-            const S* pk = pj + ld;
-            if (j < w) a0 = cfma(pj[i], f[j], a0);
-            if (j + 1 < w) a1 = cfma(pk[i], f[j + 1], a1);
-            if (i2 < n) {
-              if (j < w) c0 = cfma(pj[i2], f[j], c0);
-              if (j + 1 < w) c1 = cfma(pk[i2], f[j + 1], c1);
-            }
-          }
-          ck[i] = csub(ck[i], cadd(a0, a1));
-          if (i2 < n) ck[i2] = csub(ck[i2], cadd(c0, c1));
+    // 3. the trailing lower triangle, order m: columns a and m - 1 - a together have `len` or fewer
+    // blocks of 32 rows
+    const int k0 = p0 + w, m = n - k0;
+    if (m > 0) {
+      const int pairs = (m + 1) / 2, len = (m + 31) / 32 + 2;
+      for (int t = T.swrank(); t < pairs * len; t += T.wsize()) {
+        const int a = t / len;
+        int q = t - a * len, k = k0 + a;
+        const int na = (n - k + 31) / 32;
+        if (q >= na) {
+          q -= na;
+          k = n - 1 - a;
+          if (k == k0 + a) continue;  // the middle column of an odd order
         }
+        const int i = k + 32 * q + lane;
+        if (k + 32 * q >= n) continue;
+        S f[W];
+        const S mf = lane < W ? conjd(B[k + (size_t)(p0 + lane) * ld]) : mk<S>(0.0, 0.0);
+        S v[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) v[j] = i < n ? B[i + (size_t)(p0 + j) * ld] : mk<S>(0.0, 0.0);
+#pragma unroll
+        for (int j = 0; j < W; ++j) f[j] = shfl_c(mf, j);
+        S a0 = mk<S>(0.0, 0.0), a1 = a0;
+#pragma unroll
+        for (int j = 0; j < W; j += 2) {
+          a0 = cfma(v[j], f[j], a0);
+          a1 = cfma(v[j + 1], f[j + 1], a1);
+        }
+        if (i < n) B[i + (size_t)k * ld] = csub(B[i + (size_t)k * ld], cadd(a0, a1));
       }
       if (!T.sync()) return false;
     }
