@@ -53,6 +53,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 static_assert((kWarps & (kWarps - 1)) == 0, "the CTA reductions take a power-of-two warp count");
 
+__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 // 1 / x and 1 / sqrt(x) from the hardware's approximations (about 20 bits) by one third-order
 // iteration, r (1 + e + e^2) and r (1 + e / 2 + 3 e^2 / 8) with e the residual: within about one unit
 // in the last place.  The serial steps of the solver wait for these: three dependent operations of 64
@@ -138,10 +139,6 @@ __device__ __forceinline__ double cscale(double a, double s) { return a * s; }
 __device__ __forceinline__ double shfl_c(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 __device__ __forceinline__ double warp_sum_c(double v) { return warp_sum(v); }
 __device__ __forceinline__ double shfl_xor_c(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ double2 shfl_xor_c(double2 v, int o) {
-  return make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
-}
-
 __device__ __forceinline__ double re(double a) { return a; }
 __device__ __forceinline__ double re(double2 a) { return a.x; }
 __device__ __forceinline__ double im(double) { return 0.0; }
@@ -172,15 +169,17 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Control block of one grid-team solve (zeroed before the launch).
+constexpr int kCounters = 8;
 struct Ctl {
-  unsigned count;  // barrier arrivals (monotonic)
-  unsigned pad0;
+  unsigned count[kCounters][32];  // barrier arrivals (monotonic), each counter on a line of its own
   int err;  // 1: a barrier wait gave up
   int pad1;
   unsigned long long t[8];  // %globaltimer at the start and after each phase (measurement)
 };
 
 struct CtaTeam {
+  __device__ int cta() const { return 0; }
+  __device__ int ctas() const { return 1; }
   __device__ int rank() const { return threadIdx.x; }
   __device__ int swrank() const { return threadIdx.x >> 5; }  // rank for per-warp work
   __device__ int size() const { return blockDim.x; }
@@ -196,6 +195,8 @@ struct CtaTeam {
 // also order the CTAs' global writes.
 struct ClusterTeam {
   int crank, csize;
+  __device__ int cta() const { return crank; }
+  __device__ int ctas() const { return csize; }
   __device__ int rank() const { return crank * blockDim.x + threadIdx.x; }
   __device__ int swrank() const { return (threadIdx.x >> 5) * csize + crank; }
   __device__ int size() const { return csize * blockDim.x; }
@@ -211,6 +212,8 @@ struct GridTeam {
   Ctl* ctl;
   int* info;  // the pencil's status word: -1 when a barrier wait gave up
   unsigned long long limit_ns;
+  __device__ int cta() const { return blockIdx.x; }
+  __device__ int ctas() const { return gridDim.x; }
   __device__ int rank() const { return blockIdx.x * blockDim.x + threadIdx.x; }
   // rank for per-warp independent work, spread over the CTAs first so that n work items use every
   // SM's FP64 units instead of the first few CTAs'
@@ -221,39 +224,41 @@ struct GridTeam {
   __device__ void stamp(int k) const {
     if (rank() == 0) ctl->t[k] = global_ns();
   }
-  // Grid barrier (all CTAs are resident: cooperative launch).  The counter only grows: barrier
-  // number b (counted by every thread in its own copy of the team) is passed once it reaches
-  // b x gridDim.x.  Each CTA arrives with one release add, which makes the writes of all its
-  // threads (ordered before it by __syncthreads) visible to any thread that acquires the counter,
-  // and waits with acquire loads in a bounded spin.  Returns false when the solve has been
+  // Grid barrier (all CTAs are resident: cooperative launch).  The counters only grow: barrier number b
+  // (counted by every thread in its own copy of the team) is passed once every counter holds b arrivals
+  // of each of its CTAs (those with its number modulo kCounters: a single counter takes 150 arrivals
+  // one after another).  Each CTA arrives with one release add, which makes the writes of all its
+  // threads (ordered before it by __syncthreads) visible to any thread that acquires the counter;
+  // eight lanes acquire one counter each, in a bounded spin.  Returns false when the solve has been
   // abandoned.
   mutable unsigned epoch = 0;
   __device__ bool sync() const {
     __shared__ int s_ok;
     __syncthreads();
-    const unsigned target = ++epoch * gridDim.x;
-    if (threadIdx.x == 0) {
-      cuda::atomic_ref<unsigned, cuda::thread_scope_device> cnt(ctl->count);
+    ++epoch;
+    if (threadIdx.x < 32) {
+      const int c = threadIdx.x & (kCounters - 1);
+      cuda::atomic_ref<unsigned, cuda::thread_scope_device> cnt(ctl->count[c][0]);
       cuda::atomic_ref<int, cuda::thread_scope_device> err(ctl->err);
-      int ok = err.load(cuda::memory_order_relaxed) == 0;
+      const unsigned target = epoch * ((gridDim.x + kCounters - 1 - c) / kCounters);
+      int ok = __all_sync(0xffffffffu, err.load(cuda::memory_order_relaxed) == 0);
       if (ok) {
-        cnt.fetch_add(1u, cuda::memory_order_release);
+        if (threadIdx.x < kCounters && (blockIdx.x & (kCounters - 1)) == threadIdx.x)
+          cnt.fetch_add(1u, cuda::memory_order_release);
         const unsigned long long t0 = global_ns();
         unsigned spins = 0;
-        while (cnt.load(cuda::memory_order_acquire) < target) {
-          if (err.load(cuda::memory_order_relaxed)) {
-            ok = 0;
-            break;
-          }
-          if ((++spins & 63u) == 0 && global_ns() - t0 > limit_ns) {
-            err.store(1, cuda::memory_order_relaxed);
-            *info = -1;
-            ok = 0;
-            break;
+        while (!__all_sync(0xffffffffu, threadIdx.x >= kCounters || cnt.load(cuda::memory_order_acquire) >= target)) {
+          if ((++spins & 63u) == 0) {
+            const bool late = global_ns() - t0 > limit_ns;
+            if (__any_sync(0xffffffffu, late || err.load(cuda::memory_order_relaxed))) {
+              if (threadIdx.x == 0 && err.exchange(1, cuda::memory_order_relaxed) == 0) *info = -1;
+              ok = 0;
+              break;
+            }
           }
         }
       }
-      s_ok = ok;
+      if (threadIdx.x == 0) s_ok = ok;
     }
     __syncthreads();
     return s_ok != 0;
@@ -273,8 +278,9 @@ struct Pencil {
   S* R;         // n x n (ld n): reduction workspace, then the reflector vectors
   double* Z;    // n x n (ld n): eigenvectors of T
   double* wk;   // 6 n^2 doubles: inverse-iteration arrays
-  double* vec;  // 9 n + 8 doubles: d, e, tau (S), p (2 x S), 1/L_jj
+  double* vec;  // 11 n + 8 doubles: d, e, tau (S), p (2 x S), 1/L_jj, q (2)
   int smem_cols;  // 1: the launch gives every warp n words of S of dynamic shared memory
+  int resident;   // 1: and the tridiagonalisation its CTA's columns (beside its three vectors)
   double2* outA;  // the caller's A and B (complex128; the same as A and B when S = double2)
   double2* outB;
   int ldoa, ldob;
@@ -604,7 +610,7 @@ __device__ bool reduce_standard(const Team& T, const Pencil<S>& P) {
 
 // ---- phase 3: Householder tridiagonalisation ------------------------------------------------------
 // vec layout: d[n], e[n], tau[2n] (n words of S), p[4n] (2 n words of S: p of two consecutive
-// steps), 1/L_jj[n]
+// steps), 1/L_jj[n], q[2n] (Re conj(C v) v of two consecutive steps, complex pencils)
 template <class S>
 __device__ __forceinline__ double* vd(const Pencil<S>& P) { return P.vec; }
 template <class S>
@@ -613,6 +619,8 @@ template <class S>
 __device__ __forceinline__ S* vtau(const Pencil<S>& P) { return reinterpret_cast<S*>(P.vec + 2 * P.n); }
 template <class S>
 __device__ __forceinline__ S* vp(const Pencil<S>& P) { return reinterpret_cast<S*>(P.vec + 4 * P.n); }
+template <class S>
+__device__ __forceinline__ double* vq(const Pencil<S>& P) { return P.vec + 9 * P.n; }
 
 // Sum over the CTA (every thread passes a value; every thread gets the same total, reduced in a
 // fixed order so that all CTAs of a grid team obtain bit-identical results).
@@ -645,18 +653,20 @@ __device__ S cta_reflector(const Pencil<S>& P, int j, S* sx, bool writer) {
   for (int i = j + 2 + tid; i < n; i += blockDim.x) s = abs2_acc(sx[i], s);
   s = cta_sum_c(s);  // (its barriers also publish sx)
   if (tid == 0) {
+    // one thread's chain: the signs and the zero test on the bits, not in FP64
     const S alpha = sx[j + 1];
     double beta;
     S tj = mk<S>(0.0, 0.0), vs = mk<S>(0.0, 0.0);
-    if (s == 0.0 && im(alpha) == 0.0) {
+    if (((unsigned long long)dbits(s) << 1) == 0 && im(alpha) == 0.0) {
       beta = re(alpha);  // nothing to annihilate: H = I
     } else {
       const double a2 = abs2_acc(alpha, s);
       const double ra = fast_rsqrt(a2), an = sqrt_from(a2, ra);
-      beta = re(alpha) >= 0.0 ? -an : an;
-      const double rb = re(alpha) >= 0.0 ? -ra : ra;
-      tj = mk<S>((beta - re(alpha)) * rb, -im(alpha) * rb);
-      vs = cinv(csub(alpha, mk<S>(beta, 0.0)));  // v_i = x_i / (alpha - beta)
+      const bool pos = dbits(re(alpha)) >= 0;
+      beta = pos ? -an : an;
+      const S diff = mk<S>(re(alpha) - beta, im(alpha));  // v_i = x_i / (alpha - beta)
+      vs = cinv(diff);
+      tj = cscale(diff, pos ? ra : -ra);  // (beta - alpha) / beta
     }
     s_tau = tj;
     s_vs = vs;
@@ -677,20 +687,112 @@ __device__ S cta_reflector(const Pencil<S>& P, int j, S* sx, bool writer) {
   return tj;
 }
 
+// One pass over this CTA's columns k >= kmin, rows >= r0, by all its warps: with UPDATE the rank-2 update
+// C <- C - v w^H - w v^H; then u_k = (column k)^H vn (C is Hermitian: row k of C vn), from which
+// pn[k] = tn u_k and, for complex pencils, qn[k] = Re conj(u_k) vn_k are stored.  Column k belongs to CTA
+// k mod G.  The columns' blocks of 32 rows, one column after another, are cut into equal shares for
+// the warps, so that none of the SM's FP64 quarters idles when few columns are left; the sums of a
+// column that is cut go through shared memory.  kout: the column whose update goes to global memory
+// (the next one to be eliminated, which every CTA reads); the others stay where they are.
+template <bool UPDATE, class Team, class S>
+__device__ void column_pass(const Team& T, const Pencil<S>& P, S* cols, bool resident, int kmin, int r0, int kout,
+                            const S* sv, const S* sw, const S* sn, S tn, S* __restrict__ pn, double* __restrict__ qn) {
+  __shared__ S s_start[kWarps], s_head[kWarps];
+  __shared__ int s_k[kWarps], s_last[kWarps];
+  const int n = P.n, G = T.ctas(), cta = T.cta();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int slots = cta < n ? (n - cta + G - 1) / G : 0;
+  const int s0 = kmin > cta ? (kmin - cta + G - 1) / G : 0;
+  const int cnt = max(slots - s0, 0), nch = (n - r0 + 31) / 32, tot = cnt * nch;
+  auto put = [&](int k, S u) {
+    pn[k] = cmul(tn, u);
+    if constexpr (sizeof(S) == sizeof(double2)) qn[k] = re(cmulc(u, sn[k]));
+  };
+  int lo = warp * tot / kWarps;
+  const int hi = (warp + 1) * tot / kWarps;
+  if (lane == 0) {
+    s_k[warp] = -1;
+    s_head[warp] = mk<S>(0.0, 0.0);  // (a share may be empty)
+  }
+  while (lo < hi) {
+    const int c = lo / nch, ch = lo - c * nch, end = min(nch, ch + hi - lo);
+    const int k = (s0 + c) * G + cta;
+    S cvk = mk<S>(0.0, 0.0), cwk = cvk;
+    if (UPDATE) {
+      cvk = conjd(sv[k]);
+      cwk = conjd(sw[k]);
+    }
+    S* gk = P.A + (size_t)k * P.lda;
+    S* ck = resident ? cols + (size_t)(s0 + c) * n : gk;
+    S* dst = k == kout ? gk : ck;
+    S acc = mk<S>(0.0, 0.0);
+    const int iend = min(n, r0 + 32 * end);
+    int i = r0 + 32 * ch + lane;
+    for (; i + 96 < iend; i += 128) {
+      S a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = ck[i + 32 * u];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = i + 32 * u;
+        if (UPDATE) {
+          a[u] = cfms(sw[r], cvk, cfms(sv[r], cwk, a[u]));
+          dst[r] = a[u];
+        }
+        acc = cfmac(a[u], sn[r], acc);
+      }
+    }
+    for (; i < iend; i += 32) {
+      S a = ck[i];
+      if (UPDATE) {
+        a = cfms(sw[i], cvk, cfms(sv[i], cwk, a));
+        dst[i] = a;
+      }
+      acc = cfmac(a, sn[i], acc);
+    }
+    acc = warp_sum_c(acc);
+    if (lane == 0) {
+      if (ch == 0 && end == nch) {
+        put(k, acc);
+      } else if (ch == 0) {  // to be continued by the next warps
+        s_start[warp] = acc;
+        s_k[warp] = k;
+        s_last[warp] = ((c + 1) * nch * kWarps - 1) / tot;  // the warp with the column's last block
+      } else {
+        s_head[warp] = acc;
+      }
+    }
+    lo += end - ch;
+  }
+  __syncthreads();
+  if (tid < kWarps && s_k[tid] >= 0) {
+    S u = s_start[tid];
+    for (int q = tid + 1; q <= s_last[tid]; ++q) u = cadd(u, s_head[q]);
+    put(s_k[tid], u);
+  }
+}
+
 // One team barrier per column.  Step j applies reflector j (v_j, tau_j, and p_j = tau_j C v_j from
-// the previous step) to the trailing matrix: gamma = -(tau_j / 2) p_j^H v_j, w = p_j + gamma v_j,
+// the previous step) to the trailing matrix: gamma = -(tau_j / 2) p_j^H v_j (real: v_j^H C v_j is, so a
+// complex pencil adds up the real parts q_j that come with p_j), w = p_j + gamma v_j,
 // C <- C - v w^H - w v^H.  Every CTA forms column j+1 of the updated matrix and reflector j+1 from
-// it in shared memory (the same values in every CTA), then each warp updates its columns k >= j+2
-// and, in the same pass over the column, accumulates p_{j+1}[k] = tau_{j+1} (column k)^H v_{j+1}
-// (C is Hermitian, so that is row k of C v_{j+1}).  Rows < j+2 of those columns are never read
-// again and are not updated.  p of consecutive steps alternate between two buffers, so that a
-// CTA still reading p_j never meets the p_{j+1} that faster CTAs write.
-// sbuf: 3 n words of S of shared memory per CTA (v_j, w and v_{j+1}, indexed by row).
+// it in shared memory (the same values in every CTA), then updates its columns k >= j+2
+// and, in the same pass over the column, accumulates p_{j+1}[k] (column_pass).  Rows < j+2 of those
+// columns are never read again and are not updated.  p of consecutive steps alternate between two
+// buffers, so that a CTA still reading p_j never meets the p_{j+1} that faster CTAs write.
+// What bounds it: per step two barrier and L2 round trips, about 30 dependent FP64 operations of 64 to
+// 100 cycles each, and the update's FP64 instructions.  The CTA's columns therefore stay in shared
+// memory when they fit, and the update is spread evenly over the SM (column_pass).  Cycles per step
+// (load, reflector and barrier / update), order 564 complex: 14.6k / 7.7k (columns in L2, a warp a column: 15.9k
+// / 12.1k); 1127 real: 11.9k / 7.5k (13.9k / 8.8k).
+// sbuf: 3 n words of S of shared memory per CTA (v_j, w and v_{j+1}, indexed by row), then, when
+// P.resident, the CTA's columns.
 template <class Team, class S>
 __device__ bool tridiagonalise(const Team& T, const Pencil<S>& P, S* sbuf) {
+  constexpr bool kComplex = sizeof(S) == sizeof(double2);
   const int n = P.n, la = P.lda;
   S* A = P.A;
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x;
   const bool writer = T.rank() < (int)blockDim.x;  // the first CTA writes d, e, tau and R
   if (n == 1) {
     if (T.rank() == 0) vd(P)[0] = re(A[0]);
@@ -699,40 +801,44 @@ __device__ bool tridiagonalise(const Team& T, const Pencil<S>& P, S* sbuf) {
   S* sv = sbuf;
   S* sw = sbuf + n;
   S* sn = sbuf + 2 * n;
+  S* cols = sbuf + 3 * n;
+  const bool resident = P.resident != 0;
+  if (resident) {
+    for (int s = 0, k = T.cta(); k < n; ++s, k += T.ctas())
+      for (int i = tid; i < n; i += blockDim.x) cols[(size_t)s * n + i] = A[i + (size_t)k * la];
+  }
   // reflector 0 from column 0, and p_0 = tau_0 C v_0 (rows 1..n-1)
   for (int i = 1 + tid; i < n; i += blockDim.x) sv[i] = A[i];
   if (writer && tid == 0) vd(P)[0] = re(A[0]);
   S tau = cta_reflector(P, 0, sv, writer);
-  {
-    S* __restrict__ p0 = vp(P);
-    for (int k = 1 + T.swrank(); k < n; k += T.wsize()) {
-      const S* __restrict__ ck = A + (size_t)k * la;
-      S acc = mk<S>(0.0, 0.0);
-      for (int i = 1 + lane; i < n; i += 32) acc = cfmac(ck[i], sv[i], acc);
-      acc = warp_sum_c(acc);
-      if (lane == 0) p0[k] = cmul(tau, acc);
-    }
-  }
+  column_pass<false>(T, P, cols, resident, 1, 1, -1, sv, sv, sv, tau, vp(P), vq(P));
   if (!T.sync()) return false;
   for (int j = 0; j <= n - 2; ++j) {
-    const S* __restrict__ pj = vp(P) + (size_t)(j & 1) * n;
-    S* __restrict__ pn = vp(P) + (size_t)((j + 1) & 1) * n;
+    const S* pj = vp(P) + (size_t)(j & 1) * n;
+    const double* qj = vq(P) + (size_t)(j & 1) * n;
     // p_j and column j+1 of C are read together (one round trip to L2), staged raw in sw and sn;
     // then w = p_j + gamma v_j and column j+1 of the updated matrix, x - v conj(w_{j+1}) - w (the
     // entry of v_j in row j+1 is 1), each thread on its own rows
-    const S* __restrict__ c1 = A + (size_t)(j + 1) * la;
-    S g = mk<S>(0.0, 0.0);
+    const S* c1 = A + (size_t)(j + 1) * la;
+    double g = 0.0;
     for (int i = j + 1 + tid; i < n; i += blockDim.x) {
       const S pi = pj[i];
+      if constexpr (kComplex) g += qj[i];
+      else g = fma(pi, sv[i], g);
       sn[i] = c1[i];
       sw[i] = pi;
-      g = cfmac(pi, sv[i], g);
     }
     g = cta_sum_c(g);
-    const S gamma = cscale(cmul(tau, g), -0.5);
-    const S cw1 = conjd(cadd(pj[j + 1], gamma));
+    double gamma;  // -|tau|^2 v^H C v / 2
+    if constexpr (kComplex) gamma = -0.5 * g * abs2_acc(tau, 0.0);
+    else gamma = -0.5 * g * tau;
+    auto wof = [&](S p, S v) {
+      if constexpr (kComplex) return make_double2(fma(gamma, v.x, p.x), fma(gamma, v.y, p.y));
+      else return fma(gamma, v, p);
+    };
+    const S cw1 = conjd(wof(pj[j + 1], mk<S>(1.0, 0.0)));
     for (int i = j + 1 + tid; i < n; i += blockDim.x) {
-      const S wi = cfma(gamma, sv[i], sw[i]);
+      const S wi = wof(sw[i], sv[i]);
       const S x = csub(cfms(sv[i], cw1, sn[i]), wi);
       sw[i] = wi;
       sn[i] = x;
@@ -740,33 +846,8 @@ __device__ bool tridiagonalise(const Team& T, const Pencil<S>& P, S* sbuf) {
     }
     if (j + 1 <= n - 2) {
       const S tn = cta_reflector(P, j + 1, sn, writer);
-      // columns k >= j+2: rank-2 update of rows j+2..n-1 fused with p_{j+1}[k]
-      for (int k = j + 2 + T.swrank(); k < n; k += T.wsize()) {
-        const S cvk = conjd(sv[k]), cwk = conjd(sw[k]);
-        S* __restrict__ ck = A + (size_t)k * la;
-        S acc = mk<S>(0.0, 0.0), acc2 = acc;  // two partial sums: shorter dependent chains
-        int i = j + 2 + lane;
-        for (; i + 96 < n; i += 128) {
-          S a[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) a[u] = ck[i + 32 * u];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int r = i + 32 * u;
-            a[u] = cfms(sw[r], cvk, cfms(sv[r], cwk, a[u]));
-            ck[r] = a[u];
-            if (u & 1) acc2 = cfmac(a[u], sn[r], acc2);
-            else acc = cfmac(a[u], sn[r], acc);
-          }
-        }
-        for (; i < n; i += 32) {
-          const S a = cfms(sw[i], cvk, cfms(sv[i], cwk, ck[i]));
-          ck[i] = a;
-          acc = cfmac(a, sn[i], acc);
-        }
-        acc = warp_sum_c(cadd(acc, acc2));
-        if (lane == 0) pn[k] = cmul(tn, acc);
-      }
+      column_pass<true>(T, P, cols, resident, j + 2, j + 2, j + 2, sv, sw, sn, tn, vp(P) + (size_t)((j + 1) & 1) * n,
+                        vq(P) + (size_t)((j + 1) & 1) * n);
       tau = tn;
     }
     if (!T.sync()) return false;
@@ -796,7 +877,6 @@ struct Sturm {
   int count, ve;
   double v;
 };
-__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 // |x| as an integer: ordered like |x| for all non-NaN doubles
 __device__ __forceinline__ unsigned long long dmag(double x) {
   return (unsigned long long)dbits(x) & 0x7FFFFFFFFFFFFFFFull;
@@ -1301,11 +1381,11 @@ __global__ void __launch_bounds__(kThreads, 2) hegv_cluster_kernel(const Pencil<
 size_t pad32(size_t x) { return (x + 31) & ~(size_t)31; }
 
 // Workspace doubles of one pencil, each array padded to 32 doubles: complex, R (complex n^2);
-// real, the compact A, B and R (n^2 each); then Z (n^2), wk (6 n^2) and vec (9 n + 8).
+// real, the compact A, B and R (n^2 each); then Z (n^2), wk (6 n^2) and vec (11 n + 8).
 size_t work_doubles(int n, bool real) {
   const size_t nn = (size_t)n * n;
   const size_t own = real ? 3 * pad32(nn) : pad32(2 * nn);
-  return own + pad32(nn) + pad32(6 * nn) + pad32(9 * (size_t)n + 8);
+  return own + pad32(nn) + pad32(6 * nn) + pad32(11 * (size_t)n + 8);
 }
 
 template <class S>
@@ -1338,6 +1418,7 @@ Pencil<S> make_pencil(double2* A, int lda, double2* B, int ldb, double* w, int* 
   P.wk = P.Z + pad32(nn);
   P.vec = P.wk + pad32(6 * nn);
   P.smem_cols = 0;
+  P.resident = 0;
   return P;
 }
 
@@ -1353,6 +1434,11 @@ size_t col_smem_bytes(int n, size_t ws) {
 size_t dyn_smem_bytes(int n, size_t ws) {
   const size_t chol = ws == 8 ? chol_smem<double>() : chol_smem<double2>();
   return std::max({col_smem_bytes(n, ws), (size_t)3 * std::max(n, 1) * ws, chol});
+}
+// The tridiagonalisation's vectors and the columns of a CTA of a team of `ctas`, 0 when above `limit`.
+size_t resident_smem_bytes(int n, size_t ws, int ctas, size_t limit) {
+  const size_t b = ws * (size_t)std::max(n, 1) * (3 + (std::max(n, 1) + ctas - 1) / ctas);
+  return b <= limit ? b : 0;
 }
 constexpr int kMaxN = 4608;  // 3 n complex words must fit in shared memory (221 KB)
 
@@ -1375,12 +1461,17 @@ void launch_cta(kss_ctx ctx, std::vector<Pencil<S>>& small, size_t items_offset,
   cudaStream_t st = ctx->stream;
   int nmax = 1;
   for (const auto& P : small) nmax = std::max(nmax, P.n);
-  const size_t sm = dyn_smem_bytes(nmax, sizeof(S));
-  for (auto& P : small) P.smem_cols = col_smem_bytes(nmax, sizeof(S)) ? 1 : 0;
+  const int csize = cluster_size(ctx, (int)small.size(), nmax);
+  // two CTAs share an SM (their registers): half of its shared memory each
+  const size_t res = resident_smem_bytes(nmax, sizeof(S), csize, 110u * 1024u);
+  const size_t sm = std::max(dyn_smem_bytes(nmax, sizeof(S)), res);
+  for (auto& P : small) {
+    P.smem_cols = col_smem_bytes(nmax, sizeof(S)) ? 1 : 0;
+    P.resident = res ? 1 : 0;
+  }
   Pencil<S>* d_items = reinterpret_cast<Pencil<S>*>(static_cast<char*>(ctx->dense_items.p) + items_offset);
   KSS_CHECK_CUDA(cudaMemcpyAsync(d_items, small.data(), small.size() * sizeof(Pencil<S>), cudaMemcpyHostToDevice, st));
   ProfScope ps(ctx, prof_register(name));
-  const int csize = cluster_size(ctx, (int)small.size(), nmax);
   if (csize == 1) {
     KSS_CHECK_CUDA(cudaFuncSetAttribute(hegv_cta_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     hegv_cta_kernel<S><<<(unsigned)small.size(), kThreads, sm, st>>>(d_items, (int)small.size());
@@ -1406,12 +1497,15 @@ template <class S>
 void launch_grid(kss_ctx ctx, Pencil<S> P, const char* name) {
   cudaStream_t st = ctx->stream;
   const int n = P.n;
-  const size_t sm = dyn_smem_bytes(n, sizeof(S));
+  const int want = std::max(1, std::min((n + 3) / 4, ctx->nsm > 0 ? ctx->nsm : 1));
+  const size_t res = resident_smem_bytes(n, sizeof(S), want, 220u * 1024u);
+  const size_t sm = std::max(dyn_smem_bytes(n, sizeof(S)), res);
   KSS_CHECK_CUDA(cudaFuncSetAttribute(hegv_grid_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   int per_sm = 0;
   KSS_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hegv_grid_kernel<S>, kThreads, sm));
   const int coop = std::max(1, per_sm) * std::max(1, ctx->nsm);
-  const int G = std::max(1, std::min({(n + 3) / 4, ctx->nsm > 0 ? ctx->nsm : 1, coop}));
+  const int G = std::min(want, coop);
+  P.resident = res && G == want ? 1 : 0;
   ctx->dense_ctl.ensure(sizeof(Ctl));
   KSS_CHECK_CUDA(cudaMemsetAsync(ctx->dense_ctl.p, 0, sizeof(Ctl), st));
   P.smem_cols = col_smem_bytes(n, sizeof(S)) ? 1 : 0;
