@@ -28,8 +28,8 @@
 // a cluster of up to eight per pencil of a batch (barrier = the cluster's), or a whole cooperative grid
 // (one large pencil, barrier = a grid barrier of this file with a bounded wait).  Work that is independent per
 // column (the triangular solves, the reflector applications, the inverse iterations) needs no
-// team barrier: one warp owns a column and each lane owns the rows r = lane (mod 32), so values
-// written by one lane are read back only by that lane and everything else travels by shuffles.
+// team barrier: one warp owns a column, and what its lanes exchange goes by shuffles or behind a
+// warp barrier.
 // The barrier count is about n + n/8 per pencil (one per tridiagonalisation step, two per 16-column
 // Cholesky panel).
 //
@@ -491,30 +491,38 @@ __device__ __forceinline__ void forward_subst(const S* __restrict__ L, const dou
       if (lane > i && lane < bn) xl = cfms(L[(size_t)(b0 + i) * ld + b0 + lane], xi, xl);
     }
     if (lane < bn) x[b0 + lane] = xl;
-    // rows below, two 32-row blocks per pass and two partial sums per row (four independent
-    // accumulation chains per lane; every broadcast x_i serves both blocks)
+    // rows below, two 32-row blocks per pass (every broadcast x_i serves both), eight columns of L
+    // loaded ahead of their products: a warp has a quarter of the SM's FP64 pipe nearly to itself, and
+    // what it waits for memory is lost
     for (int r0 = b0 + bn; r0 < n; r0 += 64) {
       const int r = r0 + lane, r2 = r + 32;
+      const bool two = r0 + 32 < n;
+      const S* lp = L + (size_t)b0 * ld + r;
       S a0 = mk<S>(0.0, 0.0), a1 = a0, c0 = a0, c1 = a0;
       int i = 0;
-      for (; i + 1 < bn; i += 2) {
-        const S xi = shfl_c(xl, i), xj = shfl_c(xl, i + 1);
-        const S* li = L + (size_t)(b0 + i) * ld;
-        const S* lj = li + ld;
-        if (r < n) {
-          a0 = cfma(li[r], xi, a0);
-          a1 = cfma(lj[r], xj, a1);
+#pragma unroll 2
+      for (; i + 8 <= bn; i += 8) {
+        S l[8], m[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          l[u] = r < n ? lp[(size_t)(i + u) * ld] : mk<S>(0.0, 0.0);
+          m[u] = r2 < n ? lp[(size_t)(i + u) * ld + 32] : mk<S>(0.0, 0.0);
         }
-        if (r2 < n) {
-          c0 = cfma(li[r2], xi, c0);
-          c1 = cfma(lj[r2], xj, c1);
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+          const S xi = shfl_c(xl, i + u), xj = shfl_c(xl, i + u + 1);
+          a0 = cfma(l[u], xi, a0);
+          a1 = cfma(l[u + 1], xj, a1);
+          if (two) {
+            c0 = cfma(m[u], xi, c0);
+            c1 = cfma(m[u + 1], xj, c1);
+          }
         }
       }
-      if (i < bn) {
+      for (; i < bn; ++i) {
         const S xi = shfl_c(xl, i);
-        const S* li = L + (size_t)(b0 + i) * ld;
-        if (r < n) a0 = cfma(li[r], xi, a0);
-        if (r2 < n) c0 = cfma(li[r2], xi, c0);
+        if (r < n) a0 = cfma(lp[(size_t)i * ld], xi, a0);
+        if (r2 < n) c0 = cfma(lp[(size_t)i * ld + 32], xi, c0);
       }
       if (r < n) x[r] = csub(x[r], cadd(a0, a1));
       if (r2 < n) x[r2] = csub(x[r2], cadd(c0, c1));
@@ -539,25 +547,34 @@ __device__ __forceinline__ void backward_subst_h(const S* __restrict__ L, const 
       if (lane < i) xl = csub(xl, cmulc(L[(size_t)(b0 + lane) * ld + b0 + i], xi));
     }
     if (lane < bn) x[b0 + lane] = xl;
-    // rows above, two 32-row blocks per pass and two partial sums per row
+    // rows above, as below in the forward form (lane r reads the contiguous segment of column r)
     for (int r0 = 0; r0 < b0; r0 += 64) {
       const int r = r0 + lane, r2 = r + 32;
+      const bool two = r0 + 32 < b0;
       S a0 = mk<S>(0.0, 0.0), a1 = a0, c0 = a0, c1 = a0;
       const S* lr = L + (size_t)r * ld + b0;
       const S* lr2 = lr + (size_t)32 * ld;
       int t = 0;
-      for (; t + 1 < bn; t += 2) {
-        const S xt = shfl_c(xl, t), xu = shfl_c(xl, t + 1);
-        if (r < b0) {
-          a0 = cfmac(lr[t], xt, a0);
-          a1 = cfmac(lr[t + 1], xu, a1);
+#pragma unroll 2
+      for (; t + 8 <= bn; t += 8) {
+        S l[8], m[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          l[u] = r < b0 ? lr[t + u] : mk<S>(0.0, 0.0);
+          m[u] = r2 < b0 ? lr2[t + u] : mk<S>(0.0, 0.0);
         }
-        if (r2 < b0) {
-          c0 = cfmac(lr2[t], xt, c0);
-          c1 = cfmac(lr2[t + 1], xu, c1);
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+          const S xt = shfl_c(xl, t + u), xu = shfl_c(xl, t + u + 1);
+          a0 = cfmac(l[u], xt, a0);
+          a1 = cfmac(l[u + 1], xu, a1);
+          if (two) {
+            c0 = cfmac(m[u], xt, c0);
+            c1 = cfmac(m[u + 1], xu, c1);
+          }
         }
       }
-      if (t < bn) {
+      for (; t < bn; ++t) {
         const S xt = shfl_c(xl, t);
         if (r < b0) a0 = cfmac(lr[t], xt, a0);
         if (r2 < b0) c0 = cfmac(lr2[t], xt, c0);
@@ -1314,16 +1331,59 @@ __device__ bool back_transform(const Team& T, const Pencil<S>& P, S* smem) {
     const double* zc = P.Z + (size_t)c * n;
     for (int i = lane; i < n; i += 32) vc[i] = mk<S>(zc[i], 0.0);
     __syncwarp();
-    // V = H_0 H_1 ... H_{n-2} Z: reflector j (rows j+1..n-1, stored in column j of R) applied last-first
+    // V = H_0 H_1 ... H_{n-2} Z: reflector j (rows j+1..n-1, stored in column j of R) applied last-first,
+    // U 32-row blocks loaded ahead of their products; the first U of the next reflector while this one's
+    // sum goes around the warp
+    constexpr int U = sizeof(S) == sizeof(double) ? 8 : 4;
+    S nx[U];
+    auto first = [&](int j) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = j + 1 + lane + 32 * u;
+        nx[u] = j >= 0 && i < n ? P.R[(size_t)j * n + i] : mk<S>(0.0, 0.0);
+      }
+    };
+    first(n - 2);
     for (int j = n - 2; j >= 0; --j) {
       const S tj = tau[j];
-      if (re(tj) == 0.0 && im(tj) == 0.0) continue;
-      const S* __restrict__ rj = P.R + (size_t)j * n;
-      const int r0 = j + 1 + ((lane - j - 1) & 31);
-      S s = mk<S>(0.0, 0.0);
-      for (int i = r0; i < n; i += 32) s = cfmac(rj[i], vc[i], s);
-      s = cmul(tj, warp_sum_c(s));
-      for (int i = r0; i < n; i += 32) vc[i] = cfms(rj[i], s, vc[i]);
+      const S* rj = P.R + (size_t)j * n;
+      S h[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) h[u] = nx[u];
+      S s = mk<S>(0.0, 0.0), s2 = s;
+      const int i0 = j + 1 + lane, m = n - 1 - j;  // rows of the reflector
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (32 * u < m) {
+          if (u & 1) s2 = cfmac(h[u], i0 + 32 * u < n ? vc[i0 + 32 * u] : mk<S>(0.0, 0.0), s2);
+          else s = cfmac(h[u], i0 + 32 * u < n ? vc[i0 + 32 * u] : mk<S>(0.0, 0.0), s);
+        }
+      for (int b = 32 * U; b < m; b += 32 * U) {
+        S l[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) l[u] = i0 + b + 32 * u < n ? rj[i0 + b + 32 * u] : mk<S>(0.0, 0.0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (b + 32 * u < m) {
+            const S v = i0 + b + 32 * u < n ? vc[i0 + b + 32 * u] : mk<S>(0.0, 0.0);
+            if (u & 1) s2 = cfmac(l[u], v, s2);
+            else s = cfmac(l[u], v, s);
+          }
+      }
+      first(j - 1);
+      s = cmul(tj, warp_sum_c(cadd(s, s2)));
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (32 * u < m && i0 + 32 * u < n) vc[i0 + 32 * u] = cfms(h[u], s, vc[i0 + 32 * u]);
+      for (int b = 32 * U; b < m; b += 32 * U) {
+        S l[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) l[u] = i0 + b + 32 * u < n ? rj[i0 + b + 32 * u] : mk<S>(0.0, 0.0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (b + 32 * u < m && i0 + b + 32 * u < n) vc[i0 + b + 32 * u] = cfms(l[u], s, vc[i0 + b + 32 * u]);
+      }
+      __syncwarp();  // (the next reflector's rows lie one lane further)
     }
     __syncwarp();
     backward_subst_h(P.B, vrdiag(P), P.ldb, n, vc);
