@@ -115,37 +115,51 @@ template <typename C, typename T> __device__ __forceinline__ C scaled(T a, C b) 
   return r;
 }
 
-// Single precision: both components in one packed instruction where the operation does not mix them
-// (the FP32 passes are bound by issue slots; middle pass of 564 bands at 96 points 1.78 -> 1.70 ms).  Swapped components stay with the scalar operations,
-// where the swap is free.
-union Pair {
-  float2 f;
-  unsigned long long u;
+// Single precision with both components in one packed instruction where the operation does not mix them
+// (the passes that use it are bound by issue slots; middle pass of 564 bands at 96 points 1.78 -> 1.70
+// ms).  Swapped components stay with the scalar operations, where the swap is free.  A type of its own:
+// it rounds differently in the last bit where the compiler contracts the scalar form across additions,
+// and the single-precision density, delivered in FP64, keeps the scalar form.
+struct alignas(8) F2 {
+  float x, y;
+  F2() = default;
+  __device__ __forceinline__ F2(float a, float b) : x(a), y(b) {}
+  __device__ __forceinline__ F2(float2 a) : x(a.x), y(a.y) {}
+  __device__ __forceinline__ operator float2() const { return make_float2(x, y); }
 };
-__device__ __forceinline__ float2 add(float2 a, float2 b) {
-  Pair p{a}, q{b}, r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(p.u), "l"(q.u));
-  return r.f;
+template <typename C> struct Packed { using T = C; };
+template <> struct Packed<float2> { using T = F2; };
+__device__ __forceinline__ unsigned long long bits2(F2 a) {
+  return (unsigned long long)__float_as_uint(a.y) << 32 | __float_as_uint(a.x);
 }
-__device__ __forceinline__ float2 sub(float2 a, float2 b) {
-  Pair p{a}, q{b}, r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(p.u), "l"(q.u));
-  return r.f;
+__device__ __forceinline__ F2 from_bits2(unsigned long long u) {
+  return F2(__uint_as_float((unsigned)u), __uint_as_float((unsigned)(u >> 32)));
 }
-__device__ __forceinline__ float2 axpy(float a, float2 b, float2 c) {
-  Pair m{make_float2(a, a)}, p{b}, q{c}, r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.u) : "l"(m.u), "l"(p.u), "l"(q.u));
-  return r.f;
+__device__ __forceinline__ F2 add(F2 a, F2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+  return from_bits2(r);
 }
-__device__ __forceinline__ float2 scaled(float a, float2 b) {
-  Pair m{make_float2(a, a)}, p{b}, r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(m.u), "l"(p.u));
-  return r.f;
+__device__ __forceinline__ F2 sub(F2 a, F2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+  return from_bits2(r);
 }
-__device__ __forceinline__ float2 add_i(float2 a, float2 d, float s) {
-  return s > 0.f ? make_float2(a.x - d.y, a.y + d.x) : make_float2(a.x + d.y, a.y - d.x);
+__device__ __forceinline__ F2 axpy(float a, F2 b, F2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(bits2(F2(a, a))), "l"(bits2(b)), "l"(bits2(c)));
+  return from_bits2(r);
 }
-__device__ __forceinline__ float2 sub_i(float2 a, float2 d, float s) { return add_i(a, d, -s); }
+__device__ __forceinline__ F2 scaled(float a, F2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(F2(a, a))), "l"(bits2(b)));
+  return from_bits2(r);
+}
+__device__ __forceinline__ F2 add_i(F2 a, F2 d, float s) {
+  return s > 0.f ? F2(a.x - d.y, a.y + d.x) : F2(a.x + d.y, a.y - d.x);
+}
+__device__ __forceinline__ F2 sub_i(F2 a, F2 d, float s) { return add_i(a, d, -s); }
+__device__ __forceinline__ F2 mul(F2 a, float2 b) { return mul(a, F2(b)); }
 
 // ---- fixed point (fx64.cuh): the same codelets on 64-bit integers ----------------------------
 // (a c) for a compile-time factor c = kcos62(M, N) (SIN = false) or ksin62(M, N), in units of
@@ -243,8 +257,8 @@ __device__ __forceinline__ void rdft_base(C* v, T s) {
       const T s1 = (T)0.95105651629515357212, s2 = (T)0.58778525229247312917;
       r1 = axpy(c2, a2, axpy(c1, a1, v[0]));
       r2 = axpy(c1, a2, axpy(c2, a1, v[0]));
-      w1 = axpy(s2, b2, scaled(s1, b1));
-      w2 = axpy(-s1, b2, scaled(s2, b1));
+      w1 = axpy(s1, b1, scaled(s2, b2));
+      w2 = axpy(s2, b1, scaled(-s1, b2));
     }
     v[0] = add(v[0], add(a1, a2));
     v[1] = add_i(r1, w1, s);

@@ -217,7 +217,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int r = dnpx(t), p = t - r * npx;
     const int u3 = dw2(p), u2 = p - u3 * W2;
     float2* row = box + zwin[u3] * P2 + ywin[u2] * P1;
-    float2 v[A];
+    fftr::F2 v[A];
 #pragma unroll
     for (int i = 0; i < A; ++i) v[i] = row[r + B * i];
     fftr::rdft<A>(v, 1.f);
@@ -231,7 +231,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int k = dnpx(t), p = t - k * npx;
     const int u3 = dw2(p), u2 = p - u3 * W2;
     float2* row = box + zwin[u3] * P2 + ywin[u2] * P1 + B * k;
-    float2 v[B];
+    fftr::F2 v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = row[j];
     fftr::rdft<B>(v, 1.f);
@@ -244,7 +244,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int r = dnpy(t), p = t - r * npy;
     const int u3 = p / N, x = p - u3 * N;
     float2* col = box + zwin[u3] * P2 + x;
-    float2 v[A];
+    fftr::F2 v[A];
 #pragma unroll
     for (int i = 0; i < A; ++i) v[i] = ymap[r + B * i] >= 0 ? col[(r + B * i) * P1] : make_float2(0.f, 0.f);
     fftr::rdft<A>(v, 1.f);
@@ -258,7 +258,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int k = dnpy(t), p = t - k * npy;
     const int u3 = p / N, x = p - u3 * N;
     float2* col = box + zwin[u3] * P2 + x + (B * k) * P1;
-    float2 v[B];
+    fftr::F2 v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = col[j * P1];
     fftr::rdft<B>(v, 1.f);
@@ -270,7 +270,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
   for (int t = tid; t < NN * B; t += NT) {
     const int r = t / NN, p = t - r * NN;
     float2* col = box + (p / N) * P1 + (p % N);
-    float2 v[A];
+    fftr::F2 v[A];
 #pragma unroll
     for (int i = 0; i < A; ++i) v[i] = zmap[r + B * i] >= 0 ? col[(r + B * i) * P2] : make_float2(0.f, 0.f);
     fftr::rdft<A>(v, 1.f);
@@ -285,7 +285,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int k = t / NN, p = t - k * NN;
     float2* col = box + (p / N) * P1 + (p % N) + (B * k) * P2;
     const float* vz = V + (size_t)(B * k) * NN + p;  // position z' = B k + j at vz[j NN]
-    float2 v[B];
+    fftr::F2 v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = col[j * P2];
     fftr::rdft<B>(v, 1.f);
@@ -306,7 +306,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
   for (int t = tid; t < NN * B; t += NT) {
     const int q = t / NN, p = t - q * NN;
     float2* col = box + (p / N) * P1 + (p % N);
-    float2 v[A];
+    fftr::F2 v[A];
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = col[(q + B * m) * P2];
     fftr::rdft<A>(v, -1.f);
@@ -320,7 +320,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int r = dnpy(t), p = t - r * npy;
     const int u3 = p / N, x = p - u3 * N;
     float2* col = box + zwin[u3] * P2 + x + (B * r) * P1;
-    float2 v[B];
+    fftr::F2 v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = col[j * P1];
     fftr::rdft<B>(v, -1.f);
@@ -334,7 +334,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int q = dnpy(t), p = t - q * npy;
     const int u3 = p / N, x = p - u3 * N;
     float2* col = box + zwin[u3] * P2 + x;
-    float2 v[A];
+    fftr::F2 v[A];
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = col[(q + B * m) * P1];
     fftr::rdft<A>(v, -1.f);
@@ -348,7 +348,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int r = dnpx(t), p = t - r * npx;
     const int u3 = dw2(p), u2 = p - u3 * W2;
     float2* row = box + zwin[u3] * P2 + ywin[u2] * P1 + B * r;
-    float2 v[B];
+    fftr::F2 v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = row[j];
     fftr::rdft<B>(v, -1.f);
@@ -362,7 +362,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
     const int q = dnpx(t), p = t - q * npx;
     const int u3 = dw2(p), u2 = p - u3 * W2;
     float2* row = box + zwin[u3] * P2 + ywin[u2] * P1;
-    float2 v[A];
+    fftr::F2 v[A];
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = row[q + B * m];
     fftr::rdft<A>(v, -1.f);

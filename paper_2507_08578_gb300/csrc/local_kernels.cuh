@@ -568,6 +568,7 @@ __device__ __forceinline__ void load_twiddles(const C* row, C (&w)[n]) {
 template <typename T, int A, int B, int CW = 0>
 __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int nl) {
   using C = typename CT<T>::C;
+  using V = typename fftr::Packed<C>::T;
   using G = WideB<T, A, B>;
   constexpr int N = G::N, QS = G::QS, ZS = G::ZS;
   constexpr unsigned MW = fftr::edge_mask<A, CW>(), MF = fftr::full_mask<A>();
@@ -613,7 +614,8 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
   for (int t = tid; t < W3 * B; t += NT) {
     const int r = dw3(t), u = t - r * W3;  // rows fastest across lanes
     C* row = Q + u * QS + r;
-    C v[A], w[A];
+    V v[A];
+    C w[A];
     load_twiddles(twi + r * A, w);
     fftr::static_for<0, A>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
@@ -629,7 +631,7 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
   for (int t = tid; t < W3 * A; t += NT) {
     const int k = dw3(t), u = t - k * W3;
     C* row = Q + u * QS + B * k;
-    C v[B];
+    V v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = row[j];
     fftr::rdft<B>(v, (T)1);
@@ -643,7 +645,8 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
   // ---- z, inverse stage 1 (column p of the plane; only window rows are nonzero) ----
   for (int t = tid; t < N * B; t += NT) {
     const int r = t / N, p = t - r * N;
-    C v[A], w[A];
+    V v[A];
+    C w[A];
     load_twiddles(twi + r * A, w);
     const int u0 = r - lo3;
     const C* q0 = Q + u0 * QS + p;
@@ -673,7 +676,7 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
     const int k = t / N, p = t - k * N;
     const T* vrow = vp + (size_t)k * N + p;  // (z = k + A k2, p) at vrow[A k2 N]
     C* col = Z + p * ZS + B * k;
-    C v[B];
+    V v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = col[j];
     fftr::rdft<B>(v, (T)1);
@@ -696,7 +699,7 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
   for (int t = tid; t < N * B; t += NT) {
     const int q = t / N, p = t - q * N;
     const C* col = Z + p * ZS + q;
-    C v[A];
+    V v[A];
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = col[B * m];
     fftr::rdft_m<A, MF, MW>(v, (T)-1);
@@ -719,7 +722,8 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
   for (int t = tid; t < W3 * A; t += NT) {
     const int r = dw3(t), u = t - r * W3;
     C* row = Q + u * QS + B * r;
-    C v[B], w[B];
+    V v[B];
+    C w[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = row[j];
     fftr::rdft<B>(v, (T)-1);
@@ -733,7 +737,7 @@ __device__ __forceinline__ void pass_bw_body(const LocalArgs<T>& a, int x, int n
   for (int t = tid; t < W3 * B; t += NT) {
     const int q = dw3(t), u = t - q * W3;
     C* row = Q + u * QS + q;
-    C v[A];
+    V v[A];
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = row[B * m];
     fftr::rdft_m<A, MF, MW>(v, (T)-1);
@@ -793,7 +797,7 @@ __device__ __forceinline__ void pass_aw_body(const LocalArgs<T>& a, int u3, int 
   for (int t = tid; t < nrows * B; t += NT) {
     const int r = dnr(t), u = t - r * nrows;
     C* row = rows + u * P + r;
-    C v[A];
+    typename fftr::Packed<C>::T v[A];
     fftr::static_for<0, A>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
       if constexpr (MW >> i & 1u) v[i] = row[B * i];
@@ -813,7 +817,7 @@ __device__ __forceinline__ void pass_aw_body(const LocalArgs<T>& a, int u3, int 
   for (int t = tid; t < nrows * A; t += NT) {
     const int k = dnr(t), u = t - k * nrows;
     C* row = rows + u * P + B * k;
-    C v[B];
+    typename fftr::Packed<C>::T v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = row[j];
     fftr::rdft<B>(v, (T)1);
@@ -861,7 +865,7 @@ __device__ __forceinline__ void pass_cw_body(const LocalArgs<T>& a, int u3, int 
   for (int t = tid; t < nrows * A; t += NT) {
     const int r = dnr(t), u = t - r * nrows;
     C* row = rows + u * P + B * r;
-    C v[B];
+    typename fftr::Packed<C>::T v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = row[j];
     fftr::rdft<B>(v, (T)-1);
@@ -876,7 +880,7 @@ __device__ __forceinline__ void pass_cw_body(const LocalArgs<T>& a, int u3, int 
   for (int t = tid; t < nrows * B; t += NT) {
     const int q = dnr(t), u = t - q * nrows;
     C* row = rows + u * P + q;
-    C v[A];
+    typename fftr::Packed<C>::T v[A];
 #pragma unroll
     for (int m = 0; m < A; ++m) v[m] = row[B * m];
     fftr::rdft_m<A, MF, MW>(v, (T)-1);
