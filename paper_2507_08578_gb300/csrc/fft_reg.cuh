@@ -129,31 +129,34 @@ struct alignas(8) F2 {
 };
 template <typename C> struct Packed { using T = C; };
 template <> struct Packed<float2> { using T = F2; };
-__device__ __forceinline__ unsigned long long bits2(F2 a) {
-  return (unsigned long long)__float_as_uint(a.y) << 32 | __float_as_uint(a.x);
-}
-__device__ __forceinline__ F2 from_bits2(unsigned long long u) {
-  return F2(__uint_as_float((unsigned)u), __uint_as_float((unsigned)(u >> 32)));
-}
 __device__ __forceinline__ F2 add(F2 a, F2 b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
-  return from_bits2(r);
+  F2 r;
+  asm("{.reg .b64 p, q, s; mov.b64 p, {%2, %3}; mov.b64 q, {%4, %5}; add.rn.f32x2 s, p, q; mov.b64 {%0, %1}, s;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
 }
 __device__ __forceinline__ F2 sub(F2 a, F2 b) {
-  unsigned long long r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
-  return from_bits2(r);
+  F2 r;
+  asm("{.reg .b64 p, q, s; mov.b64 p, {%2, %3}; mov.b64 q, {%4, %5}; sub.rn.f32x2 s, p, q; mov.b64 {%0, %1}, s;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
 }
 __device__ __forceinline__ F2 axpy(float a, F2 b, F2 c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(bits2(F2(a, a))), "l"(bits2(b)), "l"(bits2(c)));
-  return from_bits2(r);
+  F2 r;
+  asm("{.reg .b64 p, q, s, t; mov.b64 p, {%2, %2}; mov.b64 q, {%3, %4}; mov.b64 s, {%5, %6};"
+      " fma.rn.f32x2 t, p, q, s; mov.b64 {%0, %1}, t;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
 }
 __device__ __forceinline__ F2 scaled(float a, F2 b) {
-  unsigned long long r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(F2(a, a))), "l"(bits2(b)));
-  return from_bits2(r);
+  F2 r;
+  asm("{.reg .b64 p, q, s; mov.b64 p, {%2, %2}; mov.b64 q, {%3, %4}; mul.rn.f32x2 s, p, q; mov.b64 {%0, %1}, s;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a), "f"(b.x), "f"(b.y));
+  return r;
 }
 __device__ __forceinline__ F2 add_i(F2 a, F2 d, float s) {
   return s > 0.f ? F2(a.x - d.y, a.y + d.x) : F2(a.x + d.y, a.y - d.x);
