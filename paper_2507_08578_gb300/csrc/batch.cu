@@ -584,22 +584,22 @@ void BatchEngine::launch_filter_t() {
         continue;
       }
       ProfScope ps(ctx, ida);
-      group_kernel<T, 0>(pc.code1)<<<pc.blocks_ac, kThreads, pc.smem_ac, ctx->stream>>>(it, pc.count, scr_warp);
+      launch_pdl(group_kernel<T, 0>(pc.code1), pc.blocks_ac, kThreads, pc.smem_ac, ctx->stream, it, pc.count, scr_warp);
     }
     for (const PassClass& pc : classes) {
       const LocalItem<T>* it = dl + (size_t)j * n + pc.first;
       if (pc.fcode) continue;
       ProfScope ps(ctx, idb);
       if (pc.wnt)
-        group_kernel_w<T>(pc.wa, pc.wb, pc.wnt, pc.wpruned)<<<pc.blocks_b, pc.wnt, pc.smem_bw, ctx->stream>>>(it, pc.count, scr_warp);
+        launch_pdl(group_kernel_w<T>(pc.wa, pc.wb, pc.wnt, pc.wpruned), pc.blocks_b, pc.wnt, pc.smem_bw, ctx->stream, it, pc.count, scr_warp);
       else
-        group_kernel<T, 1>(pc.code23)<<<pc.blocks_b, kThreads, pc.smem_b, ctx->stream>>>(it, pc.count, scr_warp);
+        launch_pdl(group_kernel<T, 1>(pc.code23), pc.blocks_b, kThreads, pc.smem_b, ctx->stream, it, pc.count, scr_warp);
     }
     for (const PassClass& pc : classes) {
       const LocalItem<T>* it = dl + (size_t)j * n + pc.first;
       if (pc.fcode) continue;
       ProfScope ps(ctx, idc);
-      group_kernel<T, 2>(pc.code1)<<<pc.blocks_ac, kThreads, pc.smem_ac, ctx->stream>>>(it, pc.count, scr_warp);
+      launch_pdl(group_kernel<T, 2>(pc.code1), pc.blocks_ac, kThreads, pc.smem_ac, ctx->stream, it, pc.count, scr_warp);
     }
     if (tc_on) tc_nn.launch(ctx, j, "nonlocal");
     if (simt_on && nn_blocks) group_gemm_nn(ctx, f64, nn, n, nn_blocks);

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "local_kernels.cuh"
+#include "pdl.cuh"
 
 namespace kss {
 namespace bk {
@@ -32,6 +33,7 @@ __device__ __forceinline__ int find_local(const LocalItem<T>* it, int n, int b, 
 template <typename T, int PASS, class Pol>
 __global__ void __launch_bounds__(kThreads) group_pass(const LocalItem<T>* __restrict__ items, int n,
                                                        int scr_warp) {
+  pdl_wait();
   __shared__ LocalArgs<T> sa;
   __shared__ RegPlan srp;
   __shared__ int s_local, s_idle;
@@ -55,6 +57,7 @@ __global__ void __launch_bounds__(kThreads) group_pass(const LocalItem<T>* __res
 // Pass B of a class with a common compile-time y/z split, in the CTA-wide form.
 template <typename T, int A, int B, int CW>
 __global__ void __launch_bounds__(kWideThreads) group_passw(const LocalItem<T>* __restrict__ items, int n, int) {
+  pdl_wait();
   __shared__ LocalArgs<T> sa;
   __shared__ int s_local, s_idle;
   if (threadIdx.x == 0) {

@@ -12,6 +12,7 @@
 #include "density.h"
 #include "kss_internal.h"
 #include "local_wide.h"
+#include "pdl.cuh"
 
 namespace kss {
 
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(NT) pass_dw(LocalArgs<T> a, int m, int G, cons
 // rho[z][y][x] += inv_vol * sum_g part[g][x][y][z]
 __global__ void density_reduce(int N1, int N2, int N3, int G, const double* __restrict__ part, double* rho,
                                double inv_vol) {
+  pdl_wait();
   const long long n = (long long)N1 * N2 * N3;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
        idx += (long long)gridDim.x * blockDim.x) {
@@ -260,7 +262,7 @@ void density_t(kss_sys s, int ik, int nb, const void* psi, int ld, const double*
     ProfScope ps(ctx, idr);
     const long long n = (long long)N1 * N2 * N3;
     const unsigned blocks = (unsigned)std::min<long long>((n + 255) / 256, 152LL * 16);
-    density_reduce<<<blocks, 256, 0, ctx->stream>>>(N1, N2, N3, G, ctx->ws_rho.as<double>(), rho, 1.0 / s->vol);
+    launch_pdl(density_reduce, blocks, 256, 0, ctx->stream, N1, N2, N3, G, ctx->ws_rho.as<double>(), rho, 1.0 / s->vol);
   }
   KSS_CHECK_CUDA(cudaGetLastError());
 }

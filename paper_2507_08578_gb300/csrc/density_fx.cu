@@ -32,6 +32,7 @@ __device__ __forceinline__ unsigned long long norm62(Cx v) {
 template <int A, int B, int CW>
 __global__ void __launch_bounds__(kFxThreads) pass_df(LocalArgs<double> a, int m, int G, const double* __restrict__ occ,
                                                       double* __restrict__ part) {
+  pdl_wait();
   using W = FxB<A, B>;
   constexpr int N = W::N, ZS = W::ZS, NT = kFxThreads;
   constexpr int R = (N * A + NT - 1) / NT;
@@ -112,7 +113,7 @@ bool launch_df(const LocalArgs<double>& a, int m, int G, const double* occ, doub
   if (resident)
     KSS_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, k, kFxThreads, sm));
   else
-    k<<<dim3(a.N1, G), kFxThreads, sm, st>>>(a, m, G, occ, part);
+    launch_pdl(k, dim3(a.N1, G), kFxThreads, sm, st, a, m, G, occ, part);
   return true;
 }
 

@@ -43,6 +43,7 @@
 #include <string>
 
 #include "gemm_tune.h"
+#include "pdl.cuh"
 #include "tc_common.cuh"
 
 namespace kss {
@@ -108,6 +109,7 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                int rowsB, int Mr, int Nr, int tnn, int kb_per_split, int kb_total, const int* __restrict__ ea,
                const int* __restrict__ eb, int* __restrict__ err, double* __restrict__ part,
                CT* __restrict__ C, long long ldc, double ar, double ai, double br, double bi) {
+  pdl_wait();
   constexpr uint32_t STAGE = OzCfg<SA, SB>::STAGE;
   constexpr int STAGES = OzCfg<SA, SB>::STAGES;
   extern __shared__ __align__(1024) unsigned char smraw[];
@@ -375,6 +377,7 @@ template <> struct Real<float2> { using T = float; };
 template <int S, typename CS>
 __global__ void oz_prep_k(const CS* __restrict__ src, long long ld, int K, int KT, __nv_bfloat16* __restrict__ dst,
                           int rows, int* __restrict__ erow, int pair) {
+  pdl_wait();
   using R = typename Real<CS>::T;
   __shared__ unsigned long long red[32];
   const int c = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
@@ -426,6 +429,7 @@ __global__ void oz_prep_k(const CS* __restrict__ src, long long ld, int K, int K
 // Exponents of the rows of an M-major complex A (element (i, k) at src[k ld + i]), one thread per i.
 template <typename CS>
 __global__ void oz_exp_m(const CS* __restrict__ src, long long ld, int M, int K, int* __restrict__ erow) {
+  pdl_wait();
   using R = typename Real<CS>::T;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M) return;
@@ -447,6 +451,7 @@ __global__ void oz_exp_m(const CS* __restrict__ src, long long ld, int M, int K,
 template <int S, typename CS>
 __global__ void oz_prep_m(const CS* __restrict__ src, long long ld, int M, int K, int KT,
                           __nv_bfloat16* __restrict__ dst, int rows, const int* __restrict__ erow) {
+  pdl_wait();
   __shared__ CS t[32][33];
   const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -481,6 +486,7 @@ __global__ void oz_prep_m(const CS* __restrict__ src, long long ld, int M, int K
 template <typename CT>
 __global__ void oz_combine(const double* __restrict__ P, int nsplit, int Mr, int Nr, int M, int N,
                            CT* __restrict__ C, long long ldc, double ar, double ai, double br, double bi) {
+  pdl_wait();
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (idx >= (long long)M * N) return;
   const int i = (int)(idx % M), j = (int)(idx / M);
@@ -564,16 +570,16 @@ void launch_oz(kss_ctx ctx, const OzOperand& a, const OzOperand& b, int M, int N
     const bool fused = splits == 1;
     {
       ProfScope ps(ctx, prof ? prof_register(name.c_str()) : prof_register("gemm_tuning"));
-      kern<<<dim3((unsigned)tiles, splits, 1), kOzThreads, Cfg::SMEM, ctx->stream>>>(
-          ma, mb, a.rows, b.rows, Mr, Nr, tnn, kps, kb_total, a.e, b.e, err_flag(ctx),
+      launch_pdl(
+          kern, dim3((unsigned)tiles, splits, 1), kOzThreads, Cfg::SMEM, ctx->stream, ma, mb, a.rows, b.rows, Mr, Nr, tnn, kps, kb_total, a.e, b.e, err_flag(ctx),
           fused ? nullptr : ctx->oz_part.as<double>(), Cd, ldd, ar, ai, br_, bi_);
     }
     KSS_CHECK_CUDA(cudaGetLastError());
     if (fused) return;
     const long long mn = (long long)M * N;
     ProfScope ps(ctx, prof ? prof_register(cname.c_str()) : prof_register("gemm_tuning"));
-    oz_combine<CT><<<(unsigned)((mn + 255) / 256), 256, 0, ctx->stream>>>(ctx->oz_part.as<double>(), splits, Mr,
-                                                                          Nr, M, N, Cd, ldd, ar, ai, br_, bi_);
+    launch_pdl(oz_combine<CT>, (unsigned)((mn + 255) / 256), 256, 0, ctx->stream, ctx->oz_part.as<double>(), splits, Mr,
+               Nr, M, N, Cd, ldd, ar, ai, br_, bi_);
     KSS_CHECK_CUDA(cudaGetLastError());
   };
   const int kind = SA == 4 ? GT_OZ44 : (sizeof(CT) == sizeof(double2) ? GT_OZ77 : GT_OZ77_C64OUT);
@@ -621,13 +627,13 @@ template <int S, typename CS>
 void prepare_as(kss_ctx ctx, OzKind kind, int n, int K, const CS* src, long long ld, const OzOperand& o) {
   if (kind == OZ_MMAJOR_A) {
     dim3 g((n + 31) / 32, (o.KT / 2 + 31) / 32);
-    oz_exp_m<CS><<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(src, ld, n, K, o.e);
-    oz_prep_m<S, CS><<<g, dim3(32, 8), 0, ctx->stream>>>(src, ld, n, K, o.KT, o.planes, o.rows, o.e);
+    launch_pdl(oz_exp_m<CS>, (unsigned)((n + 255) / 256), 256, 0, ctx->stream, src, ld, n, K, o.e);
+    launch_pdl(oz_prep_m<S, CS>, g, dim3(32, 8), 0, ctx->stream, src, ld, n, K, o.KT, o.planes, o.rows, o.e);
   } else {
     // wide CTAs where the columns alone would leave SMs short of threads
     const int nt = n < 3 * std::max(ctx->nsm, 1) && K > 2048 ? 768 : 256;
-    oz_prep_k<S, CS><<<(unsigned)n, nt, 0, ctx->stream>>>(src, ld, K, o.KT, o.planes, o.rows, o.e,
-                                                          kind == OZ_CN_A ? 1 : 0);
+    launch_pdl(oz_prep_k<S, CS>, (unsigned)n, nt, 0, ctx->stream, src, ld, K, o.KT, o.planes, o.rows, o.e,
+               kind == OZ_CN_A ? 1 : 0);
   }
 }
 

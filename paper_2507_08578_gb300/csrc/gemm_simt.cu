@@ -11,7 +11,7 @@
 #include <mutex>
 #include <string>
 
-#include "kss_internal.h"
+#include "pdl.cuh"
 
 namespace kss {
 
@@ -396,6 +396,7 @@ __global__ void __launch_bounds__(256) gg_nn(const GemmItem* __restrict__ items,
 template <typename T>
 __global__ void scale_rows_kernel(int M, int N, typename CT<T>::C* __restrict__ Cm, long long ldc,
                                   const T* __restrict__ d, T s) {
+  pdl_wait();
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (idx >= (long long)M * N) return;
   const int i = (int)(idx % M), j = (int)(idx / M);
@@ -717,10 +718,10 @@ void scale_rows(kss_ctx ctx, bool fp64, int M, int N, void* C, int ldc, const vo
   static const int id = prof_register("scale_rows");
   ProfScope ps(ctx, id);
   if (fp64)
-    scale_rows_kernel<double><<<(unsigned)((mn + 255) / 256), 256, 0, st>>>(M, N, (double2*)C, ldc,
+    launch_pdl(scale_rows_kernel<double>, (unsigned)((mn + 255) / 256), 256, 0, st, M, N, (double2*)C, ldc,
                                                                             (const double*)d, s);
   else
-    scale_rows_kernel<float><<<(unsigned)((mn + 255) / 256), 256, 0, st>>>(M, N, (float2*)C, ldc,
+    launch_pdl(scale_rows_kernel<float>, (unsigned)((mn + 255) / 256), 256, 0, st, M, N, (float2*)C, ldc,
                                                                           (const float*)d, (float)s);
   KSS_CHECK_CUDA(cudaGetLastError());
 }

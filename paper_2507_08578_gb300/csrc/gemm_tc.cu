@@ -32,6 +32,7 @@
 #include <string>
 
 #include "gemm_tune.h"
+#include "pdl.cuh"
 #include "tc_common.cuh"
 
 namespace kss {
@@ -76,6 +77,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                float* __restrict__ D, int Mr, int Nr, int tnn, int kb_per_split, int kb_total, int kp,
                int* __restrict__ err, float2* __restrict__ Cf, long long ldc, float ar, float ai, float br,
                float bi) {
+  pdl_wait();
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   // stage s: A hi, A lo, B hi, B lo tiles at base + s * kStageBytes
@@ -304,6 +306,7 @@ template <int TNP> constexpr size_t p_smem() { return 1024 + (size_t)p_stages<TN
 
 template <int TNP>
 __global__ void __launch_bounds__(kPThreads, 1) tc_persist_kernel(const __grid_constant__ TcPersistArgs a) {
+  pdl_wait();
   constexpr int S = p_stages<TNP>();
   constexpr uint32_t kA = TM * TK * 2, kB = TNP * TK * 2, kSt = p_stage_bytes<TNP>();
   extern __shared__ __align__(1024) unsigned char smraw[];
@@ -512,6 +515,7 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_persist_kernel(const __grid_c
 // Grouped combine of the split products of a persistent launch: C = (alpha rs[i]) sum_z P_z +
 // beta C, the K ranges added in a fixed order.  Block b belongs to the last product with cb0 <= b.
 __global__ void tc_group_combine(const TcProd* __restrict__ prods, int nprod) {
+  pdl_wait();
   int lo = 0, hi = nprod;
   const long long b = blockIdx.x;
   while (hi - lo > 1) {
@@ -581,6 +585,7 @@ __device__ __forceinline__ void prep_kmajor_elem(const float2* __restrict__ src,
 
 __global__ void prep_kmajor(const float2* __restrict__ src, long long ld, int K, int ncols, int Kp,
                             __nv_bfloat16* __restrict__ dst, int pair) {
+  pdl_wait();
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const int half = Kp / 2;
   if (idx >= (long long)ncols * half) return;
@@ -598,6 +603,7 @@ struct TcPrepItem {
   long long b0;
 };
 __global__ void prep_kmajor_group(const TcPrepItem* __restrict__ items, int n) {
+  pdl_wait();
   int lo = 0, hi = n;
   const long long b = blockIdx.x;
   while (hi - lo > 1) {
@@ -619,6 +625,7 @@ __global__ void prep_kmajor_group(const TcPrepItem* __restrict__ items, int n) {
 // row i are adjacent accumulator rows), each row [hi | lo].  32x32 smem transpose.
 __global__ void prep_mmajor(const float2* __restrict__ src, long long ld, int M, int K, int Kp,
                             __nv_bfloat16* __restrict__ dst) {
+  pdl_wait();
   __shared__ float2 t[32][33];
   const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -648,6 +655,7 @@ __global__ void prep_mmajor(const float2* __restrict__ src, long long ld, int M,
 // (col-major Mr x Nr, Mr = 2M): re = D(2i, j), im = D(2i + 1, j).
 __global__ void tc_combine(const float* __restrict__ P, int nsplit, int Mr, int Nr, int M, int N,
                            float2* __restrict__ C, long long ldc, float ar, float ai, float br, float bi) {
+  pdl_wait();
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (idx >= (long long)M * N) return;
   const int i = (int)(idx % M), j = (int)(idx / M);
@@ -702,7 +710,7 @@ void launch_persist(kss_ctx ctx, const TcPersistArgs& args, int grid) {
   // per device (the attribute belongs to the current device): set at every launch
   KSS_CHECK_CUDA(cudaFuncSetAttribute(tc_persist_kernel<TNP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)p_smem<TNP>()));
-  tc_persist_kernel<TNP><<<grid, kPThreads, p_smem<TNP>(), ctx->stream>>>(args);
+  launch_pdl(tc_persist_kernel<TNP>, grid, kPThreads, p_smem<TNP>(), ctx->stream, args);
   KSS_CHECK_CUDA(cudaGetLastError());
 }
 
@@ -752,8 +760,8 @@ void run_tc(kss_ctx ctx, const __nv_bfloat16* Atc, const __nv_bfloat16* Btc, int
     {
       ProfScope ps(ctx, prof_register(prof ? name.c_str() : "gemm_tuning"));
       if (ch.form == 0) {
-        tc_gemm_kernel<<<dim3((unsigned)tiles, splits, 1), kTcThreads, kTcSmem, ctx->stream>>>(
-            ma, mb, ctx->tc_part.as<float>(), Mr, Nr, tnn, kps, kb_total, Kp, ctx->tc_err.as<int>(),
+        launch_pdl(
+            tc_gemm_kernel, dim3((unsigned)tiles, splits, 1), kTcThreads, kTcSmem, ctx->stream, ma, mb, ctx->tc_part.as<float>(), Mr, Nr, tnn, kps, kb_total, Kp, ctx->tc_err.as<int>(),
             fused ? Cd : nullptr, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
         KSS_CHECK_CUDA(cudaGetLastError());
       } else {
@@ -788,8 +796,8 @@ void run_tc(kss_ctx ctx, const __nv_bfloat16* Atc, const __nv_bfloat16* Btc, int
     if (fused) return;
     const long long mn = (long long)M * N;
     ProfScope ps(ctx, prof_register(prof ? cname.c_str() : "gemm_tuning"));
-    tc_combine<<<(unsigned)((mn + 255) / 256), 256, 0, ctx->stream>>>(
-        ctx->tc_part.as<float>(), splits, Mr, Nr, M, N, Cd, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
+    launch_pdl(
+        tc_combine, (unsigned)((mn + 255) / 256), 256, 0, ctx->stream, ctx->tc_part.as<float>(), splits, Mr, Nr, M, N, Cd, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
     KSS_CHECK_CUDA(cudaGetLastError());
   };
   // Candidates: every form with no split, the plan and the splits filling one to three waves.  Each
@@ -830,7 +838,7 @@ void tc_gemm_cn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const 
   {
     ProfScope ps(ctx, prof_register("tc_prep"));
     const long long na = (long long)M * (Kp / 2);
-    prep_kmajor<<<(unsigned)((na + 255) / 256), 256, 0, ctx->stream>>>((const float2*)A, lda, K, M, Kp, Atc, 1);
+    launch_pdl(prep_kmajor, (unsigned)((na + 255) / 256), 256, 0, ctx->stream, (const float2*)A, lda, K, M, Kp, Atc, 1);
   }
   tc_gemm_cn_split(ctx, M, N, K, Atc, B, ldb, C, ldc, ar, ai, br, bi, tag);
 }
@@ -845,7 +853,7 @@ void tc_gemm_nn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const 
   {
     ProfScope ps(ctx, prof_register("tc_prep"));
     dim3 g((M + 31) / 32, (Kp / 2 + 31) / 32);
-    prep_mmajor<<<g, dim3(32, 8), 0, ctx->stream>>>((const float2*)A, lda, M, K, Kp, Atc);
+    launch_pdl(prep_mmajor, g, dim3(32, 8), 0, ctx->stream, (const float2*)A, lda, M, K, Kp, Atc);
   }
   tc_gemm_nn_split(ctx, M, N, K, Atc, B, ldb, C, ldc, ar, ai, br, bi, tag);
 }
@@ -859,7 +867,7 @@ size_t tc_split_nn_bytes(int M, int K) { return (size_t)2 * M * 2 * kpad(K) * 2;
 void tc_split_cn(kss_ctx ctx, int M, int K, const void* A, int lda, void* Atc) {
   const int Kp = kpad(K);
   const long long na = (long long)M * (Kp / 2);
-  prep_kmajor<<<(unsigned)((na + 255) / 256), 256, 0, ctx->stream>>>((const float2*)A, lda, K, M, Kp,
+  launch_pdl(prep_kmajor, (unsigned)((na + 255) / 256), 256, 0, ctx->stream, (const float2*)A, lda, K, M, Kp,
                                                                     (__nv_bfloat16*)Atc, 1);
   KSS_CHECK_CUDA(cudaGetLastError());
 }
@@ -867,7 +875,7 @@ void tc_split_cn(kss_ctx ctx, int M, int K, const void* A, int lda, void* Atc) {
 void tc_split_nn(kss_ctx ctx, int M, int K, const void* A, int lda, void* Atc) {
   const int Kp = kpad(K);
   dim3 g((M + 31) / 32, (Kp / 2 + 31) / 32);
-  prep_mmajor<<<g, dim3(32, 8), 0, ctx->stream>>>((const float2*)A, lda, M, K, Kp, (__nv_bfloat16*)Atc);
+  launch_pdl(prep_mmajor, g, dim3(32, 8), 0, ctx->stream, (const float2*)A, lda, M, K, Kp, (__nv_bfloat16*)Atc);
   KSS_CHECK_CUDA(cudaGetLastError());
 }
 
@@ -879,7 +887,7 @@ const __nv_bfloat16* prep_b(kss_ctx ctx, int N, int K, const void* B, int ldb) {
   __nv_bfloat16* Btc = ctx->tc_b.as<__nv_bfloat16>();
   ProfScope ps(ctx, prof_register("tc_prep"));
   const long long nb = (long long)N * (Kp / 2);
-  prep_kmajor<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>((const float2*)B, ldb, K, N, Kp, Btc, 0);
+  launch_pdl(prep_kmajor, (unsigned)((nb + 255) / 256), 256, 0, ctx->stream, (const float2*)B, ldb, K, N, Kp, Btc, 0);
   return Btc;
 }
 }  // namespace
@@ -1035,7 +1043,7 @@ void TcGroupPlan::launch(kss_ctx ctx, int step, const char* tag) const {
   {
     static const int id = prof_register("tc_prep_group");
     ProfScope ps(ctx, id);
-    prep_kmajor_group<<<prep_blocks_, 256, 0, ctx->stream>>>(preps, n_);
+    launch_pdl(prep_kmajor_group, prep_blocks_, 256, 0, ctx->stream, preps, n_);
     KSS_CHECK_CUDA(cudaGetLastError());
   }
   {
@@ -1049,14 +1057,14 @@ void TcGroupPlan::launch(kss_ctx ctx, int step, const char* tag) const {
     args.err = ctx->tc_err.as<int>();
     const int grid = std::max(1, std::min(nwork_, sms(ctx)));
     if (tnp_ == 64)
-      tc_persist_kernel<64><<<grid, kPThreads, p_smem<64>(), ctx->stream>>>(args);
+      launch_pdl(tc_persist_kernel<64>, grid, kPThreads, p_smem<64>(), ctx->stream, args);
     else
-      tc_persist_kernel<128><<<grid, kPThreads, p_smem<128>(), ctx->stream>>>(args);
+      launch_pdl(tc_persist_kernel<128>, grid, kPThreads, p_smem<128>(), ctx->stream, args);
     KSS_CHECK_CUDA(cudaGetLastError());
   }
   if (any_split_) {
     ProfScope ps(ctx, prof_register((std::string("tc_group_combine:") + tag).c_str()));
-    tc_group_combine<<<(unsigned)comb_blocks_, 256, 0, ctx->stream>>>(prods, n_);
+    launch_pdl(tc_group_combine, (unsigned)comb_blocks_, 256, 0, ctx->stream, prods, n_);
     KSS_CHECK_CUDA(cudaGetLastError());
   }
 }

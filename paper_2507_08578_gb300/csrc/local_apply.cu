@@ -29,6 +29,7 @@
 #include "local_kernels.cuh"
 #include "density.h"
 #include "local_wide.h"
+#include "pdl.cuh"
 #include "tune.h"
 
 namespace kss {
@@ -312,6 +313,7 @@ template <typename C, typename T>
 __global__ void gamma_unpack(const C* __restrict__ F, long long ld, const int* __restrict__ mirror,
                              const C* __restrict__ psi, const C* psi_prev, C* out, const T* __restrict__ kin,
                              int npw, int nb, T al, T be, T ga) {
+  pdl_wait();
   const long long n = (long long)npw * nb;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
@@ -342,14 +344,17 @@ __global__ void gamma_unpack(const C* __restrict__ F, long long ld, const int* _
 
 template <typename T, class Pol = RtPol>
 __global__ void __launch_bounds__(kThreads) pass_a_r(LocalArgs<T> a, RegPlan rp, int scr_warp) {
+  pdl_wait();
   pass_a_body<T, Pol>(a, rp, scr_warp, blockIdx.x, blockIdx.y);
 }
 template <typename T, class Pol = RtPol>
 __global__ void __launch_bounds__(kThreads) pass_b_r(LocalArgs<T> a, RegPlan rp, int scr_warp) {
+  pdl_wait();
   pass_b_body<T, Pol>(a, rp, scr_warp, blockIdx.x, blockIdx.y);
 }
 template <typename T, class Pol = RtPol>
 __global__ void __launch_bounds__(kThreads) pass_c_r(LocalArgs<T> a, RegPlan rp, int scr_warp) {
+  pdl_wait();
   pass_c_body<T, Pol>(a, rp, scr_warp, blockIdx.x, blockIdx.y);
 }
 
@@ -499,8 +504,8 @@ void gamma_finish(kss_sys s, int ik, int nb, const void* psi, const void* psi_pr
   ProfScope ps(ctx, idu);
   const long long n = (long long)kd.npw * nb;
   const unsigned blocks = (unsigned)std::min<long long>((n + 255) / 256, 152LL * 32);
-  gamma_unpack<C, T><<<blocks, 256, 0, ctx->stream>>>(
-      ctx->ws_gpack.as<C>(), ld, kd.d_mirror.as<int>(), (const C*)psi, (const C*)psi_prev, (C*)out,
+  launch_pdl(
+      gamma_unpack<C, T>, blocks, 256, 0, ctx->stream, ctx->ws_gpack.as<C>(), ld, kd.d_mirror.as<int>(), (const C*)psi, (const C*)psi_prev, (C*)out,
       (const T*)(f64 ? kd.d_kin64.p : kd.d_kin32.p), kd.npw, nb, (T)c.alpha, (T)c.beta, (T)c.gamma);
 }
 
@@ -553,11 +558,11 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
                       sizeof(int) * a.N3;
     if (ra <= smax && rb <= smax) {
       const PassKernels<T> kk = pick_kernels<T>(rp);
-      KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ra));
-      KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rb));
-      KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ra));
+      allow_smem(kk.a, ra);
+      allow_smem(kk.b, rb);
+      allow_smem(kk.c, ra);
       auto warp_b = [&](const LocalArgs<T>& t, int m) {
-        kk.b<<<dim3(t.N1, m), kThreads, rb, ctx->stream>>>(t, rp, scr_warp);
+        launch_pdl(kk.b, dim3(t.N1, m), kThreads, rb, ctx->stream, t, rp, scr_warp);
       };
       PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, true);
       bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
@@ -589,7 +594,7 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
         {
           ProfScope ps(ctx, ida);
           if (!(wx && wide_pass_x<T>(a, 0, m, ctx->stream, false)))
-            kk.a<<<dim3(a.W3, m), kThreads, ra, ctx->stream>>>(a, rp, scr_warp);
+            launch_pdl(kk.a, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
         }
         {
           ProfScope ps(ctx, idb);
@@ -598,7 +603,7 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
         {
           ProfScope ps(ctx, idc);
           if (!(wx && wide_pass_x<T>(a, 1, m, ctx->stream, false)))
-            kk.c<<<dim3(a.W3, m), kThreads, ra, ctx->stream>>>(a, rp, scr_warp);
+            launch_pdl(kk.c, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
         }
       }
       if (packed) gamma_finish<T>(s, ik, nb, psi, psi_prev, out, ld, c);
@@ -685,11 +690,11 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
                       sizeof(int) * a.N3;
     if (ra <= smax && rb <= smax) {
       const PassKernels<T> kk = pick_kernels<T>(rp);
-      KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ra));
-      KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rb));
-      KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ra));
+      allow_smem(kk.a, ra);
+      allow_smem(kk.b, rb);
+      allow_smem(kk.c, ra);
       auto warp_b = [&](const LocalArgs<T>& t, int m) {
-        kk.b<<<dim3(t.N1, m), kThreads, rb, ctx->stream>>>(t, rp, scr_warp);
+        launch_pdl(kk.b, dim3(t.N1, m), kThreads, rb, ctx->stream, t, rp, scr_warp);
       };
       PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, false);  // no tuning here
       bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
@@ -709,10 +714,10 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
         const int m = std::min(nc, nb - n0);
         a.n0 = n0;
         if (!(wx && wide_pass_x<T>(a, 0, m, ctx->stream, false)))
-          kk.a<<<dim3(a.W3, m), kThreads, ra, ctx->stream>>>(a, rp, scr_warp);
+          launch_pdl(kk.a, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
         if (!(sb.threads && wide_pass_b<T>(a, sb.A, sb.B, sb.threads, m, ctx->stream, false))) warp_b(a, m);
         if (!(wx && wide_pass_x<T>(a, 1, m, ctx->stream, false)))
-          kk.c<<<dim3(a.W3, m), kThreads, ra, ctx->stream>>>(a, rp, scr_warp);
+          launch_pdl(kk.c, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
       }
       KSS_CHECK_CUDA(cudaGetLastError());
       return;
@@ -746,8 +751,8 @@ void warp_pass_b(kss_ctx ctx, const LocalArgs<T>& a, int nbands) {
   const size_t rb = es * ((size_t)a.N2 + a.N3 + (size_t)a.W3 * a.N2p + (size_t)kWarps * scr_warp) +
                     sizeof(int) * a.N3;
   const PassKernels<T> kk = pick_kernels<T>(rp);
-  KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rb));
-  kk.b<<<dim3(a.N1, nbands), kThreads, rb, ctx->stream>>>(a, rp, scr_warp);
+  allow_smem(kk.b, rb);
+  launch_pdl(kk.b, dim3(a.N1, nbands), kThreads, rb, ctx->stream, a, rp, scr_warp);
 }
 template void warp_pass_b<double>(kss_ctx, const LocalArgs<double>&, int);
 template void warp_pass_b<float>(kss_ctx, const LocalArgs<float>&, int);
@@ -771,7 +776,7 @@ void pass_a_chunks(kss_sys s, int ik, int nb, LocalArgs<T> a, bool fx,
   const size_t ra = sizeof(C) * ((size_t)a.N1 + (size_t)a.W2 * a.N1p + (size_t)kWarps * scr_warp);
   if (ra > 227 * 1024) fail(KSS_ENOTSUP, "FFT box too large for the shared-memory pencil tiles");
   const PassKernels<T> kk = pick_kernels<T>(rp);
-  if (!fx) KSS_CHECK_CUDA(cudaFuncSetAttribute(kk.a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ra));
+  if (!fx) allow_smem(kk.a, ra);
   const int nc = chunk_bands(s, ik, nb, sizeof(C));
   ctx->ws_local.ensure(slab_elems(s, ik) * nc * sizeof(C) + (fx ? local_meta_bytes(s, ik, nc) : 0));
   a.work = ctx->ws_local.as<C>();
@@ -783,7 +788,7 @@ void pass_a_chunks(kss_sys s, int ik, int nb, LocalArgs<T> a, bool fx,
     {
       ProfScope ps(ctx, ida);
       if (fx) wide_pass_x<T>(a, 0, m, ctx->stream, false);
-      else kk.a<<<dim3(a.W3, m), kThreads, ra, ctx->stream>>>(a, rp, scr_warp);
+      else launch_pdl(kk.a, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
     }
     after(a, m);
   }

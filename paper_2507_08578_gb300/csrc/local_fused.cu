@@ -26,6 +26,7 @@
 // Row pitch N | 1 (odd) keeps lanes that step through pencils on distinct shared-memory banks.
 #include <cstdint>
 
+#include "pdl.cuh"
 #include "batch_kernels.cuh"
 #include "fft_reg.cuh"
 #include "kss_internal.h"
@@ -405,6 +406,7 @@ __device__ void fused_band(const FusedSmem& m, const FusedArgs& a, int n) {
 
 template <int A, int B>
 __global__ void __launch_bounds__(kFusedThreads, 1) fused_local_kernel(FusedArgs args) {
+  pdl_wait();
   constexpr int N = A * B;
   extern __shared__ __align__(128) unsigned char fsm[];
   __shared__ FusedArgs a;
@@ -422,6 +424,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_local_kernel(FusedArgs
 template <int A, int B>
 __global__ void __launch_bounds__(kFusedThreads, 1) fused_group_kernel(const bk::LocalItem<float>* __restrict__ items,
                                                                        int n, int tasks, int* err) {
+  pdl_wait();
   constexpr int N = A * B;
   constexpr int vbytes = (int)(((size_t)N * N * N * sizeof(float) + 15) & ~(size_t)15);
   extern __shared__ __align__(128) unsigned char fsm[];
@@ -521,8 +524,8 @@ int vdr_bytes(int N) { return (int)(((size_t)N * N * N * sizeof(float) + 15) & ~
 
 template <int A, int B>
 void launch_fused(const FusedArgs& fa, int grid, size_t smem, cudaStream_t st) {
-  KSS_CHECK_CUDA(cudaFuncSetAttribute(fused_local_kernel<A, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fused_local_kernel<A, B><<<grid, kFusedThreads, smem, st>>>(fa);
+  allow_smem(fused_local_kernel<A, B>, smem);
+  launch_pdl(fused_local_kernel<A, B>, grid, kFusedThreads, smem, st, fa);
 }
 
 
@@ -580,7 +583,7 @@ void fused_group_launch(kss_ctx ctx, int code, const bk::LocalItem<float>* d_ite
   switch (code) {
 #define KSS_FUSED_GROUP(x, y)                                                                       \
   case x * 32 + y:                                                                                  \
-    fused_group_kernel<x, y><<<grid, kFusedThreads, smem, ctx->stream>>>(d_items, n, tasks, err);   \
+    launch_pdl(fused_group_kernel<x, y>, grid, kFusedThreads, smem, ctx->stream, d_items, n, tasks, err); \
     break;
     KSS_FUSED_GROUP(2, 5) KSS_FUSED_GROUP(3, 4) KSS_FUSED_GROUP(3, 5) KSS_FUSED_GROUP(4, 4)
     KSS_FUSED_GROUP(3, 6) KSS_FUSED_GROUP(4, 5) KSS_FUSED_GROUP(4, 6) KSS_FUSED_GROUP(5, 5)

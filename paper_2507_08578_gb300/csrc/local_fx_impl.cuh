@@ -8,6 +8,7 @@
 
 #include "local_fx.cuh"
 #include "local_wide.h"
+#include "pdl.cuh"
 
 namespace kss {
 namespace fx_detail {
@@ -23,21 +24,26 @@ constexpr int part_of(int A, int B) { return (A * 3 + B) % 4; }
 
 template <int A, int B, int CW>
 __global__ void __launch_bounds__(kFxThreads) pass_bf(LocalArgs<double> a) {
+  pdl_wait();
   fx_pass_b<A, B, CW>(a, blockIdx.x, blockIdx.y);
 }
 template <int A, int B, int CW>
 __global__ void __launch_bounds__(kFxXThreads) pass_af(LocalArgs<double> a) {
+  pdl_wait();
   fx_pass_a<A, B, CW>(a, blockIdx.x, blockIdx.y);
 }
 template <int A, int B, int CW>
 __global__ void __launch_bounds__(kFxXThreads) pass_cf(LocalArgs<double> a) {
+  pdl_wait();
   fx_pass_c<A, B, CW>(a, blockIdx.x, blockIdx.y);
 }
 
 using Kern = void (*)(LocalArgs<double>);
 inline void launch(Kern k, const LocalArgs<double>& a, int gx, int nbands, int nt, size_t sm, cudaStream_t st) {
-  KSS_CHECK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k<<<dim3(gx, nbands), nt, sm, st>>>(a);
+  allow_smem(k, sm);
+  // put in place early only up to about a wave of CTAs (H on 20 bands of 24 planes: 59.6 -> 54.3 us; filter
+  // step of 564 bands of 96 planes: 18.37 -> 18.80 ms, the next pass taking places from this one's tail)
+  launch_pdl_if((long long)gx * nbands <= 1024, k, dim3(gx, nbands), nt, sm, st, a);
 }
 
 template <int PART>

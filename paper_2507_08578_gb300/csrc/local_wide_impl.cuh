@@ -6,6 +6,7 @@
 
 #include "local_kernels.cuh"
 #include "local_wide.h"
+#include "pdl.cuh"
 
 namespace kss {
 namespace wide_detail {
@@ -14,6 +15,7 @@ using namespace lk;
 
 template <typename T, int A, int B, int CW>
 __global__ void __launch_bounds__(kWideThreads) pass_bw(LocalArgs<T> a) {
+  pdl_wait();
   pass_bw_body<T, A, B, CW>(a, blockIdx.x, blockIdx.y);
 }
 
@@ -27,8 +29,8 @@ bool launch_one(const LocalArgs<T>& a, int nt, int nbands, cudaStream_t st, bool
   constexpr int PC = wide_edge(A);
   const int cw = wide_prune_cw(A, B, a.lo2, a.W2, a.lo3, a.W3);
   const auto k = PC > 0 && cw > 0 && cw <= PC ? pass_bw<T, A, B, PC> : pass_bw<T, A, B, 0>;
-  KSS_CHECK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k<<<dim3(a.N1, nbands), nt, sm, st>>>(a);
+  allow_smem(k, sm);
+  launch_pdl(k, dim3(a.N1, nbands), nt, sm, st, a);
   return true;
 }
 
@@ -60,17 +62,19 @@ constexpr int kWideXThreads = 256;
 
 template <typename T, int A, int B, int NT, int CW = 0>
 __global__ void __launch_bounds__(NT) pass_aw(LocalArgs<T> a) {
+  pdl_wait();
   pass_aw_body<T, A, B, NT, CW>(a, blockIdx.x, blockIdx.y);
 }
 template <typename T, int A, int B, int NT, int CW = 0>
 __global__ void __launch_bounds__(NT) pass_cw(LocalArgs<T> a) {
+  pdl_wait();
   pass_cw_body<T, A, B, NT, CW>(a, blockIdx.x, blockIdx.y);
 }
 
 template <typename T, int NT, class K>
 void launch_x1(K kern, const LocalArgs<T>& a, size_t sm, int nbands, cudaStream_t st) {
-  KSS_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  kern<<<dim3(a.W3, nbands), NT, sm, st>>>(a);
+  allow_smem(kern, sm);
+  launch_pdl(kern, dim3(a.W3, nbands), NT, sm, st, a);
 }
 
 // which = 0: pass A (inverse transforms), 1: pass C (forward transforms)
