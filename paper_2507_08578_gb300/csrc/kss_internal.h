@@ -423,9 +423,10 @@ void small_gemm_cn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, con
 void small_gemm_nn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc,
                    double ar, double ai, double br, double bi, const char* tag);
 // (complex128 products of small sizes go to the functions above)
+// herm (M = N): the caller knows that the result is Hermitian, as Y^H Y and Y^H H Y are
 void oz_gemm_cn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc,
                 double ar, double ai, double br, double bi, const char* tag, const OzOperand* a_pre = nullptr,
-                bool f64in = true, bool f64out = true, int digits = 0);
+                bool f64in = true, bool f64out = true, int digits = 0, bool herm = false);
 void oz_gemm_nn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc,
                 double ar, double ai, double br, double bi, const char* tag, const OzOperand* a_pre = nullptr,
                 bool f64in = true, bool f64out = true, int digits = 0);

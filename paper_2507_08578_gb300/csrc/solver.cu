@@ -242,17 +242,17 @@ void rr_issue(kss_solver_s* s, bool f64, const void* Y, const void* HY, void* Xo
   // The generalised eigensolve reads the lower triangles of S and Hs only: the Gram products
   // compute the tiles on and below the diagonal (about half the work) and zero the rest.
   if (f64) {
-    // FP64 Gram matrices on the tensor cores (FP64-accurate digit products, full matrices)
-    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, MY, npw, s->S.p, nb, 1, 0, 0, 0, "gram");
-    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, HY, npw, s->Hs.p, nb, 1, 0, 0, 0, "gram");
+    // FP64 Gram matrices on the tensor cores (FP64-accurate digit products)
+    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, MY, npw, s->S.p, nb, 1, 0, 0, 0, "gram", nullptr, true, true, 0, true);
+    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, HY, npw, s->Hs.p, nb, 1, 0, 0, 0, "gram", nullptr, true, true, 0, true);
   } else if (s->gram64) {
     gemm_cn_c64_acc64_lower(ctx, nb, npw, Y, npw, MY, npw, s->S.p, nb, "gram");
     gemm_cn_c64_acc64_lower(ctx, nb, npw, Y, npw, HY, npw, s->Hs.p, nb, "gram");
   } else {
     // Gram matrices of the complex64 block on the tensor cores: exact products of the FP32 values
     // (4 digits each), summed exactly per chunk and in FP64 across chunks, delivered in FP64
-    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, MY, npw, s->S.p, nb, 1, 0, 0, 0, "gram", nullptr, false, true);
-    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, HY, npw, s->Hs.p, nb, 1, 0, 0, 0, "gram", nullptr, false, true);
+    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, MY, npw, s->S.p, nb, 1, 0, 0, 0, "gram", nullptr, false, true, 0, true);
+    oz_gemm_cn(ctx, nb, nb, npw, Y, npw, HY, npw, s->Hs.p, nb, 1, 0, 0, 0, "gram", nullptr, false, true, 0, true);
   }
   subspace_eig(s, ctx);  // real symmetric at Gamma (real-space-real blocks)
   if (f64) {

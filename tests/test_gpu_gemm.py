@@ -226,3 +226,21 @@ def test_small_fp64_products(ctx, op, M, N, Kd, alpha, beta):
     torch.cuda.synchronize()
     bound = (4 * Kd + 16) * 2.0 ** -53 * (abs(alpha) * (np.abs(Am) @ np.abs(B.T)) + abs(beta) * np.abs(C0.T))
     assert np.all(np.abs(tC.cpu().numpy().T - ref) <= 2 * bound)
+
+
+@pytest.mark.parametrize("M,Kd", [(64, 4000), (65, 4000), (130, 1200), (300, 200), (564, 6000)])
+@pytest.mark.parametrize("alpha,beta", [(1.0, 0.0), (0.6 + 0.3j, -0.4 + 0.2j)])
+def test_block_with_itself(ctx, M, Kd, alpha, beta):
+    """A^H A in FP64 forms the tiles on and below the diagonal and mirrors them: within the digit form's
+    1e-12 of the numpy product at tile edges, remainders and with a K split, and exactly Hermitian."""
+    import torch
+    rng = np.random.default_rng(M + Kd)
+    A, C0 = crand(rng, (M, Kd)), crand(rng, (M, M))
+    ref = alpha * (A.conj() @ A.T) + beta * C0.T
+    tA, tC = torch.from_numpy(A).cuda(), torch.from_numpy(C0).cuda()
+    K.kss_gemm(ctx, 0, tA, tA, tC, alpha, beta, K.KSS_PREC_FP64)
+    torch.cuda.synchronize()
+    got = tC.cpu().numpy().T
+    assert np.max(np.abs(got - ref)) < 1e-12 * np.max(np.abs(ref))
+    if beta == 0:
+        assert np.array_equal(got, got.conj().T)
