@@ -107,7 +107,7 @@ template <int SA, int SB, typename CT>
 __global__ void __launch_bounds__(kOzThreads, 1)
 oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int rowsA,
                int rowsB, int Mr, int Nr, int tnn, int herm, int kb_per_split, int kb_total, const int* __restrict__ ea,
-               const int* __restrict__ eb, int* __restrict__ err, double* __restrict__ part,
+               const int* __restrict__ eb, int ebs, int* __restrict__ err, double* __restrict__ part,
                CT* __restrict__ C, long long ldc, double ar, double ai, double br, double bi) {
   pdl_wait();
   constexpr uint32_t STAGE = OzCfg<SA, SB>::STAGE;
@@ -276,7 +276,7 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // value a1 2^(E - 28) + a2 2^(E - 56), both put into the fraction of a number with that unit (a1
         // around 1.5 2^52: below 2^50 for as many chunks as a split takes), whose exponent also takes E
         // as far as it fits; rounded once
-        const int E = er + eb[col], Ec = max(-980, min(980, E));
+        const int E = er + eb[col * ebs], Ec = max(-980, min(980, E));
         const long long hi = a1[j] + (a2[j] >> 28), lo = a2[j] & ((1LL << 28) - 1);
         const long long b1 = ((long long)(1023 + 52 - 28 + Ec) << 52) + (1LL << 51);
         const long long b2 = (long long)(1023 + 52 - 56 + Ec) << 52;
@@ -520,11 +520,11 @@ __global__ void oz_combine(const double* __restrict__ P, int nsplit, int Mr, int
   *dst = r;
 }
 
-CUtensorMap make_map(const void* base, long long rows, int kt, int box_rows) {
+CUtensorMap make_map(const void* base, long long rows, int kt, int box_rows, int pitch = 1) {
   CUtensorMap m;
   std::memset(&m, 0, sizeof(m));
   const cuuint64_t dims[2] = {(cuuint64_t)kt, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)kt * 2};
+  const cuuint64_t strides[1] = {(cuuint64_t)kt * 2 * pitch};
   const cuuint32_t box[2] = {(cuuint32_t)TK, (cuuint32_t)box_rows};
   const cuuint32_t es[2] = {1, 1};
   const CUresult r = tc::encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims,
@@ -569,7 +569,7 @@ void launch_oz(kss_ctx ctx, const OzOperand& a, const OzOperand& b, int M, int N
   int plan = 1;
   if (tiles < nsm) plan = (int)std::max(1LL, std::min<long long>(nsm / tiles, kb_total / (2 * CHUNK)));
   const CUtensorMap ma = make_map(a.planes, (long long)SA * a.rows, a.KT, TM);
-  const CUtensorMap mb = make_map(b.planes, (long long)SB * b.rows, b.KT, TN);
+  const CUtensorMap mb = make_map(b.planes, (long long)SB * b.rows, b.KT, TN, b.pitch);
   auto kern = oz_gemm_kernel<SA, SB, CT>;
   KSS_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM));
   const std::string name = std::string(SA == 7 ? "tc_gemm_oz7:" : "tc_gemm_oz4:") + tag;
@@ -583,9 +583,9 @@ void launch_oz(kss_ctx ctx, const OzOperand& a, const OzOperand& b, int M, int N
     if (!fused) ctx->oz_part.ensure((size_t)splits * Mr * Nr * sizeof(double));
     {
       ProfScope ps(ctx, prof ? prof_register(name.c_str()) : prof_register("gemm_tuning"));
-      launch_pdl(
-          kern, dim3((unsigned)tiles, splits, 1), kOzThreads, Cfg::SMEM, ctx->stream, ma, mb, a.rows, b.rows, Mr, Nr, tnn, herm ? 1 : 0, kps, kb_total, a.e, b.e, err_flag(ctx),
-          fused ? nullptr : ctx->oz_part.as<double>(), Cd, ldd, ar, ai, br_, bi_);
+      launch_pdl(kern, dim3((unsigned)tiles, splits, 1), kOzThreads, Cfg::SMEM, ctx->stream, ma, mb, a.rows, b.rows, Mr,
+                 Nr, tnn, herm ? 1 : 0, kps, kb_total, a.e, b.e, b.pitch, err_flag(ctx),
+                 fused ? nullptr : ctx->oz_part.as<double>(), Cd, ldd, ar, ai, br_, bi_);
     }
     KSS_CHECK_CUDA(cudaGetLastError());
     if (fused) return;
@@ -700,10 +700,19 @@ void oz_gemm_cn(kss_ctx ctx, int M, int N, int K, const void* A, int lda, const 
     ctx->oz_a.ensure(oz_operand_bytes(2 * M, K, S));
     a = oz_prepare(ctx, OZ_CN_A, M, K, A, lda, ctx->oz_a.p, f64in, S);
   }
-  ctx->oz_b.ensure(oz_operand_bytes(N, K, S));
-  const OzOperand b = oz_prepare(ctx, OZ_B, N, K, B, ldb, ctx->oz_b.p, f64in, S);
-  // a block with itself is Hermitian: half the tiles (564 x 564 x 34181: 2.47 -> 1.33 ms)
-  herm = M == N && (herm || (A == B && lda == ldb && !a_pre));
+  // A block with itself: Hermitian, half the tiles (564 x 564 x 34181: 2.47 -> 1.33 ms), and its B rows
+  // are the even rows of the A planes
+  const bool self = A == B && lda == ldb && M == N && !a_pre;
+  herm = M == N && (herm || self);
+  OzOperand b;
+  if (self) {
+    b = a;
+    b.rows = N;
+    b.pitch = 2;
+  } else {
+    ctx->oz_b.ensure(oz_operand_bytes(N, K, S));
+    b = oz_prepare(ctx, OZ_B, N, K, B, ldb, ctx->oz_b.p, f64in, S);
+  }
   run_oz(ctx, a, b, M, N, C, f64out, ldc, ar, ai, br, bi, tag, herm);
 }
 

@@ -760,9 +760,9 @@ void run_tc(kss_ctx ctx, const __nv_bfloat16* Atc, const __nv_bfloat16* Btc, int
     {
       ProfScope ps(ctx, prof_register(prof ? name.c_str() : "gemm_tuning"));
       if (ch.form == 0) {
-        launch_pdl(
-            tc_gemm_kernel, dim3((unsigned)tiles, splits, 1), kTcThreads, kTcSmem, ctx->stream, ma, mb, ctx->tc_part.as<float>(), Mr, Nr, tnn, kps, kb_total, Kp, ctx->tc_err.as<int>(),
-            fused ? Cd : nullptr, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
+        launch_pdl(tc_gemm_kernel, dim3((unsigned)tiles, splits, 1), kTcThreads, kTcSmem, ctx->stream, ma, mb,
+                   ctx->tc_part.as<float>(), Mr, Nr, tnn, kps, kb_total, Kp, ctx->tc_err.as<int>(),
+                   fused ? Cd : nullptr, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
         KSS_CHECK_CUDA(cudaGetLastError());
       } else {
         const int tnp = ch.form == 2 ? 64 : 128;
@@ -796,8 +796,8 @@ void run_tc(kss_ctx ctx, const __nv_bfloat16* Atc, const __nv_bfloat16* Btc, int
     if (fused) return;
     const long long mn = (long long)M * N;
     ProfScope ps(ctx, prof_register(prof ? cname.c_str() : "gemm_tuning"));
-    launch_pdl(
-        tc_combine, (unsigned)((mn + 255) / 256), 256, 0, ctx->stream, ctx->tc_part.as<float>(), splits, Mr, Nr, M, N, Cd, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
+    launch_pdl(tc_combine, (unsigned)((mn + 255) / 256), 256, 0, ctx->stream, ctx->tc_part.as<float>(), splits, Mr, Nr, M,
+               N, Cd, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
     KSS_CHECK_CUDA(cudaGetLastError());
   };
   // Candidates: every form with no split, the plan and the splits filling one to three waves.  Each

@@ -70,6 +70,7 @@ struct OzOperand {
   int* e = nullptr;
   int rows = 0, KT = 0;
   int S = 7;                       // digits per value: 7 (complex128 data) or 4 (complex64 data)
+  int pitch = 1;  // rows of the planes (and of e) from one operand row to the next
 };
 
 // Per-k-point data.
