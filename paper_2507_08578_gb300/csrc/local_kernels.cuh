@@ -5,7 +5,7 @@
 
 #include <algorithm>
 
-#include "fft_reg.cuh"
+#include "fft_f2.cuh"
 #include "kss_internal.h"
 
 namespace kss {
