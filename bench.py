@@ -253,13 +253,13 @@ def run_reference(args, rank: int):
 # ncu DRAM bytes per band of the middle pass (production schedule 12 x 8 at 384 threads, pruned
 # stages) with the L2 state the step leaves (--cache-control none; a full-chunk production launch:
 # profiles/c2_pass_b_dram_traffic.md)
-PASS_B_DRAM_PER_BAND = {"fp64": (19.000832e6 + 47.424256e6) / 27, "mixed": (9.314304e6 + 41.612032e6) / 54}
-PASS_B_SCHEDULE = {"fp64": "12x8 @384", "mixed": "12x8 @384"}
+# (single precision; the fixed-point pass of double precision has not been counted)
+PASS_B_DRAM_PER_BAND = {"mixed": (9.314304e6 + 41.612032e6) / 54}
+PASS_B_SCHEDULE = {"mixed": "12x8 @384"}
 # FP instructions the middle pass executes per band (ncu counts: 2 per FMA, 1 per add / multiply)
 # over the dense-transform count 4 x 5 N^3 log2 N, for the production schedule (12 x 8 at 384
 # threads with the pruned strided stages, CW = 3)
-PASS_B_EXECUTED_PER_ALGORITHMIC = {"fp64": (2 * 349526016 + 685449216 + 207194112) / 27 / (4 * 5 * 96 ** 3 * math.log2(96)),
-                                   "mixed": (2 * 707014656 + 1399762944 + 439271424) / 54 / (4 * 5 * 96 ** 3 * math.log2(96))}
+PASS_B_EXECUTED_PER_ALGORITHMIC = {"mixed": (2 * 707014656 + 1399762944 + 439271424) / 54 / (4 * 5 * 96 ** 3 * math.log2(96))}
 
 
 def algorithmic_work(s, npw, nb, degree, box, applies, rr_calls):
@@ -566,7 +566,8 @@ def run_ours(args, rank: int, world: int, local_rank: int):
         roof = {"kernel": dom, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak, "traffic": None,
                 "peak_note": ("FP64 CUDA-core rate derived from the unit counts and clock: 152 SMs x "
-                              "2 FP64 FMA per clock x 2 flops x 2070 MHz = 1.26, nominal 1.25"
+                              "2 FP64 FMA per clock x 2 flops x 2070 MHz = 1.26, nominal 1.25; the passes "
+                              "run in 64-bit fixed point on the integer pipes, so frac can exceed 1"
                               if args.form == "fp64" else
                               "FP32 CUDA-core rate derived from 152 SMs x 128 lanes x 2 x 2070 MHz"),
                 "measured_peak": probe, "frac_of_measured": ach / probe,
@@ -578,7 +579,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
                                       "note": "the longest kernel family of the step is not an FFT pass"}
         roof["fft_path_hbm"] = fft_path_hbm(fam, applies, npw, 16 if args.form == "fp64" else 8, hbm_peak()[0])
         sched_now = [f"{e['A']}x{e['B']} @{e['threads']}" for e in K.kss_autotune_table() if e["N"] == 96]
-        if dom == "local_pass_b" and args.workload == "c2" and sched_now and \
+        if dom == "local_pass_b" and args.form == "mixed" and args.workload == "c2" and sched_now and \
                 all(x == PASS_B_SCHEDULE[args.form] for x in sched_now):
             # FP instructions the pruned pass executes (ncu counts of this schedule) over the
             # dense-transform count: the executed rate against the measured FMA throughput
@@ -678,8 +679,8 @@ def run_ours(args, rank: int, world: int, local_rank: int):
     sched = [f"{e['N1']}x{e['N']}^2 W3<={e['W3']}: {e['A']}x{e['B']} @{e['threads']} "
              f"({e['ncand']} timed)" for e in table]
     c2_sched = [f"{e['A']}x{e['B']} @{e['threads']}" for e in table if e["N"] == 96 and e["N1"] == 96]
-    if roof is not None and roof["kernel"] == "local_pass_b" and args.workload == "c2" and c2_sched and \
-            all(x == PASS_B_SCHEDULE[args.form] for x in c2_sched):
+    if roof is not None and roof["kernel"] == "local_pass_b" and args.form == "mixed" and args.workload == "c2" and \
+            c2_sched and all(x == PASS_B_SCHEDULE[args.form] for x in c2_sched):
         roof["traffic"] = PASS_B_DRAM_PER_BAND[args.form] * applies / roof["launches"]
         roof["traffic_note"] = ("DRAM bytes per launch: ncu bytes per band of this kernel and schedule (L2 as "
                                 "the step leaves it) x the bands per launch of this run")
