@@ -268,7 +268,8 @@ kss_status kss_apply_H_noalloc(kss_sys sys, int ik, int nb, const void* psi, voi
  *   op 0: C = alpha A^H B + beta C, A is K x M (lda >= K), B is K x N (ldb >= K)
  *   op 1: C = alpha A B + beta C,   A is M x K (lda >= M), B is K x N (ldb >= K)
  * Column-major DEVICE matrices; C is M x N (ldc >= M) and must not overlap A or B.
- * KSS_PREC_FP64: complex128 on the FP64 pipe.  KSS_PREC_MIXED: complex64 on the tensor cores,
+ * KSS_PREC_FP64: complex128, as exact digit products on the tensor cores (small products on the
+ * FP64 pipe).  KSS_PREC_MIXED: complex64 on the tensor cores,
  * every FP32 value split into BF16 hi + lo, products hi*hi + hi*lo + lo*hi accumulated in FP32
  * (relative error of order 1e-5).  Errors: KSS_EINVAL, KSS_ETIMEOUT (a bounded device wait gave
  * up; the context stays usable). */
@@ -288,7 +289,7 @@ kss_status kss_gemm(kss_ctx ctx, int op, int M, int N, int K, const void* A, int
  * undefined).  real != 0: the pencils are real symmetric (imaginary parts ignored; solved in
  * real arithmetic; eigenvectors and factor written with zero imaginary parts).  Hand-written
  * kernels (Cholesky, reduction to standard form, Householder tridiagonalisation, bisection and
- * inverse iteration, back-transformation): one CTA per pencil, or a cooperative grid for a
+ * inverse iteration, back-transformation): one CTA or a cluster of them per pencil, a cooperative grid for a
  * single pencil of order >= 32.  Synchronises the context stream.
  * Errors: KSS_EINVAL (count < 0, NULL arrays, bad sizes), KSS_ETIMEOUT (a bounded grid-barrier
  * wait gave up), KSS_ECUDA. */

@@ -654,7 +654,8 @@ __global__ void prep_mmajor(const float2* __restrict__ src, long long ld, int M,
 // C (complex, col-major ldc) = alpha * D + beta * C with D assembled from the K-split partials
 // (col-major Mr x Nr, Mr = 2M): re = D(2i, j), im = D(2i + 1, j).
 __global__ void tc_combine(const float* __restrict__ P, int nsplit, int Mr, int Nr, int M, int N,
-                           float2* __restrict__ C, long long ldc, float ar, float ai, float br, float bi) {
+                           float2* __restrict__ C, long long ldc, float ar, float ai, float br, float bi,
+                           const float* __restrict__ rs, float s) {
   pdl_wait();
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (idx >= (long long)M * N) return;
@@ -675,6 +676,11 @@ __global__ void tc_combine(const float* __restrict__ P, int nsplit, int Mr, int 
     const float2 o2 = *dst;
     out.x += br * o2.x - bi * o2.y;
     out.y += br * o2.y + bi * o2.x;
+  }
+  if (rs) {
+    const float f = rs[i] * s;
+    out.x *= f;
+    out.y *= f;
   }
   *dst = out;
 }
@@ -725,8 +731,10 @@ void ensure_err(kss_ctx ctx) {
 // products: written by the GEMM kernel itself without a K-split, else through partial sums.
 // Schedule: form 0 (one CTA per 128 x 128 tile and split, tc_gemm_kernel) or the persistent
 // kernel on 128- (form 1) or 64-column (form 2) tiles, and the K-split; autotuned per shape.
+// Rows of the result are scaled by rs[i] s when rs is given (by the combine kernel where there is one).
 void run_tc(kss_ctx ctx, const __nv_bfloat16* Atc, const __nv_bfloat16* Btc, int Kp, int M, int N,
-            float2* C, int ldc, double ar, double ai, double br, double bi, const char* tag) {
+            float2* C, int ldc, double ar, double ai, double br, double bi, const char* tag,
+            const float* rs = nullptr, double s = 1.0) {
   const int Mr = 2 * M, Nr = N;
   const int tmn = (Mr + TM - 1) / TM, tnn = (Nr + TN - 1) / TN;
   const int kb_total = Kp / TK;
@@ -793,11 +801,14 @@ void run_tc(kss_ctx ctx, const __nv_bfloat16* Atc, const __nv_bfloat16* Btc, int
         else launch_persist<128>(ctx, args, grid);
       }
     }
-    if (fused) return;
+    if (fused) {
+      if (prof && rs) scale_rows(ctx, false, M, N, Cd, ldd, rs, s);
+      return;
+    }
     const long long mn = (long long)M * N;
     ProfScope ps(ctx, prof_register(prof ? cname.c_str() : "gemm_tuning"));
     launch_pdl(tc_combine, (unsigned)((mn + 255) / 256), 256, 0, ctx->stream, ctx->tc_part.as<float>(), splits, Mr, Nr, M,
-               N, Cd, ldd, (float)ar, (float)ai, (float)br_, (float)bi_);
+               N, Cd, ldd, (float)ar, (float)ai, (float)br_, (float)bi_, prof ? rs : nullptr, (float)s);
     KSS_CHECK_CUDA(cudaGetLastError());
   };
   // Candidates: every form with no split, the plan and the splits filling one to three waves.  Each
@@ -893,10 +904,11 @@ const __nv_bfloat16* prep_b(kss_ctx ctx, int N, int K, const void* B, int ldb) {
 }  // namespace
 
 void tc_gemm_cn_split(kss_ctx ctx, int M, int N, int K, const void* Atc, const void* B, int ldb, void* C, int ldc,
-                      double ar, double ai, double br, double bi, const char* tag) {
+                      double ar, double ai, double br, double bi, const char* tag, const float* row_scale, double s) {
   if (M <= 0 || N <= 0 || K <= 0) return;
   const __nv_bfloat16* Btc = prep_b(ctx, N, K, B, ldb);
-  run_tc(ctx, (const __nv_bfloat16*)Atc, Btc, kpad(K), M, N, (float2*)C, ldc, ar, ai, br, bi, tag);
+  run_tc(ctx, (const __nv_bfloat16*)Atc, Btc, kpad(K), M, N, (float2*)C, ldc, ar, ai, br, bi, tag,
+         row_scale, s);
 }
 
 void tc_gemm_nn_split(kss_ctx ctx, int M, int N, int K, const void* Atc, const void* B, int ldb, void* C, int ldc,

@@ -384,7 +384,8 @@ size_t tc_split_nn_bytes(int M, int K);
 void tc_split_cn(kss_ctx ctx, int M, int K, const void* A, int lda, void* Atc);
 void tc_split_nn(kss_ctx ctx, int M, int K, const void* A, int lda, void* Atc);
 void tc_gemm_cn_split(kss_ctx ctx, int M, int N, int K, const void* Atc, const void* B, int ldb, void* C, int ldc,
-                      double ar, double ai, double br, double bi, const char* tag);
+                      double ar, double ai, double br, double bi, const char* tag,
+                      const float* row_scale = nullptr, double s = 1.0);
 void tc_gemm_nn_split(kss_ctx ctx, int M, int N, int K, const void* Atc, const void* B, int ldb, void* C, int ldc,
                       double ar, double ai, double br, double bi, const char* tag);
 // C (complex128) = A^H B for complex64 A, B with FP64 accumulation.

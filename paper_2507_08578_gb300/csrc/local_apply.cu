@@ -957,8 +957,9 @@ void apply_h(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev, v
               0.0, 0.0, "cprj");
     else
       tc_gemm_cn_split(ctx, s->nproj, nb, kd.npw, beta_split_cn(s, ik), psi, ld, ctx->ws_cprj.p, s->nproj,
-                       1.0, 0.0, 0.0, 0.0, "cprj");
-    if (!small)
+                       1.0, 0.0, 0.0, 0.0, "cprj", s->d_D32.as<float>(), c.alpha);
+    // (the small and the split-BF16 products scale as they add up their partial sums)
+    if (!small && (f64 || c.fp32_proj))
       scale_rows(ctx, f64, s->nproj, nb, ctx->ws_cprj.p, s->nproj, f64 ? s->d_D64.p : s->d_D32.p, c.alpha);
   }
   if (f64)
