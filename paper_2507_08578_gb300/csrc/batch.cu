@@ -20,6 +20,7 @@
 #include "batch_kernels.cuh"
 #include "local_fused.h"
 #include "local_kernels.cuh"
+#include "local_wide.h"
 #include "tune.h"
 
 namespace kss {
@@ -93,6 +94,7 @@ void fill_args(kss_sys s, int ik, LocalArgs<T>& a) {
   a.Vx = (const T*)(f64 ? s->d_Vx64.p : s->d_Vx32.p);
   a.ld = kd.npw;
   a.n0 = 0;
+  if (f64) fx_args(s, a.fx);
 }
 
 size_t al256(size_t n) { return (n + 255) & ~(size_t)255; }

@@ -429,13 +429,6 @@ int chunk_bands(kss_sys s, int ik, int nb, size_t es) {
   return (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, target / per));
 }
 
-void fx_args(kss_sys s, FxTables& f) {
-  f.r1 = s->d_rot[0].as<fx::Rot>();
-  f.r2 = s->d_rot[1].as<fx::Rot>();
-  f.vhigh = s->d_vhigh.as<int>();
-  f.invn = 1.0 / ((double)s->N[0] * s->N[1] * s->N[2]);
-}
-
 // Double precision: whether the passes of `a` run in fixed point (all three or none: the slab
 // between them is in that form).  The CTA-wide schedule of the tuner and an instance for the x edge.
 template <typename T>
@@ -740,6 +733,13 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
 }
 
 }  // namespace
+
+void fx_args(kss_sys s, FxTables& f) {
+  f.r1 = s->d_rot[0].as<fx::Rot>();
+  f.r2 = s->d_rot[1].as<fx::Rot>();
+  f.vhigh = s->d_vhigh.as<int>();
+  f.invn = 1.0 / ((double)s->N[0] * s->N[1] * s->N[2]);
+}
 
 template <typename T>
 void warp_pass_b(kss_ctx ctx, const LocalArgs<T>& a, int nbands) {

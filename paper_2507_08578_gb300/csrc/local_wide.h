@@ -21,6 +21,11 @@ bool wide_pass_b(const lk::LocalArgs<T>& a, int A, int B, int nt, int nbands, cu
 template <typename T>
 bool wide_pass_x(const lk::LocalArgs<T>& a, int which, int nbands, cudaStream_t st, bool dry);
 
+// Tables of the fixed-point passes that belong to the system (not V and the exponents, which go with a
+// schedule and a slab).  Every LocalArgs<double> carries them: whoever asks the tuner for a schedule
+// has it time the fixed-point pass.
+void fx_args(kss_sys s, lk::FxTables& f);
+
 // The (A, B) pairs with instances, in KSS_WIDE_SPLITS order.
 inline const std::vector<std::pair<int, int>>& wide_splits() {
   static const std::vector<std::pair<int, int>> v = {

@@ -56,6 +56,9 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   KSS_CHECK_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) return builtin<T>(a, s2);
 
+  // (in double precision the candidates are the fixed-point passes)
+  KSS_REQUIRE(sizeof(T) == 4 || (a.fx.r2 && a.fx.vhigh), "pass-B tuner: arguments without the fixed-point tables");
+
   using C = typename lk::CT<T>::C;
   lk::LocalArgs<T> t = a;
   t.W3 = W3b;

@@ -311,3 +311,37 @@ def test_config4_full_batch_mixed(ctx):
     finally:
         for h in handles:
             K.kss_sys_destroy(h)
+
+
+@pytest.mark.parametrize("how", ["cleared", "switched_on"])
+def test_server_tunes_between_pumps(ctx, how):
+    """A double-precision server whose schedule table is emptied between pumps, or whose tuning is
+    switched on between them: the batch engine itself then asks the tuner for the schedules of the
+    running units (their first applications, which usually did, lie behind).  Same levels as ever."""
+    opts = K.make_opts(tol=1e-9, seed=3)
+    systems = small_systems()
+    K.kss_autotune_clear()
+    K.kss_autotune_set(ctx, 0 if how == "switched_on" else 1)
+    K.kss_server_start(ctx, 8 << 30, 64, opts)
+    try:
+        tickets = [submit(ctx, s) for s in systems[:2]]
+        for _ in range(2):
+            K.kss_server_pump(ctx, 1e-3)  # one lockstep iteration
+        assert all(K.kss_server_poll(ctx, t, len(s.kpts), s.nband) is None for t, s in zip(tickets, systems))
+        if how == "cleared":
+            K.kss_autotune_clear()
+        else:
+            assert K.kss_autotune_table() == []
+            K.kss_autotune_set(ctx, 1)
+        tickets.append(submit(ctx, systems[2]))  # the set of active units changes
+        res = drain(ctx, tickets, [(len(s.kpts), s.nband) for s in systems])
+        tuned = {(e["N1"], e["N"]) for e in K.kss_autotune_table()}
+    finally:
+        K.kss_server_stop(ctx)
+        K.kss_autotune_set(ctx, 1)
+        K.kss_autotune_clear()
+    for s, r in zip(systems, res):
+        box = O.system_box(s)
+        assert (box[0], box[1]) in tuned
+        for ik in range(len(s.kpts)):
+            assert np.max(np.abs(r[1][ik] - oracle_levels(s, ik, s.nband))) < 1e-8
