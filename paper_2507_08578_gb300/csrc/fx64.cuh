@@ -129,6 +129,7 @@ __device__ __forceinline__ long long mulc(long long a, Limbs c) {
 // every point of a plane, and a transform collects those of all N^3 points in its G = 0 output
 // (measured: 4e-14 of the rms there, 100 times the error of the others).
 __device__ __forceinline__ long long half(long long a) { return (a + ((unsigned)a >> 1 & 1u)) >> 1; }
+// (a + 2^(s - 1) must be in range)
 __device__ __forceinline__ long long shr_round(long long a, int s) {
   return (a + ((1LL << (s - 1)) - 1) + ((a >> s) & 1)) >> s;
 }
@@ -184,10 +185,16 @@ __device__ __forceinline__ Cx shift(Cx v, int s) {
   return Cx{v.x << -s, v.y << -s};
 }
 
-// a 2^s (s <= 0: left shift by -s, which must not overflow; s > 0: rounded right shift)
+// a 2^s (s <= 0: left shift by -s, which must not overflow; s > 0: rounded right shift), |a| < 2^62.8.
+// shr_round adds half a unit first, which from s = 61 on would leave the range: those shifts round what
+// they drop by itself.
 __device__ __forceinline__ long long scale2(long long a, int s) {
   if (s <= 0) return a << (s < -63 ? 63 : -s);
-  return s > 62 ? 0 : shr_round(a, s);
+  if (s <= 60) return shr_round(a, s);
+  if (s > 63) return 0;
+  const long long q = a >> s;
+  const unsigned long long low = (unsigned long long)a & ((1ULL << s) - 1);
+  return q + (long long)((low + ((1ULL << (s - 1)) - 1) + (unsigned long long)(q & 1)) >> s);
 }
 
 // A double x = +-m 2^(e - 1075) as an integer multiple of 2^E, rounded; |x| < 2^(E + 63) (finite x)
