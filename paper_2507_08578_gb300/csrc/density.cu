@@ -217,7 +217,7 @@ void density_t(kss_sys s, int ik, int nb, const void* psi, int ld, const double*
   // bands: 9.8 ms, 33.9 on the FP64 pipe)
   bool fx = false;
   if constexpr (sizeof(T) == 8)
-    fx = wide_pass_x<T>(args, 0, 0, nullptr, true) &&
+    fx = fx_pass_x(args, 0, 0, nullptr, true) &&
          density_pass_fx(args, sp.A, sp.B, 0, 1, nullptr, nullptr, nullptr, &resident);
   if (!fx && !pass_d<T>(args, sp.A, sp.B, 0, 1, nullptr, nullptr, nullptr, true, &resident))
     fail(KSS_ENOTSUP, "no density kernel instance for this FFT length / window");

@@ -18,8 +18,9 @@
 //     (local_wide.cu), every transform stage spread over all lanes of the CTA;
 //   * passes A/C (and pass B otherwise) with a compile-time split: per-warp two-level register
 //     codelets (fft_reg.cuh, CtPol), else the same with runtime sizes (RtPol);
-//   * double precision with a CTA-wide pass B and an x edge of KSS_FX_X: all three passes in fixed
-//     point (local_fx.cuh), 3 to 4 times the FP64 pipe's rate; other boxes in FP64;
+//   * double precision with N2 = N3, a CTA-wide pass B and an x edge of KSS_FX_X: all three passes in
+//     fixed point (local_fx.cuh), 3 to 4 times the FP64 pipe's rate; other boxes in FP64, in the same
+//     CTA-wide forms where they have instances;
 //   * lengths that do not split into two codelets of size <= 16: warp-level Stockham FFTs
 //     (radix 4/2/3/5) on contiguous pencils in shared memory (the kernels in this file).
 // The slab lives in a workspace of nc bands (chunked so that it stays L2-resident).
@@ -429,15 +430,22 @@ int chunk_bands(kss_sys s, int ik, int nb, size_t es) {
   return (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, target / per));
 }
 
-// Double precision: whether the passes of `a` run in fixed point (all three or none: the slab
-// between them is in that form).  The CTA-wide schedule of the tuner and an instance for the x edge.
+// The CTA-wide form of pass B and of passes A (which = 0) and C (1), in fixed point (fx) or in the
+// data's own precision.  False, and nothing launched, when the schedule or the box has none.
 template <typename T>
-bool fx_passes(const LocalArgs<T>& a, const PassBSched& sb) {
-  if constexpr (sizeof(T) == 8)
-    return sb.threads && wide_pass_b<T>(a, sb.A, sb.B, sb.threads, 0, nullptr, true) &&
-           wide_pass_x<T>(a, 0, 0, nullptr, true) && wide_pass_x<T>(a, 1, 0, nullptr, true);
-  else
-    return false;
+bool wide_b(const LocalArgs<T>& a, const PassBSched& sb, bool fx, int m, cudaStream_t st, bool dry = false) {
+  if (!sb.threads) return false;
+  if constexpr (sizeof(T) == 8) {
+    if (fx) return fx_pass_b(a, sb.A, sb.B, sb.threads, m, st, dry);
+  }
+  return wide_pass_b<T>(a, sb.A, sb.B, sb.threads, m, st, dry);
+}
+template <typename T>
+bool wide_x(const LocalArgs<T>& a, int which, bool fx, int m, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (fx) return fx_pass_x(a, which, m, st, false);
+  }
+  return wide_pass_x<T>(a, which, m, st, false);
 }
 
 // Kernel arguments of the local passes for (system, k-point, band block).
@@ -558,14 +566,10 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
         launch_pdl(kk.b, dim3(t.N1, m), kThreads, rb, ctx->stream, t, rp, scr_warp);
       };
       PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, true);
-      bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
-      if (f64) {
-        wx = fx_passes<T>(a, sb);
-        if (wx) a.fx.V = (const fx::Limbs*)vfx_view(s, sb.A, sb.B);
-        else sb.threads = 0;
-      } else if (sb.threads) {
-        a.Vpi = (const T*)vpi_view(s, sb.A, sb.B, false);
-      }
+      // all three passes in fixed point or none
+      const bool fx = fx_available_t(a) && wide_b(a, sb, true, 0, nullptr, true);
+      if (fx) a.fx.V = (const fx::Limbs*)vfx_view(s, sb.A, sb.B);
+      else if (wide_b(a, sb, false, 0, nullptr, true)) a.Vpi = (const T*)vpi_view(s, sb.A, sb.B, f64);
       static const int ida = prof_register(f64 ? "local_pass_a<f64>" : "local_pass_a<f32>");
       static const int idb = prof_register(f64 ? "local_pass_b<f64>" : "local_pass_b<f32>");
       static const int idc = prof_register(f64 ? "local_pass_c<f64>" : "local_pass_c<f32>");
@@ -586,16 +590,16 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
         a.n0 = n0;
         {
           ProfScope ps(ctx, ida);
-          if (!(wx && wide_pass_x<T>(a, 0, m, ctx->stream, false)))
+          if (!wide_x(a, 0, fx, m, ctx->stream))
             launch_pdl(kk.a, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
         }
         {
           ProfScope ps(ctx, idb);
-          if (!(sb.threads && wide_pass_b<T>(a, sb.A, sb.B, sb.threads, m, ctx->stream, false))) warp_b(a, m);
+          if (!wide_b(a, sb, fx, m, ctx->stream)) warp_b(a, m);
         }
         {
           ProfScope ps(ctx, idc);
-          if (!(wx && wide_pass_x<T>(a, 1, m, ctx->stream, false)))
+          if (!wide_x(a, 1, fx, m, ctx->stream))
             launch_pdl(kk.c, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
         }
       }
@@ -690,26 +694,27 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
         launch_pdl(kk.b, dim3(t.N1, m), kThreads, rb, ctx->stream, t, rp, scr_warp);
       };
       PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, false);  // no tuning here
-      bool wx = wide_pass_x<T>(a, 0, 0, nullptr, true);
-      // The CTA-wide form needs V in its split's layout; that view is built (allocated) by the
-      // first ordinary application, and without it this path takes the per-warp form.
-      if (f64) {
+      // The CTA-wide forms need V in their split's layout; that view is built (allocated) by the first
+      // ordinary application, and without it this path takes the per-warp form.
+      bool fx = false;
+      if (meta && fx_available_t(a) && wide_b(a, sb, true, 0, nullptr, true)) {
         auto it = s->vfx.find(sb.A * 32 + sb.B);
-        wx = meta && it != s->vfx.end() && fx_passes<T>(a, sb);
-        if (wx) a.fx.V = it->second.template as<fx::Limbs>();
-        else sb.threads = 0;
-      } else if (sb.threads) {
-        auto it = s->vpi32.find(sb.A * 32 + sb.B);
-        if (it != s->vpi32.end()) a.Vpi = (const T*)it->second.p;
+        fx = it != s->vfx.end();
+        if (fx) a.fx.V = it->second.template as<fx::Limbs>();
+      }
+      if (!fx && sb.threads) {
+        auto& cache = f64 ? s->vpi64 : s->vpi32;
+        auto it = cache.find(sb.A * 32 + sb.B);
+        if (it != cache.end()) a.Vpi = (const T*)it->second.p;
         else sb.threads = 0;
       }
       for (int n0 = 0; n0 < nb; n0 += nc) {
         const int m = std::min(nc, nb - n0);
         a.n0 = n0;
-        if (!(wx && wide_pass_x<T>(a, 0, m, ctx->stream, false)))
+        if (!wide_x(a, 0, fx, m, ctx->stream))
           launch_pdl(kk.a, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
-        if (!(sb.threads && wide_pass_b<T>(a, sb.A, sb.B, sb.threads, m, ctx->stream, false))) warp_b(a, m);
-        if (!(wx && wide_pass_x<T>(a, 1, m, ctx->stream, false)))
+        if (!wide_b(a, sb, fx, m, ctx->stream)) warp_b(a, m);
+        if (!wide_x(a, 1, fx, m, ctx->stream))
           launch_pdl(kk.c, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
       }
       KSS_CHECK_CUDA(cudaGetLastError());
@@ -787,7 +792,7 @@ void pass_a_chunks(kss_sys s, int ik, int nb, LocalArgs<T> a, bool fx,
     a.n0 = n0;
     {
       ProfScope ps(ctx, ida);
-      if (fx) wide_pass_x<T>(a, 0, m, ctx->stream, false);
+      if (fx) wide_x(a, 0, true, m, ctx->stream);
       else launch_pdl(kk.a, dim3(a.W3, m), kThreads, ra, ctx->stream, a, rp, scr_warp);
     }
     after(a, m);

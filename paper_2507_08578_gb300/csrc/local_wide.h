@@ -1,4 +1,5 @@
-// Host entry of the CTA-wide pass B instances (local_wide_impl.cuh).
+// Host entries of the CTA-wide passes (local_wide_impl.cuh) and of their fixed-point form in double
+// precision (local_fx_impl.cuh).
 #pragma once
 
 #include "local_kernels.cuh"
@@ -20,6 +21,19 @@ bool wide_pass_b(const lk::LocalArgs<T>& a, int A, int B, int nt, int nbands, cu
 // its shared memory does not fit; dry = true only checks availability.
 template <typename T>
 bool wide_pass_x(const lk::LocalArgs<T>& a, int which, int nbands, cudaStream_t st, bool dry);
+
+// The same in fixed point: pass B (256 or 384 threads), passes A and C.
+bool fx_pass_b(const lk::LocalArgs<double>& a, int A, int B, int nt, int nbands, cudaStream_t st, bool dry);
+bool fx_pass_x(const lk::LocalArgs<double>& a, int which, int nbands, cudaStream_t st, bool dry);
+
+// Whether all three passes of `a` have a fixed-point instance (the slab between them is in that form, so
+// it is all or none): the x edge, and one split of N2 == N3 at least.
+bool fx_available(const lk::LocalArgs<double>& a);
+template <typename T>
+bool fx_available_t(const lk::LocalArgs<T>& a) {
+  if constexpr (sizeof(T) == 8) return fx_available(a);
+  else return false;
+}
 
 // Tables of the fixed-point passes that belong to the system (not V and the exponents, which go with a
 // schedule and a slab).  Every LocalArgs<double> carries them: whoever asks the tuner for a schedule

@@ -1,7 +1,9 @@
-// Kernel instances of the CTA-wide passes (local_kernels.cuh) in single precision: pass B
-// (pass_bw_body) for every split of KSS_WIDE_SPLITS, run at 128, 256 or 384 threads per CTA, passes A
-// and C (pass_aw_body, pass_cw_body) for the x splits of KSS_WIDEX_SPLITS.  (Double precision:
-// local_fx_impl.cuh.)
+// Kernel instances of the CTA-wide passes (local_kernels.cuh) for one precision: pass B
+// (pass_bw_body) for every split of KSS_WIDE_SPLITS, run at 256 or 384 threads per CTA (and 128 in
+// single precision), passes A and C (pass_aw_body, pass_cw_body) for the x splits of
+// KSS_WIDEX_SPLITS.  Included by one translation unit per precision (local_wide_f32.cu,
+// local_wide_f64.cu).  Double precision takes them where the fixed-point passes (local_fx_impl.cuh)
+// have no instance: an x edge outside KSS_FX_X, or N2 != N3 with a CTA-wide x edge.
 #pragma once
 
 #include "local_kernels.cuh"
@@ -38,7 +40,7 @@ bool launch_one(const LocalArgs<T>& a, int nt, int nbands, cudaStream_t st, bool
 // and four-warp barriers idle fewer warps.
 template <typename T>
 bool dispatch(const LocalArgs<T>& a, int A, int B, int nt, int nbands, cudaStream_t st, bool dry) {
-  if (a.N2 != a.N3 || A * B != a.N2 || (nt != 128 && nt != 256 && nt != 384)) return false;
+  if (a.N2 != a.N3 || A * B != a.N2 || (nt != 256 && nt != 384 && (nt != 128 || sizeof(T) == 8))) return false;
   switch (A * 32 + B) {
 #define KSS_CASE(x, y) \
   case x * 32 + y:     \

@@ -1,7 +1,7 @@
 // Autotuner of the FFT radix schedule of pass B (the y/z transforms of the local-potential path,
 // §5.1 batched FFTs).  For a box length N = N2 = N3 the candidates are the CTA-wide form with
 // every compile-time split N = A * B at 256 and 384 threads per CTA (and 128 in single precision),
-// and the per-warp form.  Each
+// in fixed point where the box runs so in double precision, and the per-warp form.  Each
 // candidate runs one warm-up and three timed launches (the fastest counts) on a zero-filled
 // scratch slab of the same window and of the production chunk size (CUDA events on the context's
 // stream); the fastest candidate is kept for the process in a table keyed by device, precision,
@@ -18,23 +18,38 @@ namespace kss {
 
 namespace {
 
-using Key = std::tuple<int, int, int, int, int, int, int>;  // device, bytes/real, N1, N2, N3, W3 (rounded), 0
+using Key = std::tuple<int, int, int, int, int, int>;  // device, bytes/real, N1, N2, N3, W3 (rounded)
 
 struct Entry {
   PassBSched s;
   int device, prec, N1, N, W3, W2;
 };
 
+// What is kept for a configuration: a schedule of the floating-point passes and one of the
+// fixed-point passes (double precision).  The table has one entry for both, the fixed-point one where
+// that is there, and a pinned schedule is pinned for both.
+struct Slot {
+  Entry e[2];
+  bool has[2] = {false, false};
+};
+
 std::mutex g_mu;
-std::map<Key, Entry> g_table;
+std::map<Key, Slot> g_table;
 std::vector<Key> g_order;  // insertion order (for listing)
 
+// The CTA-wide pass B of schedule c, in fixed point (fx) or in the data's precision (dry: whether there is one).
 template <typename T>
-PassBSched builtin(const lk::LocalArgs<T>& a, const fftr::Split& s2) {
-  PassBSched s;
-  s.A = s2.A;
-  s.B = s2.B;
-  s.threads = wide_pass_b<T>(a, s2.A, s2.B, lk::kWideThreads, 0, nullptr, true) ? lk::kWideThreads : 0;
+bool wide(const lk::LocalArgs<T>& a, const PassBSched& c, bool fx, int nbands, cudaStream_t st, bool dry) {
+  if constexpr (sizeof(T) == 8) {
+    if (fx) return fx_pass_b(a, c.A, c.B, c.threads, nbands, st, dry);
+  }
+  return wide_pass_b<T>(a, c.A, c.B, c.threads, nbands, st, dry);
+}
+
+template <typename T>
+PassBSched builtin(const lk::LocalArgs<T>& a, const fftr::Split& s2, bool fx) {
+  PassBSched s{s2.A, s2.B, lk::kWideThreads, 0, 0};
+  if (!wide(a, s, fx, 0, nullptr, true)) s.threads = 0;
   return s;
 }
 
@@ -45,19 +60,19 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   // Configurations are keyed by box and the window height W3 rounded up to a multiple of 8 (the
   // y-stage task count); a schedule tuned at the rounded height fits every smaller one.
   const int W3b = std::min(a.N3, (a.W3 + 7) / 8 * 8);
-  const Key key{ctx->device, (int)sizeof(T), a.N1, a.N2, a.N3, W3b, 0};
+  const Key key{ctx->device, (int)sizeof(T), a.N1, a.N2, a.N3, W3b};
+  const bool fx = fx_available_t(a);
   {
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_table.find(key);
-    if (it != g_table.end()) return it->second.s;
+    if (it != g_table.end() && it->second.has[fx]) return it->second.e[fx].s;
   }
-  if (!may_tune || !ctx->autotune) return builtin<T>(a, s2);
+  if (!may_tune || !ctx->autotune) return builtin<T>(a, s2, fx);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   KSS_CHECK_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
-  if (cs != cudaStreamCaptureStatusNone) return builtin<T>(a, s2);
+  if (cs != cudaStreamCaptureStatusNone) return builtin<T>(a, s2, fx);
 
-  // (in double precision the candidates are the fixed-point passes)
-  KSS_REQUIRE(sizeof(T) == 4 || (a.fx.r2 && a.fx.vhigh), "pass-B tuner: arguments without the fixed-point tables");
+  KSS_REQUIRE(!fx || (a.fx.r2 && a.fx.vhigh), "pass-B tuner: arguments without the fixed-point tables");
 
   using C = typename lk::CT<T>::C;
   lk::LocalArgs<T> t = a;
@@ -66,9 +81,10 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   std::vector<PassBSched> cand;
   if (a.N2 == a.N3)
     for (const auto& ab : wide_splits())
-      for (int nt : {128, 256, 384})  // 128: single precision only (the dry check says which exist)
-        if (ab.first * ab.second == a.N2 && wide_pass_b<T>(t, ab.first, ab.second, nt, 0, nullptr, true))
-          cand.push_back(PassBSched{ab.first, ab.second, nt, 0, 0});
+      for (int nt : {128, 256, 384}) {  // 128: single precision only (the dry check says which exist)
+        const PassBSched c{ab.first, ab.second, nt, 0, 0};
+        if (c.A * c.B == a.N2 && wide(t, c, fx, 0, nullptr, true)) cand.push_back(c);
+      }
   cand.push_back(PassBSched{s2.A, s2.B, 0, 0, 0});
   // scratch slab of the production chunk size (the local passes keep kSlabChunkBytes of slab per
   // launch), so that candidates are timed at the launch shape they will run at
@@ -88,7 +104,7 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   KSS_CHECK_CUDA(cudaEventCreate(&e0));
   KSS_CHECK_CUDA(cudaEventCreate(&e1));
   auto launch = [&](const PassBSched& c) {
-    if (c.threads) wide_pass_b<T>(t, c.A, c.B, c.threads, nbt, ctx->stream, false);
+    if (c.threads) wide(t, c, fx, nbt, ctx->stream, false);
     else warp_pass_b<T>(ctx, t, nbt);
   };
   int best = -1;
@@ -113,11 +129,13 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   PassBSched s = cand[best];
   s.ncand = (int)cand.size();
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_table.count(key)) {
-    g_table[key] = Entry{s, ctx->device, sizeof(T) == 8 ? KSS_PREC_FP64 : KSS_PREC_MIXED, a.N1, a.N2, W3b, a.W2};
-    g_order.push_back(key);
+  if (!g_table.count(key)) g_order.push_back(key);
+  Slot& slot = g_table[key];
+  if (!slot.has[fx]) {
+    slot.e[fx] = Entry{s, ctx->device, sizeof(T) == 8 ? KSS_PREC_FP64 : KSS_PREC_MIXED, a.N1, a.N2, W3b, a.W2};
+    slot.has[fx] = true;
   }
-  return g_table[key].s;
+  return slot.e[fx].s;
 }
 
 template PassBSched pass_b_schedule<double>(kss_ctx, const lk::LocalArgs<double>&, const fftr::Split&, bool);
@@ -146,7 +164,8 @@ kss_status kss_autotune_get(int i, kss_tune_entry* out) {
   if (!out) return KSS_EINVAL;
   std::lock_guard<std::mutex> lock(g_mu);
   if (i < 0 || i >= (int)g_order.size()) return KSS_EINVAL;
-  const Entry& e = g_table.at(g_order[i]);
+  const Slot& slot = g_table.at(g_order[i]);
+  const Entry& e = slot.e[slot.has[1]];
   out->device = e.device;
   out->precision = e.prec;
   out->N1 = e.N1;
@@ -168,14 +187,16 @@ kss_status kss_autotune_put(const kss_tune_entry* e) {
     return KSS_EINVAL;
   const int bytes = e->precision == KSS_PREC_FP64 ? 8 : 4;
   const int W3b = std::min(e->N, (e->W3 + 7) / 8 * 8);
-  const Key key{e->device, bytes, e->N1, e->N, e->N, W3b, 0};
+  const Key key{e->device, bytes, e->N1, e->N, e->N, W3b};
   PassBSched s;
   s.A = e->A;
   s.B = e->B;
   s.threads = e->threads;
   std::lock_guard<std::mutex> lock(g_mu);
   if (!g_table.count(key)) g_order.push_back(key);
-  g_table[key] = Entry{s, e->device, e->precision, e->N1, e->N, W3b, e->W2};
+  Slot& slot = g_table[key];
+  slot.e[0] = slot.e[1] = Entry{s, e->device, e->precision, e->N1, e->N, W3b, e->W2};
+  slot.has[0] = slot.has[1] = true;
   return KSS_OK;
 }
 
