@@ -20,7 +20,6 @@
 #include "batch_kernels.cuh"
 #include "local_fused.h"
 #include "local_kernels.cuh"
-#include "local_wide.h"
 #include "tune.h"
 
 namespace kss {
@@ -94,7 +93,6 @@ void fill_args(kss_sys s, int ik, LocalArgs<T>& a) {
   a.Vx = (const T*)(f64 ? s->d_Vx64.p : s->d_Vx32.p);
   a.ld = kd.npw;
   a.n0 = 0;
-  if (f64) fx_args(s, a.fx);
 }
 
 size_t al256(size_t n) { return (n + 255) & ~(size_t)255; }
@@ -298,7 +296,7 @@ void BatchEngine::prepare_t() {
     fill_args<T>(units[u]->sys, units[u]->ik, au);
     RegPlan rp;
     std::memcpy(&rp, &p, sizeof(RegPlan));
-    bs[u] = pass_b_schedule<T>(ctx, au, rp.s2, true);
+    bs[u] = pass_b_schedule<T>(ctx, au, rp.s2, true, false);
     pruned[u] = bs[u].threads && pruned_w<T>(au, bs[u].A, bs[u].B);
     if (bs[u].threads && (!group_kernel_w<T>(bs[u].A, bs[u].B, bs[u].threads, pruned[u]) ||
                           wide_b_smem(au.N2, au.W3, es) > 227 * 1024 || au.N2 != au.N3))

@@ -430,6 +430,13 @@ int chunk_bands(kss_sys s, int ik, int nb, size_t es) {
   return (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, target / per));
 }
 
+void fx_args(kss_sys s, FxTables& f) {
+  f.r1 = s->d_rot[0].as<fx::Rot>();
+  f.r2 = s->d_rot[1].as<fx::Rot>();
+  f.vhigh = s->d_vhigh.as<int>();
+  f.invn = 1.0 / ((double)s->N[0] * s->N[1] * s->N[2]);
+}
+
 // The CTA-wide form of pass B and of passes A (which = 0) and C (1), in fixed point (fx) or in the
 // data's own precision.  False, and nothing launched, when the schedule or the box has none.
 template <typename T>
@@ -565,9 +572,10 @@ void run_local(kss_sys s, int ik, int nb, const void* psi, const void* psi_prev,
       auto warp_b = [&](const LocalArgs<T>& t, int m) {
         launch_pdl(kk.b, dim3(t.N1, m), kThreads, rb, ctx->stream, t, rp, scr_warp);
       };
-      PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, true);
       // all three passes in fixed point or none
-      const bool fx = fx_available_t(a) && wide_b(a, sb, true, 0, nullptr, true);
+      const bool fxa = fx_available_t(a);
+      const PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, true, fxa);
+      const bool fx = fxa && wide_b(a, sb, true, 0, nullptr, true);
       if (fx) a.fx.V = (const fx::Limbs*)vfx_view(s, sb.A, sb.B);
       else if (wide_b(a, sb, false, 0, nullptr, true)) a.Vpi = (const T*)vpi_view(s, sb.A, sb.B, f64);
       static const int ida = prof_register(f64 ? "local_pass_a<f64>" : "local_pass_a<f32>");
@@ -693,11 +701,12 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
       auto warp_b = [&](const LocalArgs<T>& t, int m) {
         launch_pdl(kk.b, dim3(t.N1, m), kThreads, rb, ctx->stream, t, rp, scr_warp);
       };
-      PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, false);  // no tuning here
+      const bool fxa = fx_available_t(a);
+      PassBSched sb = pass_b_schedule<T>(ctx, a, rp.s2, false, fxa);  // no tuning here
       // The CTA-wide forms need V in their split's layout; that view is built (allocated) by the first
       // ordinary application, and without it this path takes the per-warp form.
       bool fx = false;
-      if (meta && fx_available_t(a) && wide_b(a, sb, true, 0, nullptr, true)) {
+      if (meta && fxa && wide_b(a, sb, true, 0, nullptr, true)) {
         auto it = s->vfx.find(sb.A * 32 + sb.B);
         fx = it != s->vfx.end();
         if (fx) a.fx.V = it->second.template as<fx::Limbs>();
@@ -738,13 +747,6 @@ void run_local_ws(kss_sys s, int ik, int nb, const void* psi, void* out, int ld,
 }
 
 }  // namespace
-
-void fx_args(kss_sys s, FxTables& f) {
-  f.r1 = s->d_rot[0].as<fx::Rot>();
-  f.r2 = s->d_rot[1].as<fx::Rot>();
-  f.vhigh = s->d_vhigh.as<int>();
-  f.invn = 1.0 / ((double)s->N[0] * s->N[1] * s->N[2]);
-}
 
 template <typename T>
 void warp_pass_b(kss_ctx ctx, const LocalArgs<T>& a, int nbands) {

@@ -35,11 +35,6 @@ bool fx_available_t(const lk::LocalArgs<T>& a) {
   else return false;
 }
 
-// Tables of the fixed-point passes that belong to the system (not V and the exponents, which go with a
-// schedule and a slab).  Every LocalArgs<double> carries them: whoever asks the tuner for a schedule
-// has it time the fixed-point pass.
-void fx_args(kss_sys s, lk::FxTables& f);
-
 // The (A, B) pairs with instances, in KSS_WIDE_SPLITS order.
 inline const std::vector<std::pair<int, int>>& wide_splits() {
   static const std::vector<std::pair<int, int>> v = {

@@ -1,7 +1,7 @@
 // Autotuner of the FFT radix schedule of pass B (the y/z transforms of the local-potential path,
 // §5.1 batched FFTs).  For a box length N = N2 = N3 the candidates are the CTA-wide form with
 // every compile-time split N = A * B at 256 and 384 threads per CTA (and 128 in single precision),
-// in fixed point where the box runs so in double precision, and the per-warp form.  Each
+// in fixed point where the caller runs it so (double precision), and the per-warp form.  Each
 // candidate runs one warm-up and three timed launches (the fastest counts) on a zero-filled
 // scratch slab of the same window and of the production chunk size (CUDA events on the context's
 // stream); the fastest candidate is kept for the process in a table keyed by device, precision,
@@ -56,12 +56,11 @@ PassBSched builtin(const lk::LocalArgs<T>& a, const fftr::Split& s2, bool fx) {
 }  // namespace
 
 template <typename T>
-PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::Split& s2, bool may_tune) {
+PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::Split& s2, bool may_tune, bool fx) {
   // Configurations are keyed by box and the window height W3 rounded up to a multiple of 8 (the
   // y-stage task count); a schedule tuned at the rounded height fits every smaller one.
   const int W3b = std::min(a.N3, (a.W3 + 7) / 8 * 8);
   const Key key{ctx->device, (int)sizeof(T), a.N1, a.N2, a.N3, W3b};
-  const bool fx = fx_available_t(a);
   {
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_table.find(key);
@@ -138,8 +137,8 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   return slot.e[fx].s;
 }
 
-template PassBSched pass_b_schedule<double>(kss_ctx, const lk::LocalArgs<double>&, const fftr::Split&, bool);
-template PassBSched pass_b_schedule<float>(kss_ctx, const lk::LocalArgs<float>&, const fftr::Split&, bool);
+template PassBSched pass_b_schedule<double>(kss_ctx, const lk::LocalArgs<double>&, const fftr::Split&, bool, bool);
+template PassBSched pass_b_schedule<float>(kss_ctx, const lk::LocalArgs<float>&, const fftr::Split&, bool, bool);
 
 }  // namespace kss
 

@@ -19,8 +19,11 @@ struct PassBSched {
 // CTA-wide form with the cost-model split at 384 threads when it exists, else the per-warp form).
 // Candidates are timed at the window height rounded up to a multiple of 8, each launch sizing its
 // shared memory from the arguments it is given (the per-warp form through warp_pass_b).
+// fx: the CTA-wide candidates are the fixed-point kernels, else those in the data's precision; the caller
+// asks for the ones that it launches (a single application of a box with fixed-point instances, against
+// the batch engine, whose grouped passes are in FP64).
 template <typename T>
-PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::Split& s2, bool may_tune);
+PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::Split& s2, bool may_tune, bool fx);
 
 // The per-warp pass B (compile-time split when available) for args a over nbands bands on the
 // context stream; used by the tuner as that form's timing (local_apply.cu).
