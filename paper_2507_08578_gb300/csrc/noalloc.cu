@@ -14,7 +14,10 @@ namespace {
 
 // The scratch array.  In host code `g_noalloc_scratch` is only a host-side stand-in for the
 // symbol, never a device address: host code must use the address from cudaGetSymbolAddress.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[KSS_NOALLOC_SCRATCH_BYTES];
+// Behind it, room for the plane exponents of one band in the fixed-point passes (boxes of up to 96 points
+// an edge have instances: 1.5 KB).
+constexpr size_t kMetaBytes = 4096;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[KSS_NOALLOC_SCRATCH_BYTES + kMetaBytes];
 
 // The address is looked up once per context, on that context's first call, with its device
 // current, and kept in the context.  A context made after the CUDA context of its device was torn
@@ -78,12 +81,15 @@ extern "C" kss_status kss_apply_H_noalloc(kss_sys sys, int ik, int nb, const voi
       part = std::max(cprj, (free_after / 2) / cprj * cprj);
     }
     const size_t slab_off = cprj + align256(part);
-    int nc = (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, (cap - slab_off) / plane));
-    // the plane exponents of the double-precision passes sit behind the slab; a request whose only
-    // slab leaves no room for them runs the form without
-    auto meta_end = [&](int c) { return slab_off + align256(plane * c) + local_meta_bytes(sys, ik, c); };
-    if (f64 && nc > 1 && meta_end(nc) > cap) --nc;
-    void* meta = f64 && meta_end(nc) <= cap ? base + slab_off + align256(plane * nc) : nullptr;
+    // Double precision: the plane exponents of the fixed-point passes sit behind the slab of nc bands.  Where
+    // the scratch holds the slab of one band and not its exponents, these go behind the scratch.
+    const size_t meta1 = f64 ? local_meta_bytes(sys, ik, 1) : 0;
+    const size_t room = cap - slab_off, pad = f64 ? 256 : 0;
+    size_t fit = room > pad ? (room - pad) / (plane + meta1) : 0;
+    unsigned char* meta = nullptr;
+    if (f64 && fit) meta = base + slab_off + align256(plane * std::min<size_t>(nb, fit));
+    else if (f64 && meta1 <= kMetaBytes) meta = base + cap;
+    const int nc = (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, fit));
     if (sys->nproj) {
       void* C = base;
       const bool ok = gemm_cn_ws(ctx, f64, sys->nproj, nb, kd.npw, f64 ? kd.d_beta64.p : kd.d_beta32.p,

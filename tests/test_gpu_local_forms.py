@@ -74,3 +74,32 @@ def test_uneven_boxes_match_oracle(ctx, box):
     finally:
         K.kss_sys_destroy(sysh)
         K.kss_autotune_clear()
+
+
+@pytest.mark.parametrize("box,a,ecut,natom,nb,nproj", [
+    ((24, 24, 24), 10.0, 10.0, 4, 12, 0),      # every band in one chunk
+    ((24, 24, 24), 10.0, 10.0, 4, 1700, 0),    # more bands than the scratch holds: several chunks
+    ((36, 36, 36), 9.0, 8.0, 60, 8729, 4),     # room for one slab and not for its exponents
+    ((64, 48, 48), 10.0, 10.0, 4, 12, 0)])     # CTA-wide passes in FP64
+def test_noalloc_runs_the_same_passes(ctx, box, a, ecut, natom, nb, nproj):
+    """The entry point that allocates nothing takes the passes of kss_apply_H however much of its
+    scratch the band block leaves, so the local part agrees bit for bit (projector energies of zero
+    where there are projectors: their products are summed in another order)."""
+    import torch
+    s = W.make_system("fn", a, ecut, natom, 4, seed=25, fft_box=box, nproj_per_atom=nproj)
+    s.D = np.zeros_like(s.D)
+    sysh = setup(ctx, s)
+    try:
+        K.kss_autotune_clear()
+        K.kss_autotune_set(ctx, 1)
+        npw = K.kss_sphere(sysh, 0).shape[0]
+        g = torch.Generator(device="cuda").manual_seed(4)
+        psi = torch.randn(nb, npw, dtype=torch.complex128, device="cuda", generator=g)
+        ref, out = torch.empty_like(psi), torch.empty_like(psi)
+        K.kss_apply_H(sysh, 0, psi, ref, K.KSS_PREC_FP64)
+        K.kss_apply_H_noalloc(sysh, 0, psi, out, K.KSS_PREC_FP64)
+        torch.cuda.synchronize()
+        assert torch.equal(ref, out)
+    finally:
+        K.kss_sys_destroy(sysh)
+        K.kss_autotune_clear()
