@@ -113,6 +113,17 @@ __host__ __device__ constexpr int v_exp(int high) {
   return (f > 1 ? f : 1) - 1022;
 }
 
+// Component i of a slab of size kSlabBits, to time the passes on: the indices hashed, spread evenly over two
+// bits less, as in a band most components lie below the largest.  So no stage of the y transform finds its
+// input outside its range and stops to shift it (fit).
+constexpr int kSlabBits = 59;
+__host__ __device__ constexpr long long slab_value(unsigned long long i) {
+  unsigned long long h = i * 0x9E3779B97F4A7C15ull + 1;
+  h ^= h >> 29;
+  h *= 0xBF58476D1CE4E5B9ull;
+  return (long long)h >> (65 - kSlabBits);
+}
+
 #ifdef __CUDACC__
 __device__ __forceinline__ int lo32(long long a) { return (int)a; }
 // high limb that goes with the signed low limb

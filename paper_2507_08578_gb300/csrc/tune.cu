@@ -2,9 +2,10 @@
 // §5.1 batched FFTs).  For a box length N = N2 = N3 the candidates are the CTA-wide form with
 // every compile-time split N = A * B at 256 and 384 threads per CTA (and 128 in single precision),
 // in fixed point where the caller runs it so (double precision), and the per-warp form.  Each
-// candidate runs one warm-up and three timed launches (the fastest counts) on a zero-filled
-// scratch slab of the same window and of the production chunk size (CUDA events on the context's
-// stream); the fastest candidate is kept for the process in a table keyed by device, precision,
+// candidate runs one warm-up and three timed launches (the fastest counts) on a scratch slab of
+// the same window and of the production chunk size (CUDA events on the context's stream): zeros in
+// floating point, whose time does not depend on the values, and values of the size that pass A leaves
+// in fixed point; the fastest candidate is kept for the process in a table keyed by device, precision,
 // box and window.  All candidates compute the same transform; they differ only in rounding order.
 #include <map>
 #include <mutex>
@@ -44,6 +45,20 @@ bool wide(const lk::LocalArgs<T>& a, const PassBSched& c, bool fx, int nbands, c
     if (fx) return fx_pass_b(a, c.A, c.B, c.threads, nbands, st, dry);
   }
   return wide_pass_b<T>(a, c.A, c.B, c.threads, nbands, st, dry);
+}
+
+// A fixed-point slab like those of pass A, with the plane entries to match, and V as the pass reads it (its
+// layout aside).  On zeros the pass would shift a plane before six of its eight stages (measured on a
+// slab of zeros: 2 to 5 % above the same launch on bands, more for some splits than for others).
+__global__ void fill_fx(long long* work, long long n, int2* ma, long long nm, fx::Limbs* V, long long nv,
+                        const double* __restrict__ Vx, double points, const int* __restrict__ vhigh) {
+  const int E = fx::v_exp(*vhigh) - 63;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n || i < nv;
+       i += (long long)gridDim.x * blockDim.x) {
+    if (i < n) work[i] = fx::slab_value((unsigned long long)i);
+    if (i < nm) ma[i] = make_int2(0, fx::kSlabBits);
+    if (i < nv) V[i] = fx::limbs(fx::from_double(Vx[i] * points, E));
+  }
 }
 
 template <typename T>
@@ -90,14 +105,28 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   const size_t per_band = (size_t)t.N1 * t.W3 * t.W2 * sizeof(C);
   const int nbt = (int)std::max<size_t>(1, std::min<size_t>(64, kSlabChunkBytes / per_band));
   const size_t elems = (size_t)t.N1 * t.W3 * t.W2 * nbt;
-  const size_t bytes = elems * sizeof(C) + sizeof(int2) * (size_t)nbt * (t.N1 + t.W3);
+  const size_t nmeta = (size_t)nbt * (t.N1 + t.W3), nv = fx ? (size_t)t.N1 * t.N2 * t.N3 : 0;
+  const size_t bytes = elems * sizeof(C) + (fx ? sizeof(int2) * nmeta + sizeof(fx::Limbs) * nv : 0);
   ctx->ws_tune.ensure(bytes);
-  KSS_CHECK_CUDA(cudaMemsetAsync(ctx->ws_tune.p, 0, bytes, ctx->stream));
   t.work = ctx->ws_tune.as<C>();
-  t.fx.ma = reinterpret_cast<int2*>(t.work + elems);
-  t.fx.mb = t.fx.ma + (size_t)nbt * t.W3;
+  // (a launch overwrites the slab, whose plane entries then no longer hold: filled anew for each)
+  auto refill = [&](const PassBSched& c) {
+    if constexpr (sizeof(T) == 8) {
+      if (fx && c.threads) {
+        t.fx.ma = reinterpret_cast<int2*>(t.work + elems);
+        t.fx.mb = t.fx.ma + (size_t)nbt * t.W3;
+        fx::Limbs* V = reinterpret_cast<fx::Limbs*>(t.fx.ma + nmeta);
+        t.fx.V = V;
+        fill_fx<<<152 * 8, 256, 0, ctx->stream>>>(reinterpret_cast<long long*>(t.work), 2 * (long long)elems, t.fx.ma,
+                                                  (long long)nmeta, V, (long long)nv, t.Vx,
+                                                  (double)t.N1 * t.N2 * t.N3, t.fx.vhigh);
+        KSS_CHECK_CUDA(cudaGetLastError());
+        return;
+      }
+    }
+    KSS_CHECK_CUDA(cudaMemsetAsync(ctx->ws_tune.p, 0, elems * sizeof(C), ctx->stream));
+  };
   t.Vpi = t.Vx;  // any N1 x N x N array: the values do not matter for timing
-  t.fx.V = reinterpret_cast<const fx::Limbs*>(t.Vx);
   t.n0 = 0;
   cudaEvent_t e0, e1;
   KSS_CHECK_CUDA(cudaEventCreate(&e0));
@@ -108,9 +137,11 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   };
   int best = -1;
   for (size_t i = 0; i < cand.size(); ++i) {
+    refill(cand[i]);
     launch(cand[i]);  // warm-up (and shared-memory attribute)
     double tmin = 1e300;
     for (int r = 0; r < 3; ++r) {  // the fastest of three timed launches
+      if (fx) refill(cand[i]);
       KSS_CHECK_CUDA(cudaEventRecord(e0, ctx->stream));
       launch(cand[i]);
       KSS_CHECK_CUDA(cudaEventRecord(e1, ctx->stream));
