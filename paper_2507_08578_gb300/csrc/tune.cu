@@ -73,7 +73,9 @@ PassBSched builtin(const lk::LocalArgs<T>& a, const fftr::Split& s2, bool fx) {
 template <typename T>
 PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::Split& s2, bool may_tune, bool fx) {
   // Configurations are keyed by box and the window height W3 rounded up to a multiple of 8 (the
-  // y-stage task count); a schedule tuned at the rounded height fits every smaller one.
+  // y-stage task count).  A candidate has to fit at the rounded height, so that the choice fits every
+  // smaller one; it is timed on the caller's own window, which decides between the pruned and the full
+  // instance of a split.
   const int W3b = std::min(a.N3, (a.W3 + 7) / 8 * 8);
   const Key key{ctx->device, (int)sizeof(T), a.N1, a.N2, a.N3, W3b};
   {
@@ -89,15 +91,15 @@ PassBSched pass_b_schedule(kss_ctx ctx, const lk::LocalArgs<T>& a, const fftr::S
   KSS_REQUIRE(!fx || (a.fx.r2 && a.fx.vhigh), "pass-B tuner: arguments without the fixed-point tables");
 
   using C = typename lk::CT<T>::C;
-  lk::LocalArgs<T> t = a;
-  t.W3 = W3b;
+  lk::LocalArgs<T> t = a, tall = a;
+  tall.W3 = W3b;
   // candidates: CTA-wide splits x threads, then the per-warp form
   std::vector<PassBSched> cand;
   if (a.N2 == a.N3)
     for (const auto& ab : wide_splits())
       for (int nt : {128, 256, 384}) {  // 128: single precision only (the dry check says which exist)
         const PassBSched c{ab.first, ab.second, nt, 0, 0};
-        if (c.A * c.B == a.N2 && wide(t, c, fx, 0, nullptr, true)) cand.push_back(c);
+        if (c.A * c.B == a.N2 && wide(tall, c, fx, 0, nullptr, true)) cand.push_back(c);
       }
   cand.push_back(PassBSched{s2.A, s2.B, 0, 0, 0});
   // scratch slab of the production chunk size (the local passes keep kSlabChunkBytes of slab per

@@ -17,8 +17,8 @@ struct PassBSched {
 // From the process-wide table if present; else, when tuning is allowed (ctx->autotune, not inside
 // a stream capture), by timing every candidate on a scratch slab; else the built-in choice (the
 // CTA-wide form with the cost-model split at 384 threads when it exists, else the per-warp form).
-// Candidates are timed at the window height rounded up to a multiple of 8, each launch sizing its
-// shared memory from the arguments it is given (the per-warp form through warp_pass_b).
+// Candidates fit the window height rounded up to a multiple of 8 and are timed at the height of `a`, each
+// launch sizing its shared memory from the arguments it is given (the per-warp form through warp_pass_b).
 // fx: the CTA-wide candidates are the fixed-point kernels, else those in the data's precision; the caller
 // asks for the ones that it launches (a single application of a box with fixed-point instances, against
 // the batch engine, whose grouped passes are in FP64).
