@@ -590,8 +590,9 @@ kss_status kss_autotune_clear(void);
  * SMs in one, two or three waves) on the device and keeps the fastest for the process; every
  * schedule computes the same product (the K ranges are added in a fixed order).  kind: 0
  * split-BF16 complex64 products, 1 FP64 digit products, 2 the same with a complex64 result, 3
- * 4-digit products of complex64 data.  Mr: real rows of the product (twice the complex rows), Nr:
- * columns, kblocks: K in k-blocks of the kernel. */
+ * 4-digit products of complex64 data (small FP64 products, on the CUDA cores, have no entry).  Mr:
+ * real rows of the product (twice the complex rows), Nr: columns, kblocks: K in k-blocks of the
+ * kernel. */
 typedef struct {
   int device, kind, Mr, Nr, kblocks;
   int splits;  /* chosen K-split (CTAs along K) */

@@ -567,7 +567,20 @@ void launch_oz(kss_ctx ctx, const OzOperand& a, const OzOperand& b, int M, int N
   }
   // closed-form plan; the autotuner times it against other splits at first use of the shape
   int plan = 1;
-  if (tiles < nsm) plan = (int)std::max(1LL, std::min<long long>(nsm / tiles, kb_total / (2 * CHUNK)));
+  if (herm) {
+    // the split with the shortest waves x (chunks of a CTA + its fill and drain, most of a chunk's time)
+    const int chunks = (kb_total + CHUNK - 1) / CHUNK;
+    double tb = 1e300;
+    for (int sp = 1; sp <= std::min(32, std::max(1, chunks / 2)); ++sp) {
+      const double t = (double)((tiles * sp + nsm - 1) / nsm) * ((chunks + sp - 1) / sp + 0.7);
+      if (t < tb) {
+        tb = t;
+        plan = sp;
+      }
+    }
+  } else if (tiles < nsm) {
+    plan = (int)std::max(1LL, std::min<long long>(nsm / tiles, kb_total / (2 * CHUNK)));
+  }
   const CUtensorMap ma = make_map(a.planes, (long long)SA * a.rows, a.KT, TM);
   const CUtensorMap mb = make_map(b.planes, (long long)SB * b.rows, b.KT, TN, b.pitch);
   auto kern = oz_gemm_kernel<SA, SB, CT>;
@@ -595,26 +608,11 @@ void launch_oz(kss_ctx ctx, const OzOperand& a, const OzOperand& b, int M, int N
                Nr, M, N, herm ? 1 : 0, Cd, ldd, ar, ai, br_, bi_);
     KSS_CHECK_CUDA(cudaGetLastError());
   };
-  if (herm) {
-    // the split with the shortest waves x (chunks of a CTA + its fill and drain, most of a chunk's time)
-    const int chunks = (kb_total + CHUNK - 1) / CHUNK;
-    int best = 1;
-    double tb = 1e300;
-    for (int sp = 1; sp <= std::min(32, std::max(1, chunks / 2)); ++sp) {
-      const double t = (double)((tiles * sp + nsm - 1) / nsm) * ((chunks + sp - 1) / sp + 0.7);
-      if (t < tb) {
-        tb = t;
-        best = sp;
-      }
-    }
-    launch(best, C, ldc, br, bi, true);
-    return;
-  }
   const int kind = SA == 4 ? GT_OZ44 : (sizeof(CT) == sizeof(double2) ? GT_OZ77 : GT_OZ77_C64OUT);
   const int splits = tuned_split(ctx, kind, Mr, Nr, kb_total, tiles, 2 * CHUNK, plan, [&](int sp) {
     ctx->tune_c.ensure((size_t)M * N * sizeof(CT));
     launch(sp, ctx->tune_c.as<CT>(), M, 0.0, 0.0, false);
-  });
+  }, herm);
   launch(splits, C, ldc, br, bi, true);
 }
 

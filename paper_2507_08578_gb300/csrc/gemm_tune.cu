@@ -28,19 +28,28 @@ struct Entry {
   int form;
 };
 
+// The schedules kept for a shape: of products that form all output tiles, and of those with a Hermitian
+// result, which form half of them and fill the SMs with other splits.  The table has one entry for both
+// (the first where that is there), and a pinned schedule is pinned for both.
+struct Slot {
+  Entry e[2];
+  bool has[2] = {false, false};
+};
+
 std::mutex g_mu;
-std::map<Key, Entry> g_table;
+std::map<Key, Slot> g_table;
 std::vector<Key> g_order;
 
 }  // namespace
 
 GemmChoice tuned_gemm(kss_ctx ctx, int kind, int Mr, int Nr, int kb_total, std::vector<GemmChoice> cand,
-                      GemmChoice plan, const std::function<void(GemmChoice)>& run) {
+                      GemmChoice plan, const std::function<void(GemmChoice)>& run, bool herm) {
   const Key key{ctx->device, kind, Mr, Nr, kb_total};
   {
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_table.find(key);
-    if (it != g_table.end()) return GemmChoice{it->second.form, it->second.splits};
+    if (it != g_table.end() && it->second.has[herm])
+      return GemmChoice{it->second.e[herm].form, it->second.e[herm].splits};
   }
   if (!ctx->autotune) return plan;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -75,16 +84,18 @@ GemmChoice tuned_gemm(kss_ctx ctx, int kind, int Mr, int Nr, int kb_total, std::
   KSS_CHECK_CUDA(cudaEventDestroy(e1));
   KSS_CHECK_CUDA(cudaGetLastError());
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_table.count(key)) {
-    g_table[key] = Entry{ctx->device, kind, Mr, Nr, kb_total, best.splits, tbest, (int)cand.size(), best.form};
-    g_order.push_back(key);
+  if (!g_table.count(key)) g_order.push_back(key);
+  Slot& slot = g_table[key];
+  if (!slot.has[herm]) {
+    slot.e[herm] = Entry{ctx->device, kind, Mr, Nr, kb_total, best.splits, tbest, (int)cand.size(), best.form};
+    slot.has[herm] = true;
   }
-  const Entry& e = g_table[key];
+  const Entry& e = slot.e[herm];
   return GemmChoice{e.form, e.splits};
 }
 
 int tuned_split(kss_ctx ctx, int kind, int Mr, int Nr, int kb_total, long long tiles, int min_kb, int plan,
-                const std::function<void(int)>& run) {
+                const std::function<void(int)>& run, bool herm) {
   const int smax = std::max(1, kb_total / std::max(1, min_kb));
   const int nsm = std::max(1, ctx->nsm);
   std::vector<GemmChoice> cand{{0, plan}, {0, 1}};
@@ -92,7 +103,7 @@ int tuned_split(kss_ctx ctx, int kind, int Mr, int Nr, int kb_total, long long t
     cand.push_back({0, (int)std::max(1LL, (long long)w * nsm / std::max(1LL, tiles))});
   for (auto& c : cand) c.splits = std::max(1, std::min(c.splits, smax));
   const GemmChoice g = tuned_gemm(ctx, kind, Mr, Nr, kb_total, cand, GemmChoice{0, std::max(1, std::min(plan, smax))},
-                                  [&](GemmChoice c) { run(c.splits); });
+                                  [&](GemmChoice c) { run(c.splits); }, herm);
   return std::max(1, std::min(g.splits, smax));
 }
 
@@ -119,7 +130,8 @@ kss_status kss_autotune_gemm_get(int i, kss_gemm_tune_entry* out) {
   if (!out) return KSS_EINVAL;
   std::lock_guard<std::mutex> lock(g_mu);
   if (i < 0 || i >= (int)g_order.size()) return KSS_EINVAL;
-  const Entry& e = g_table[g_order[i]];
+  const Slot& slot = g_table[g_order[i]];
+  const Entry& e = slot.e[slot.has[0] ? 0 : 1];
   out->device = e.device;
   out->kind = e.kind;
   out->Mr = e.Mr;
@@ -139,7 +151,9 @@ kss_status kss_autotune_gemm_put(const kss_gemm_tune_entry* e) {
   std::lock_guard<std::mutex> lock(g_mu);
   const Key key{e->device, e->kind, e->Mr, e->Nr, e->kblocks};
   if (!g_table.count(key)) g_order.push_back(key);
-  g_table[key] = Entry{e->device, e->kind, e->Mr, e->Nr, e->kblocks, e->splits, 0.0, 0, e->form};
+  Slot& slot = g_table[key];
+  slot.e[0] = slot.e[1] = Entry{e->device, e->kind, e->Mr, e->Nr, e->kblocks, e->splits, 0.0, 0, e->form};
+  slot.has[0] = slot.has[1] = true;
   return KSS_OK;
 }
 

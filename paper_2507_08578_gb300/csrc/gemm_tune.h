@@ -23,8 +23,9 @@ struct GemmChoice {
 // when tuning is allowed (ctx->autotune, not inside a stream capture), the fastest of `cand`, each
 // timed by `run(choice)` (one warm-up and the fastest of three timed runs, CUDA events on the
 // context stream); else `plan`.  The caller clamps a pinned entry to what its kernels accept.
+// herm: the product forms half of the tiles, its result being Hermitian; timed apart from the others.
 GemmChoice tuned_gemm(kss_ctx ctx, int kind, int Mr, int Nr, int kb_total, std::vector<GemmChoice> cand,
-                      GemmChoice plan, const std::function<void(GemmChoice)>& run);
+                      GemmChoice plan, const std::function<void(GemmChoice)>& run, bool herm = false);
 // K-split for a (kind, Mr real rows, Nr columns, kb_total k-blocks) product: the process-wide table
 // entry if present; else, when tuning is allowed (ctx->autotune, not inside a stream capture), the
 // fastest of the candidates, each timed by `run(splits)` (which launches the product with that
@@ -33,7 +34,7 @@ GemmChoice tuned_gemm(kss_ctx ctx, int kind, int Mr, int Nr, int kb_total, std::
 // split, and the splits that fill the SMs in one, two or three waves, each keeping at least
 // `min_kb` k-blocks per CTA.  Returns a split in [1, kb_total / min_kb] (at least 1).
 int tuned_split(kss_ctx ctx, int kind, int Mr, int Nr, int kb_total, long long tiles, int min_kb, int plan,
-                const std::function<void(int)>& run);
+                const std::function<void(int)>& run, bool herm = false);
 // Empty the K-split table (kss_autotune_clear).
 void gemm_tune_clear();
 

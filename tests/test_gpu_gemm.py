@@ -244,3 +244,54 @@ def test_block_with_itself(ctx, M, Kd, alpha, beta):
     assert np.max(np.abs(got - ref)) < 1e-12 * np.max(np.abs(ref))
     if beta == 0:
         assert np.array_equal(got, got.conj().T)
+
+
+def test_hermitian_products_follow_the_table(ctx):
+    """A block with itself has a tuned entry, and a pinned K-split is the one that runs: the partial sums
+    of another split round differently (1e-12 of the largest entry, the digit form's bar, and not bit for
+    bit), those of the same split do not."""
+    import torch
+    rng = np.random.default_rng(77)
+    M, Kd = 300, 20000
+    A = crand(rng, (M, Kd))
+    ref = A.conj() @ A.T
+    tA = torch.from_numpy(A).cuda()
+
+    def run():
+        tC = torch.zeros((M, M), dtype=torch.complex128, device="cuda")
+        K.kss_gemm(ctx, 0, tA, tA, tC, 1.0, 0.0, K.KSS_PREC_FP64)
+        torch.cuda.synchronize()
+        got = tC.cpu().numpy().T
+        assert np.max(np.abs(got - ref)) < 1e-12 * np.max(np.abs(ref))
+        return got
+
+    K.kss_autotune_clear()
+    try:
+        run()
+        (e,) = [e for e in K.kss_autotune_gemm_table() if e["kind"] == 1]
+        assert (e["Mr"], e["Nr"]) == (2 * M, M) and e["ncand"] >= 2 and e["ms"] > 0
+        out = {}
+        for sp in (1, 7, 20, 7):
+            K.kss_autotune_gemm_put(e["device"], 1, e["Mr"], e["Nr"], e["kblocks"], sp)
+            got = run()
+            assert sp not in out or np.array_equal(out[sp], got)
+            out[sp] = got
+        assert not np.array_equal(out[1], out[7]) and not np.array_equal(out[7], out[20])
+    finally:
+        K.kss_autotune_clear()
+
+
+def test_four_digit_gram_products_have_entries(ctx):
+    """The Gram products of a mixed-form solve (4-digit products of its complex64 block) are tuned."""
+    import workloads as W
+    from tests.kss_helpers import setup
+    s = W.make_system("gg", 8.0, 8.0, 4, 12, seed=51, kpts=[[0.25, 0.25, 0.25]])
+    sysh = setup(ctx, s)
+    K.kss_autotune_clear()
+    try:
+        K.kss_chebfi_solve(sysh, 0, s.nband, K.make_opts(prec=K.KSS_PREC_MIXED, seed=5))
+        gram = [e for e in K.kss_autotune_gemm_table() if e["kind"] == 3]
+        assert gram and all(e["Mr"] == 2 * e["Nr"] for e in gram)
+    finally:
+        K.kss_sys_destroy(sysh)
+        K.kss_autotune_clear()
