@@ -265,6 +265,9 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(acce));
     }
+    // the lanes with a row, both or neither of a complex pair (Mr is even), which the exchange below names:
+    // what is converged there does not depend on the branches between
+    const unsigned rows = __ballot_sync(0xffffffffu, row < Mr);
     if (ok && nkb > 0 && row < Mr) {
       const int er = ea[row], col0 = tn * TN + colh;
       const bool cplx = ai != 0.0 || bi != 0.0;
@@ -290,12 +293,12 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // row 2i is Re C(i, col), row 2i + 1 is Im C(i, col): consecutive words of C
         R* dst = reinterpret_cast<R*>(C + (size_t)col * ldc) + row;
         double o = ar == 1.0 ? v : ar * v;
-        if (cplx) {  // (Mr is even: both rows of a pair are here)
-          const double w = __shfl_xor_sync(__activemask(), v, 1);
+        if (cplx) {
+          const double w = __shfl_xor_sync(rows, v, 1);
           o = (row & 1) ? o + ai * w : o - ai * w;
           if (br != 0.0 || bi != 0.0) {
             const double q = *dst, p = dst[(row & 1) ? -1 : 1];
-            __syncwarp(__activemask());
+            __syncwarp(rows);
             o += (row & 1) ? br * q + bi * p : br * q - bi * p;
           }
         } else if (br != 0.0) {

@@ -295,3 +295,31 @@ def test_four_digit_gram_products_have_entries(ctx):
     finally:
         K.kss_sys_destroy(sysh)
         K.kss_autotune_clear()
+
+
+def test_digit_products_complex_alpha_at_the_exponent_limit(ctx):
+    """Complex alpha and beta where some rows of a warp need their exponent applied apart (below 2^-980
+    after scaling) and their neighbours do not, with a ragged last tile: each row within the digit form's
+    1e-12 of its largest entry."""
+    import torch
+    rng = np.random.default_rng(5)
+    M, N, Kd = 165, 170, 700
+    ex = np.where(np.arange(M) % 3 == 1, -900, -80)
+    A, B = crand(rng, (M, Kd)), crand(rng, (N, Kd))
+    up = np.ldexp(1.0, -ex)  # what brings a row of the result back, less 2^-80 of B
+    tA = torch.from_numpy(A * np.ldexp(1.0, ex)[:, None]).cuda()
+    tB = torch.from_numpy(B * 2.0 ** -80).cuda()
+    C0 = crand(rng, (N, M)) * np.ldexp(1.0, ex)[None, :] * 2.0 ** -80
+    alpha, beta = 0.6 + 0.3j, -0.4 + 0.2j
+    ref = alpha * (A.conj() @ B.T) + beta * ((C0 * 2.0 ** 80).T * up[:, None])
+    K.kss_autotune_clear()
+    try:
+        for sp in (1, 2):  # written by the product itself, and through partial sums
+            K.kss_autotune_gemm_put(0, 1, 2 * M, N, (2 * Kd + 31) // 32, sp)
+            tC = torch.from_numpy(C0).cuda()
+            K.kss_gemm(ctx, 0, tA, tB, tC, alpha, beta, K.KSS_PREC_FP64)
+            torch.cuda.synchronize()
+            got = (tC.cpu().numpy().T * 2.0 ** 80) * up[:, None]
+            assert np.all(np.abs(got - ref) < 1e-12 * np.max(np.abs(ref), axis=1)[:, None])
+    finally:
+        K.kss_autotune_clear()
