@@ -44,6 +44,7 @@
 #include <vector>
 
 #include "kss_internal.h"
+#include "recip64.cuh"
 
 namespace kss {
 
@@ -54,35 +55,6 @@ constexpr int kWarps = kThreads / 32;
 static_assert((kWarps & (kWarps - 1)) == 0, "the CTA reductions take a power-of-two warp count");
 
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
-// 1 / x and 1 / sqrt(x) from the hardware's approximations (about 20 bits) by one third-order
-// iteration, r (1 + e + e^2) and r (1 + e / 2 + 3 e^2 / 8) with e the residual: within about one unit
-// in the last place.  The serial steps of the solver wait for these: three dependent operations of 64
-// cycles where a correctly rounded division takes about ten.  Arguments near the ends of the exponent
-// range take the ordinary operations.
-__device__ __forceinline__ bool mid_range(double x) {
-  const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
-  return e - 0x06000000u < 0x73000000u;  // 2^-926 .. 2^914
-}
-__device__ __forceinline__ double fast_rcp(double x) {
-  if (!mid_range(x)) return 1.0 / x;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-__device__ __forceinline__ double fast_rsqrt(double x) {  // x > 0
-  if (!mid_range(x)) return 1.0 / sqrt(x);
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x * r, r, 1.0);
-  return fma(r * e, fma(0.375, e, 0.5), r);
-}
-// sqrt(x) from r = 1 / sqrt(x)
-__device__ __forceinline__ double sqrt_from(double x, double r) {
-  if (!mid_range(x)) return sqrt(x);
-  const double q = x * r;
-  return fma(fma(-q, q, x), 0.5 * r, q);
-}
 
 // ---- complex helpers ---------------------------------------------------------------------------
 // On GB300 an SM retires about two FP64 fused multiply-adds per clock, so every FP64 instruction
