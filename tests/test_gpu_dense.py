@@ -222,3 +222,26 @@ def test_batches_on_clusters(ctx, count, n, real):
     for i in list(range(0, count, max(1, count // 12))) + [count - 1]:
         if i != bad:
             check(*ps[i], *out[i])
+
+
+@pytest.mark.parametrize("n,real", [(1300, False), (1216, False), (1217, False), (1830, True)])
+def test_orders_whose_columns_stay_in_memory(ctx, n, real):
+    """Single pencils around and above the order up to which a CTA of the grid holds its columns in
+    shared memory during the tridiagonalisation (1216 complex, 1824 real).  B as well conditioned as a
+    filtered block's Gram matrix: at these orders the spread of levels that a badly conditioned B gives
+    leaves hundreds of them closer than 1e-5 |T|, which one thread orthogonalises."""
+    A, B = pencil(n, seed=n, real=real, cond=1.0)
+    info, [(w, X)] = run(ctx, [(A, B)], real=real)
+    assert info[0] == 0
+    check(A, B, w, X)
+
+
+@pytest.mark.parametrize("count,n,real", [(3, 300, False), (2, 420, True), (130, 170, False), (470, 122, True)])
+def test_batches_whose_columns_stay_in_memory(ctx, count, n, real):
+    """Batches above the order at which a CTA holds its columns, on clusters of 8 (two forms) and 4 and
+    on single CTAs, unevenly: the smaller pencils of a batch take the form of the largest."""
+    ps = [pencil(n - (i % 5) * (n // 9), seed=400 + i % 11, real=real, cond=1.0) for i in range(count)]
+    info, out = run(ctx, ps, real=real)
+    assert np.all(info == 0)
+    for i in list(range(0, count, max(1, count // 6))) + [count - 1]:
+        check(*ps[i], *out[i])
