@@ -1246,9 +1246,36 @@ __device__ bool tridiagonal_eig(const Team& T, const Pencil<S>& P, S* smem) {
         // orthogonalise against the cluster's earlier vectors, then normalise
         for (int q = k0; q < m; ++q) {
           const double* zq = P.Z + (size_t)q * n;
-          double s2 = 0.0;
-          for (int i = 0; i < n; ++i) s2 += zq[i] * x[(size_t)i * n + m];
-          for (int i = 0; i < n; ++i) x[(size_t)i * n + m] -= s2 * zq[i];
+          double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+          int i = 0;
+          for (; i + U <= n; i += U) {
+            double z[U], v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              z[u] = zq[i + u];
+              v[u] = x[(size_t)(i + u) * n + m];
+            }
+#pragma unroll
+            for (int u = 0; u < U; u += 4) {
+              s0 = fma(z[u], v[u], s0);
+              s1 = fma(z[u + 1], v[u + 1], s1);
+              s2 = fma(z[u + 2], v[u + 2], s2);
+              s3 = fma(z[u + 3], v[u + 3], s3);
+            }
+          }
+          for (; i < n; ++i) s0 = fma(zq[i], x[(size_t)i * n + m], s0);
+          const double dot = (s0 + s1) + (s2 + s3);
+          for (i = 0; i + U <= n; i += U) {
+            double z[U], v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              z[u] = zq[i + u];
+              v[u] = x[(size_t)(i + u) * n + m];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) x[(size_t)(i + u) * n + m] = fma(-dot, z[u], v[u]);
+          }
+          for (; i < n; ++i) x[(size_t)i * n + m] = fma(-dot, zq[i], x[(size_t)i * n + m]);
         }
         double n0 = 0.0, n1 = 0.0, n2 = 0.0, n3 = 0.0;  // four independent chains
         int i = 0;
