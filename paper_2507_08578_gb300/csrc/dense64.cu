@@ -1501,14 +1501,48 @@ size_t resident_smem_bytes(int n, size_t ws, int ctas, size_t limit) {
 }
 constexpr int kMaxN = 4608;  // 3 n complex words must fit in shared memory (221 KB)
 
-// CTAs per pencil of a batch, a portable cluster at most.  A pencil's serial steps leave most of an SM
-// idle and several short waves even out uneven orders, so the line lies at six CTAs per SM (pencils of
-// order 20 to 141; 12 of them on 1, 2, 4, 8 CTAs each: 25.6, 13.7, 7.9, 5.1 ms; 217 of them: 28.0, 18.5,
-// 14.5, 18.2 ms).  At least four columns a CTA.
-int cluster_size(kss_ctx ctx, int count, int nmax) {
-  int c = 8;
-  while (c > 1 && ((long long)count * c > 6LL * std::max(ctx->nsm, 1) || 4 * c > nmax)) c /= 2;
-  return c;
+// Shared memory of one CTA of a batch on teams of `ctas`; resident: with its columns.  Two CTAs share an
+// SM (their registers), so the columns may take half of its shared memory.
+size_t batch_smem(int n, size_t ws, int ctas, bool* resident = nullptr) {
+  const size_t res = resident_smem_bytes(n, ws, ctas, 110u * 1024u);
+  if (resident) *resident = res != 0;
+  return std::max(dyn_smem_bytes(n, ws), res);
+}
+
+// CTAs per pencil of a batch (orders n[], words of ws bytes), a portable cluster at most and four columns
+// a CTA at least: the size with the shortest estimated time, in units of the largest pencil on one CTA.
+//   * c CTAs take t = s + (1 - s) / c, the serial share s being 10 / n complex and 18 / n real;
+//   * two CTAs on an SM slow each other by the share b = (1 - s) / c / t of their time that is not serial:
+//     f = 1 + 0.7 b^1.5;
+//   * a wave is two CTAs an SM, less 4 and 5 % for clusters of 4 and 8, which do not span the chip's SM groups; a
+//     last wave of half that or less has its SMs to itself;
+//   * pencils of uneven order count by their order cubed (the large ones start first).
+// Fitted to batches of 20 to 1000 equal pencils of orders 20 to 260 on 1, 2, 4 and 8 CTAs each: within 0.6 %
+// of the best size on average, 8 % at most.  (As many CTAs as six an SM allow took up to 1.7 times the
+// best for 76 or 152 pencils, more than one CTA each had taken: 152 of order 64 complex 5.95 -> 3.98 ms, of
+// order 150 35.5 -> 26.7; 217 uneven ones of 20 to 141, on 1, 2, 4, 8 CTAs 28.0, 18.5, 14.5, 18.2 ms, stay
+// on 4.)
+template <class P>
+int cluster_size(kss_ctx ctx, const std::vector<P>& pencils, int nmax, size_t ws) {
+  const double s = std::min(0.7, (ws == 8 ? 18.0 : 10.0) / nmax), nsm = std::max(ctx->nsm, 1);
+  double count = 0;
+  for (const auto& p : pencils) count += std::pow((double)p.n / nmax, 3);
+  if (count > 0.8 * pencils.size()) count = (double)pencils.size();
+  int best = 1;
+  double tbest = 1e300;
+  for (int c = 8; c >= 1; c /= 2) {
+    if (c > 1 && 4 * c > nmax) continue;
+    const bool pairs = batch_smem(nmax, ws, c) <= 113u * 1024u;
+    const double t = s + (1.0 - s) / c, b = (1.0 - s) / c / t, f = pairs ? 1.0 + 0.7 * std::pow(b, 1.5) : 1.0;
+    const double wave = (pairs ? 2 : 1) * nsm / c * (c == 8 ? 0.95 : c == 4 ? 0.96 : 1.0);
+    const double full = std::floor(count / wave), rest = count - full * wave;
+    const double time = t * (full * f + (rest < 1e-9 ? 0.0 : 2.0 * rest <= wave + 4.0 ? 1.0 : f));
+    if (time < tbest) {
+      tbest = time;
+      best = c;
+    }
+  }
+  return best;
 }
 
 template <class S>
@@ -1520,10 +1554,9 @@ void launch_cta(kss_ctx ctx, std::vector<Pencil<S>>& small, size_t items_offset,
   cudaStream_t st = ctx->stream;
   int nmax = 1;
   for (const auto& P : small) nmax = std::max(nmax, P.n);
-  const int csize = cluster_size(ctx, (int)small.size(), nmax);
-  // two CTAs share an SM (their registers): half of its shared memory each
-  const size_t res = resident_smem_bytes(nmax, sizeof(S), csize, 110u * 1024u);
-  const size_t sm = std::max(dyn_smem_bytes(nmax, sizeof(S)), res);
+  const int csize = cluster_size(ctx, small, nmax, sizeof(S));
+  bool res = false;
+  const size_t sm = batch_smem(nmax, sizeof(S), csize, &res);
   for (auto& P : small) {
     P.smem_cols = col_smem_bytes(nmax, sizeof(S)) ? 1 : 0;
     P.resident = res ? 1 : 0;

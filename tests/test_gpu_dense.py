@@ -245,3 +245,14 @@ def test_batches_whose_columns_stay_in_memory(ctx, count, n, real):
     assert np.all(info == 0)
     for i in list(range(0, count, max(1, count // 6))) + [count - 1]:
         check(*ps[i], *out[i])
+
+
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("count", [20, 60, 76, 152])
+def test_batches_of_equal_order(ctx, count, real):
+    """Batches that fill the chip once with clusters of 8, 4 and 2, and with single CTAs (order 64)."""
+    ps = [pencil(64, seed=500 + i % 5, real=real) for i in range(count)]
+    info, out = run(ctx, ps, real=real)
+    assert np.all(info == 0)
+    for i in (0, 1, count // 2, count - 1):
+        check(*ps[i], *out[i])
