@@ -132,3 +132,50 @@ def test_density_scales_and_special_bands(ctx, box, a, ecut, kpt):
         assert np.all(np.isnan(rho_of(bad, w)))
     finally:
         K.kss_sys_destroy(sysh)
+
+
+@pytest.mark.parametrize("box,a,ecut", [((24, 24, 24), 10.0, 10.0), ((30, 30, 30), 8.0, 10.0)])
+def test_density_no_further_from_the_true_one_than_fp64_transforms(ctx, box, a, ecut):
+    """Against the density in extended precision (at least 11 bits beyond double, from the sums
+    themselves): closer than the one from FP64 FFTs, whose rounded factors act on every band alike, and
+    within 2^-52 of it in the mean square: the blocks' values are off by a few 2^-56 of their rms, and the
+    last operations round at most twice a band (four bands)."""
+    import torch
+    ld, cl = np.longdouble, np.clongdouble
+    assert np.finfo(ld).nmant >= 63
+    s = W.make_system("fd", a, ecut, 3, 4, seed=17, kpts=[[0.25] * 3], fft_box=box, nproj_per_atom=0)
+    sysh = setup(ctx, s)
+    try:
+        b = O.make_basis(s.lattice, s.ecut, s.kpts[0], box)
+        _, vol = O.reciprocal_lattice(s.lattice)
+        m = np.asarray(b.miller) % np.array(box)
+        w = np.array([2.0, 2.0, 0.7, 1.3])
+        c = W.random_block(b.npw, 4, seed=5) / (1.0 + np.asarray(b.kinetic))
+        c /= np.linalg.norm(c, axis=1)[:, None]
+        rho = torch.zeros(tuple(reversed(box)), dtype=torch.float64, device="cuda")
+        K.kss_density_accumulate(sysh, 0, torch.from_numpy(c).cuda(), w, rho)
+        torch.cuda.synchronize()
+        pi = ld("3.14159265358979323846264338327950288419716939937510")
+        k = np.arange(box[0])
+        t = (np.outer(k, k) % box[0]).astype(ld) * (2 * pi / box[0])
+        F = np.cos(t) + 1j * np.sin(t)
+        ref = np.zeros(rho.shape, ld)
+        grid = np.zeros((4,) + rho.shape, complex)
+        grid[:, m[:, 2], m[:, 1], m[:, 0]] = c
+        for n in range(4):
+            g = grid[n].astype(cl)
+            g = np.einsum("zyx,xa->zya", g, F)
+            g = np.einsum("zya,yb->zba", g, F)
+            g = np.einsum("zba,zc->cba", g, F)
+            ref += ld(w[n]) * (g.real ** 2 + g.imag ** 2) / ld(vol)
+        r = np.fft.ifftn(grid, axes=(1, 2, 3)) * np.prod(box)
+        fft = np.einsum("n,nzyx->zyx", w / vol, r.real ** 2 + r.imag ** 2)
+
+        def err(x):
+            return float(np.sqrt(np.sum((x.astype(ld) - ref) ** 2) / np.sum(ref ** 2)))
+
+        got = err(rho.cpu().numpy())
+        assert got < 2.0 ** -52
+        assert got < err(fft)
+    finally:
+        K.kss_sys_destroy(sysh)
