@@ -245,21 +245,37 @@ def run_reference(args, rank: int):
 # ------------------------------------------------------------------------------------------------
 # GPU arm
 
-# DRAM bytes per band of the middle FFT pass on the C2 workload, from one ncu capture of two
-# production launches each (dram__bytes_read.sum + dram__bytes_write.sum, mean of the two):
-# pass_bw<double, 8, 12, 384> moved 73.53 + 7.28 MB per 27-band launch, pass_bw<float, 12, 8, 384>
-# 69.94 + 6.15 MB per 54-band launch.  Valid for that kernel and schedule only (the bench reports
-# null traffic when the autotuner picked another).
-# ncu DRAM bytes per band of the middle pass (production schedule 12 x 8 at 384 threads, pruned
-# stages) with the L2 state the step leaves (--cache-control none; a full-chunk production launch:
-# profiles/c2_pass_b_dram_traffic.md)
-# (single precision; the fixed-point pass of double precision has not been counted)
-PASS_B_DRAM_PER_BAND = {"mixed": (9.314304e6 + 41.612032e6) / 54}
-PASS_B_SCHEDULE = {"mixed": "12x8 @384"}
-# FP instructions the middle pass executes per band (ncu counts: 2 per FMA, 1 per add / multiply)
-# over the dense-transform count 4 x 5 N^3 log2 N, for the production schedule (12 x 8 at 384
-# threads with the pruned strided stages, CW = 3)
-PASS_B_EXECUTED_PER_ALGORITHMIC = {"mixed": (2 * 707014656 + 1399762944 + 439271424) / 54 / (4 * 5 * 96 ** 3 * math.log2(96))}
+# What the middle FFT pass does per band on the 96-point box, by the schedule that ran: ncu counts of
+# full launches inside a filter step (profiles/c2_pass_b_counts.md), valid for these kernels and schedules
+# only (other schedules report null).
+#   inst: warp instructions; heavy: those of the multiply-add pipe's heavy half (the 32 x 32 + 64-bit
+#   multiply-adds of the fixed-point form); flops: single-precision operations (2 per FMA, packed ones
+#   twice); dram: bytes read and written with the L2 state that the step leaves
+PASS_B_COUNTS = {
+    "fp64": {"12x8 @384": {"inst": 386367734 / 27, "heavy": 182349516 / 27,
+                           "dram": (19270400 + 48644096 + 12470784 + 42099456) / 54},
+             "8x12 @384": {"inst": 383913003 / 27, "heavy": 182528201 / 27,
+                           "dram": (16174848 + 45824256 + 12482816 + 42310656) / 54}},
+    "mixed": {"12x8 @384": {"inst": 118158912 / 54, "heavy": 43355954 / 54,
+                            "flops": (2 * 528519168 + 213829632 + 470458368 + 2 * 631701504 + 4 * 39481344) / 54,
+                            "dram": (7630592 + 48060160 + 6867968 + 46360064) / 108}},
+}
+SMS = 152
+
+
+def pass_b_issue(counts, bands, ms, sm_mhz):
+    """The middle pass against what its SMs can issue: warp instructions per second over four a clock
+    and SM, and those of the heavy multiply-add pipe over its two."""
+    if not counts or not sm_mhz or ms <= 0:
+        return None
+    rate = bands / (ms / 1000.0) / 1e9
+    clk = SMS * sm_mhz * 1e6 / 1e9
+    return {"achieved": counts["inst"] * rate, "peak": 4 * clk, "unit": "G warp instructions/s",
+            "frac": counts["inst"] * rate / (4 * clk),
+            "multiply_add_heavy": {"achieved": counts["heavy"] * rate, "peak": 2 * clk,
+                                   "frac": counts["heavy"] * rate / (2 * clk)},
+            "note": "ncu instruction counts of this kernel and schedule x the bands of this run, over the "
+                    "issue slots at the SM clock sampled in this run"}
 
 
 def algorithmic_work(s, npw, nb, degree, box, applies, rr_calls):
@@ -557,34 +573,48 @@ def run_ours(args, rank: int, world: int, local_rank: int):
     counted = [f for f in fam if f in work and f.startswith("local_pass")]
     dom = max(counted, key=lambda f: fam[f][1]) if counted else top
     dl, dms = fam[dom]
-    peak = FP64_PEAK_TFLOPS if args.form == "fp64" else FP32_PEAK_TFLOPS
+    peak = FP32_PEAK_TFLOPS
     # the CUDA cores' FMA throughput measured on this device right after the timed region
     probe = K.kss_peak_probe(ctx, 0 if args.form == "fp64" else 1)
     roof = None
+    sched_now = {f"{e['A']}x{e['B']} @{e['threads']}" for e in K.kss_autotune_table() if e["N"] == 96}
+    counts = None
+    if dom == "local_pass_b" and args.workload == "c2" and len(sched_now) == 1:
+        counts = PASS_B_COUNTS[args.form].get(next(iter(sched_now)))
     if dom in work and dms > 0:
         ach = work[dom] / (dms / 1000.0) / 1e12
-        roof = {"kernel": dom, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                "frac": ach / peak, "traffic": None,
-                "peak_note": ("FP64 CUDA-core rate derived from the unit counts and clock: 152 SMs x "
-                              "2 FP64 FMA per clock x 2 flops x 2070 MHz = 1.26, nominal 1.25; the passes "
-                              "run in 64-bit fixed point on the integer pipes, so frac can exceed 1"
-                              if args.form == "fp64" else
-                              "FP32 CUDA-core rate derived from 152 SMs x 128 lanes x 2 x 2070 MHz"),
-                "measured_peak": probe, "frac_of_measured": ach / probe,
-                "measured_note": "kss_peak_probe in this run: independent FMA chains, 8 CTAs per SM, "
-                                 "best of three launches",
-                "launches": dl, "avg_launch_ms": dms / dl}
+        if args.form == "fp64":
+            # 64-bit fixed point: no FP64 peak bounds it
+            roof = {"kernel": dom, "bound": "issue", "achieved": None, "peak": None,
+                    "unit": "G warp instructions/s", "frac": None, "traffic": None}
+            roof.update((pass_b_issue(counts, applies, dms, ck["sm_mhz"]) if dom == "local_pass_b" else None) or {})
+            roof["fp64_equivalent"] = {"achieved": ach, "unit": "TFLOP/s", "fp64_pipe_measured": probe,
+                                       "note": "dense-transform operations per second; the passes run in 64-bit "
+                                               "fixed point on the integer pipes, beside the FP64 pipe's FMA "
+                                               "rate (kss_peak_probe) for comparison only"}
+        else:
+            roof = {"kernel": dom, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+                    "frac": ach / peak, "traffic": None,
+                    "peak_note": "FP32 CUDA-core rate derived from 152 SMs x 128 lanes x 2 x 2070 MHz",
+                    "measured_peak": probe, "frac_of_measured": ach / probe,
+                    "measured_note": "kss_peak_probe in this run: independent FMA chains, 8 CTAs per SM, "
+                                     "best of three launches"}
+            if counts:
+                # single-precision operations the pruned pass executes over the dense-transform count
+                x = counts["flops"] / (4 * 5 * 96 ** 3 * math.log2(96))
+                roof["executed_per_algorithmic"] = x
+                roof["executed_frac_of_measured"] = ach * x / probe
+                roof["issue"] = pass_b_issue(counts, applies, dms, ck["sm_mhz"])
+        roof["launches"] = dl
+        roof["avg_launch_ms"] = dms / dl
+        if counts:
+            roof["traffic"] = counts["dram"] * applies / dl
+            roof["traffic_note"] = ("DRAM bytes per launch: ncu bytes per band of this kernel and schedule (L2 as "
+                                    "the step leaves it) x the bands per launch of this run")
         if top != dom:
             roof["longest_family"] = {"kernel": top, "ms": fam[top][1],
                                       "note": "the longest kernel family of the step is not an FFT pass"}
         roof["fft_path_hbm"] = fft_path_hbm(fam, applies, npw, 16 if args.form == "fp64" else 8, hbm_peak()[0])
-        sched_now = [f"{e['A']}x{e['B']} @{e['threads']}" for e in K.kss_autotune_table() if e["N"] == 96]
-        if dom == "local_pass_b" and args.form == "mixed" and args.workload == "c2" and sched_now and \
-                all(x == PASS_B_SCHEDULE[args.form] for x in sched_now):
-            # FP instructions the pruned pass executes (ncu counts of this schedule) over the
-            # dense-transform count: the executed rate against the measured FMA throughput
-            roof["executed_per_algorithmic"] = PASS_B_EXECUTED_PER_ALGORITHMIC[args.form]
-            roof["executed_frac_of_measured"] = ach * PASS_B_EXECUTED_PER_ALGORITHMIC[args.form] / probe
 
     # ---- the FP64 products on the tensor cores (FP64 form) ----
     fp64_gemm = None
@@ -678,13 +708,6 @@ def run_ours(args, rank: int, world: int, local_rank: int):
     # pass-B schedules the autotuner picked (box, window, split, threads per CTA; 0 = per-warp form)
     sched = [f"{e['N1']}x{e['N']}^2 W3<={e['W3']}: {e['A']}x{e['B']} @{e['threads']} "
              f"({e['ncand']} timed)" for e in table]
-    c2_sched = [f"{e['A']}x{e['B']} @{e['threads']}" for e in table if e["N"] == 96 and e["N1"] == 96]
-    if roof is not None and roof["kernel"] == "local_pass_b" and args.form == "mixed" and args.workload == "c2" and \
-            c2_sched and all(x == PASS_B_SCHEDULE[args.form] for x in c2_sched):
-        roof["traffic"] = PASS_B_DRAM_PER_BAND[args.form] * applies / roof["launches"]
-        roof["traffic_note"] = ("DRAM bytes per launch: ncu bytes per band of this kernel and schedule (L2 as "
-                                "the step leaves it) x the bands per launch of this run")
-
     if rank == 0:
         line = {
             "metric": "band H-applies/s", "value": value, "unit": "band-applies/s",
@@ -895,9 +918,10 @@ def run_density(args):
     if name in prof:
         l, kms = prof[name]
         ach = bands * 2 * 5.0 * 96 ** 3 * math.log2(96) / (kms / 1000.0) / 1e12
-        peak = FP64_PEAK_TFLOPS if prec == K.KSS_PREC_FP64 else FP32_PEAK_TFLOPS
+        # (in double precision the transforms run in fixed point, which no floating-point peak bounds)
+        peak = None if prec == K.KSS_PREC_FP64 else FP32_PEAK_TFLOPS
         roof = {"kernel": name, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                "frac": ach / peak, "traffic": None, "launches": l, "avg_launch_ms": kms / l}
+                "frac": ach / peak if peak else None, "traffic": None, "launches": l, "avg_launch_ms": kms / l}
     K.kss_sys_destroy(sysh)
     K.kss_destroy(ctx)
     print(json.dumps({"metric": "band densities/s", "value": bands / (ms / 1000.0), "unit": "bands/s",
