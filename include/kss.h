@@ -571,7 +571,9 @@ kss_status kss_autotune_count(int* n);
 kss_status kss_autotune_get(int i, kss_tune_entry* out);
 /* Insert or replace the entry for (device, precision, N1, N, W3 rounded up to a multiple of 8):
  * pins a schedule (e.g. one read back from an earlier run, for run-to-run identical rounding).
- * A, B, threads as in kss_tune_entry (ms, ncand, W2 ignored).  A pinned schedule without a
+ * A, B, threads as in kss_tune_entry (ms, ncand, W2 ignored).  In double precision the entry holds for
+ * the fixed-point passes of a single application and for the batch engine's FP64 passes alike (which
+ * are otherwise timed apart; the table lists the former where both are there).  A pinned schedule without a
  * kernel instance, or whose shared memory does not fit a configuration's window, falls back to
  * the per-warp form at use.  KSS_EINVAL for inconsistent fields (A * B != N, threads not in
  * {0, 128, 256, 384}, W3 outside [1, N], unknown precision). */

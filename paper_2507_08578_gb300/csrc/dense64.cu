@@ -1615,8 +1615,8 @@ void hegv_batched(kss_ctx ctx, const std::vector<HegvItem>& items) {
   size_t total = 0;
   for (const auto& it : items) total += work_doubles(std::max(it.n, 1), it.real);
   ctx->dense_ws.ensure(total * sizeof(double));
-  // one CTA per pencil, real and complex pencils in separate launches; a single large pencil on a
-  // cooperative grid
+  // a CTA or a cluster of them per pencil, real and complex pencils in separate launches; a single large
+  // pencil on a cooperative grid
   std::vector<Pencil<double>> small_r;
   std::vector<Pencil<double2>> small_c;
   double* p = ctx->dense_ws.as<double>();

@@ -10,8 +10,8 @@
 //
 // What bounds them: integer issue.  FP64 runs at 2 lane-operations a clock and SM, which held these
 // passes in FP64 at 80 % of that pipe's issue; in integers a butterfly is two 128-lane adds.  Measured
-// at the 96-point box, 564 bands (A / B / C, ms): FP64 3.05 / 52.3 / 3.49, fixed point 1.04 / 12.9 /
-// 1.35; at the 54-point box, 47 bands (us): 104 / 938 / 111 and 29 / 262 / 39.  Error of T psi + V psi
+// at the 96-point box, 564 bands (A / B / C, ms): FP64 3.05 / 52.3 / 3.49, fixed point 1.02 / 12.9 /
+// 1.41; at the 54-point box, 47 bands (us): 104 / 938 / 111 and 29 / 242 / 39.  Error of T psi + V psi
 // against long double, bands falling off as 1 / (1 + T^2), relative to |V psi|: FP64 4.8e-16 and
 // fixed point 1.8e-16 at 96 points, 8.2e-16 and 1.8e-16 at 54; flat bands 1.47e-15 and 1.37e-15
 // (the rounding of the outputs).
