@@ -103,3 +103,28 @@ def test_noalloc_runs_the_same_passes(ctx, box, a, ecut, natom, nb, nproj):
     finally:
         K.kss_sys_destroy(sysh)
         K.kss_autotune_clear()
+
+
+@pytest.mark.parametrize("box", [(64, 48, 48), (96, 48, 54), (72, 30, 36)])
+def test_gamma_pairs_without_fixed_point(ctx, box):
+    """Real-space-real bands, two per transform, an odd one left over, in the FP64 forms: 1e-13 of the
+    pair's |H psi|, as the transform is of the pair's sum."""
+    import torch
+    s = W.make_system("fg", 8.0, 10.0, 3, 4, seed=26, fft_box=box)
+    sysh = setup(ctx, s)
+    try:
+        p = O.build_problem(s, 0, box=box)
+        c = W.random_block(p.basis.npw, 7, seed=10)
+        c = c + c[:, ::-1].conj()  # the canonical order at Gamma is symmetric
+        psi = torch.from_numpy(c).cuda()
+        out = torch.empty_like(psi)
+        K.kss_apply_H_gamma(sysh, 0, psi, out, K.KSS_PREC_FP64)
+        torch.cuda.synchronize()
+        ref = p.apply(c)
+        err = np.linalg.norm(out.cpu().numpy() - ref, axis=1)
+        norm = np.linalg.norm(ref, axis=1)
+        pair = np.maximum(norm, np.append(norm.reshape(-1)[:6].reshape(3, 2)[:, ::-1].reshape(-1), 0.0))
+        assert np.all(err < 1e-13 * pair)
+    finally:
+        K.kss_sys_destroy(sysh)
+        K.kss_autotune_clear()
